@@ -51,15 +51,18 @@ typedef enum {
  * FP32 numbers (about 48 significand bits, FP32's exponent range) computed on
  * the FP32 pipe; GB300 issues FP64 on about 1/67 of its FP32 lanes. */
 typedef enum {
-    MLC_TIER_FP64 = 0,     /* FP64 charge and result; every step in FP64 arithmetic on
-                              the FP64 pipe (the plain FP64 solve)                        */
+    MLC_TIER_FP64 = 0,     /* FP64 charge and result; every step to FP64 accuracy: the local
+                              convolutions as exact-split tensor-core products (FP64 operands
+                              in seven 8-bit digits, sums of digit products held exactly),
+                              the other steps in FP64 arithmetic                          */
     MLC_TIER_SPLIT = 1,    /* FP32 charge; local convolutions (FFTs on the CUDA cores) and
                               the Legendre ring sums in FP32, the moments in FP32 with an
                               FP64 last contraction; coarse charge, coarse solve, boundary
                               values (subtract, interpolate, accumulate) and Dirichlet
                               solves in FP64; FP64 result                                 */
-    MLC_TIER_DF = 2,       /* FP64 charge and result; moments in FP64, every other step in
-                              double-float arithmetic                                     */
+    MLC_TIER_DF = 2,       /* FP64 charge and result; moments in FP64, local convolutions as
+                              in MLC_TIER_FP64, every other step in double-float
+                              arithmetic                                                  */
     MLC_TIER_SPLIT_DF = 3  /* as MLC_TIER_SPLIT with double-float in place of FP64 in the
                               steps after the local convolutions                          */
 } mlc_tier;
@@ -94,7 +97,10 @@ typedef struct {
     int dgf_zeta;   /* -1: 2                                                            */
     int conv_chunk; /* patches per launch group of the local convolutions: their spectra
                        (the scratch between the forward and inverse transforms) exist
-                       for one group at a time; -1: the library's choice (1024)        */
+                       for one group at a time; -1: the library's choice (1024).  In the
+                       FP64 and double-float tiers it bounds the scratch (that of the
+                       spectra of so many patches), which holds the operands and results
+                       of more patches at once                                         */
     int levels;     /* number of levels of the multilevel MLC (Sec. 5); -1: 2, the
                        two-level algorithm of Sec. 4.  With levels > 2 the global coarse
                        solve phi^H = G^H * F^H becomes the MLC solve of F^H on the next

@@ -40,7 +40,8 @@ void batch_layout(int count, const mlc_plan_t *plans, const void *const *f, void
     std::vector<int> reps;
     for (int k = 0; k < count; ++k) {
         for (size_t g = 0; g < reps.size(); ++g)
-            if (same_patch_geometry(plans[reps[g]]->g, plans[k]->g)) {
+            if (same_patch_geometry(plans[reps[g]]->g, plans[k]->g) &&
+                plans[reps[g]]->limb_tabs == plans[k]->limb_tabs) {
                 gof[k] = (int)g;
                 break;
             }
@@ -131,6 +132,7 @@ cudaError_t batch_enqueue(const std::vector<mlc_plan_t> &plans, const BatchLayou
         it.chunk = chunk;
         it.a1 = gr.a1;
         it.a4 = gr.a4;
+        it.cap = gr.cap;
         TRYE(cudaStreamWaitEvent(S.aux[g], ev_start, 0));
         TRYE(cudaStreamWaitEvent(S.conv[g], ev_start, 0));
         TRYE(launch_moments(gr.rep, it, S.aux[g]));
@@ -345,6 +347,7 @@ extern "C" mlc_status mlc_batch_solve(int count, const mlc_plan_t *plans, const 
             c->scratch.push_back(p);
             gr.a1 = p;
             gr.a4 = (char *)p + conv_scratch_a4_offset(G, nit);
+            gr.cap = conv_scratch_bytes(G, nit);
         }
         if (e == cudaSuccess)
             e = cudaMemcpy(c->d_items, items.data(), items.size() * sizeof(int2), cudaMemcpyHostToDevice);

@@ -1,12 +1,12 @@
-// Solve-time kernels of the FP64 tier of the two-level MLC (Sec. 4).
+// Solve-time kernels of the two-level MLC (Sec. 4).
 //
 //   moments     Legendre coefficients by composite Boole's rule (Step 1)
-//   fwd_x/col/inv_x
-//               Hockney convolutions (App. A.2): zero-padded periodic
-//               convolution of length M, as pruned radix-2 FFTs in shared
-//               memory; used for the local fields phi^{i,h} (eq.
-//               initiallocalproblemsmlcII) and for the coarse solve
-//               phi^H = G^H * F^H (Step 2)
+//   fwd_x/slab/inv_x
+//               Hockney convolutions (App. A.2) of the split tiers: zero-padded
+//               periodic convolution of length M by pruned FP32 FFTs, for the
+//               local fields phi^{i,h} (eq. initiallocalproblemsmlcII; the FP64
+//               and double-float tiers form them in limb_conv.cu)
+//   cfft        the coarse solve phi^H = G^H * F^H (Step 2), mixed-radix FFTs
 //   resid       phi^{i,h} - I^H(phi^{i,h}) on the face nodes of Omega_alpha
 //   assemble    F^H = sum_i F^{i,H} (eq. FDLD), a fixed-order gather
 //   boundary    phi^B (eqs. philocmlcII, mlcfulldiscr) in the linear form
@@ -52,8 +52,7 @@ __device__ __forceinline__ int floordiv(int a, int b) {  // b > 0
 // numbers (|lo| a few ulp(hi) at most), about 48 significand bits.  Sums use
 // the error-free two-sum of Knuth, products the FMA-based two-product; the
 // FFT and DST error bounds are relative to the data norm, so no operation
-// renormalises the pair.  GB300 issues FP32 on ~67x more lanes than FP64, so
-// the FP64 tier's transforms and ring sums run in this arithmetic.
+// renormalises the pair.  GB300 issues FP32 on ~67x more lanes than FP64.
 // ---------------------------------------------------------------------------
 struct dfl {
     float hi, lo;
@@ -103,8 +102,6 @@ __device__ __forceinline__ dfl operator+(dfl a, dfl b) { return df_add(a, b); }
 __device__ __forceinline__ dfl operator-(dfl a, dfl b) { return df_sub(a, b); }
 __device__ __forceinline__ dfl operator-(dfl a) { return df_neg(a); }
 __device__ __forceinline__ dfl operator*(dfl a, dfl b) { return df_mul(a, b); }
-__device__ __forceinline__ dfl &operator*=(dfl &a, dfl b) { return a = df_mul(a, b); }
-__device__ __forceinline__ dfl &operator+=(dfl &a, dfl b) { return a = df_add(a, b); }
 __device__ __forceinline__ dcx cmul(dcx a, dcx w) { return dc_mul(a, w); }
 // a + w x in double-float (one product, one sum)
 __device__ __forceinline__ dfl df_fma(dfl w, dfl x, dfl a) { return df_add(a, df_mul(w, x)); }
@@ -118,7 +115,7 @@ __device__ __forceinline__ dcx renorm(dcx v) { return {fast_two_sum(v.x.hi, v.x.
 __device__ __forceinline__ float2 renorm(float2 v) { return v; }
 __device__ __forceinline__ double2 renorm(double2 v) { return v; }
 
-// Complex type of each working precision (FP64 tier: double-float; split tier: float).
+// Complex type of each working precision.
 template <typename R> struct Cx;
 template <> struct Cx<float> {
     using T = float2;
@@ -274,19 +271,6 @@ __device__ __forceinline__ bool mbar_wait_bounded(unsigned long long *bar, unsig
     for (int i = 0; i < tries; ++i)
         if (mbar_try_wait(bar, parity)) return true;
     return false;
-}
-
-// Plan record and local patch index of a work item.
-// Item `item` of a launch covers patch p of its plan; the item index itself
-// is the slot of the item in the launch's local-convolution scratch.
-__device__ __forceinline__ const PlanPtrs &item_plan(const Items &it, int item, int &p) {
-    if (it.items) {
-        const int2 v = it.items[item];
-        p = v.y;
-        return it.plans[v.x];
-    }
-    p = item + it.first;
-    return it.plans[0];
 }
 
 template <int LOG2M, typename C>
@@ -449,81 +433,6 @@ __global__ void __launch_bounds__(256) k_slab(SlabArgs a) {
 }
 
 // ---------------------------------------------------------------------------
-// The same slab for 16-byte complex entries (FP64, double-float) at M = 128,
-// whose M x M slab does not fit in shared memory: after the forward y
-// transform of the nin input z columns, the ky rows go through the forward z
-// transform, the kernel spectrum and the inverse z transform rb rows at a
-// time in a row buffer, and each row keeps only the nz output z positions,
-// written back over its own input; the inverse y transform then runs on those
-// nz columns.  S: M rows of sw >= max(nin, nz) entries.  Same arithmetic per
-// entry as k_slab (the z transforms of a row do not depend on the others).
-// ---------------------------------------------------------------------------
-template <int LOG2M, typename R>
-__global__ void __launch_bounds__(256) k_slab_rows(SlabArgs a, int sw, int rb) {
-    using C = typename Cx<R>::T;
-    constexpr int M = 1 << LOG2M, MH = M / 2 + 1, P = M + 1;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    C *s_tw = (C *)smem_raw;
-    C *S = s_tw + M / 2;
-    C *B = S + M * sw;  // rb rows of P
-    const int kx = blockIdx.x % MH;
-    int p;
-    const PlanPtrs &PP = item_plan(a.it, blockIdx.x / MH, p);
-    const int nin = a.nin, W = a.nout, nz = a.nz;
-    load_twiddles<LOG2M>(s_tw, (const C *)a.tw);
-    for (int e = threadIdx.x; e < M * nin; e += blockDim.x) S[(e / nin) * sw + e % nin] = Cx<R>::mk(0, 0);
-    __syncthreads();
-    const long q = blockIdx.x / MH;  // scratch slot
-    const C *in = (const C *)a.it.a1 + (q * MH + kx) * nin * nin;
-    for (int e = threadIdx.x; e < nin * nin; e += blockDim.x) {
-        const int zi = e / nin, yi = e % nin;
-        S[yi * sw + zi] = in[e];
-    }
-    __syncthreads();
-    // forward y on the nin z columns (natural in, bit-reversed ky rows out)
-    fft_dif<LOG2M>(S, nin, 1, sw, s_tw, false);
-    const R *khat = (const R *)PP.khat;
-    int pos0 = a.out_off % M;
-    if (pos0 < 0) pos0 += M;
-    for (int r0 = 0; r0 < M; r0 += rb) {
-        const int nr = min(rb, M - r0);
-        for (int e = threadIdx.x; e < nr * M; e += blockDim.x) {
-            const int l = e / M, c = e % M;
-            B[l * P + c] = c < nin ? S[(r0 + l) * sw + c] : Cx<R>::mk(0, 0);
-        }
-        __syncthreads();
-        fft_dif<LOG2M>(B, nr, P, 1, s_tw, false);  // forward z (bit-reversed kz)
-        for (int e = threadIdx.x; e < nr * M; e += blockDim.x) {
-            const int l = e / M, c = e % M;
-            const int ky0 = brev_bits(r0 + l, LOG2M), kz0 = brev_bits(c, LOG2M);
-            const int ky = ky0 < M - ky0 ? ky0 : M - ky0;
-            const int kz = kz0 < M - kz0 ? kz0 : M - kz0;
-            const R k = khat[((long)kx * MH + ky) * MH + kz];
-            C v = B[l * P + c];
-            v.x *= k;
-            v.y *= k;
-            B[l * P + c] = v;
-        }
-        __syncthreads();
-        fft_dit<LOG2M>(B, nr, P, 1, s_tw, true);  // inverse z (natural z)
-        for (int e = threadIdx.x; e < nr * nz; e += blockDim.x) {
-            const int l = e / nz, jz = e % nz;
-            const int pz = (pos0 + a.zrow[jz]) % M;
-            S[(r0 + l) * sw + jz] = B[l * P + pz];
-        }
-        __syncthreads();
-    }
-    // inverse y on the nz output columns (bit-reversed ky in, natural y out)
-    fft_dit<LOG2M>(S, nz, 1, sw, s_tw, true);
-    C *out = (C *)a.it.a4 + q * a.nz * a.blk;
-    for (int e = threadIdx.x; e < nz * W; e += blockDim.x) {
-        const int jz = e / W, yo = e % W;
-        const int py = (pos0 + yo) % M;
-        out[(long)jz * a.blk + kx * W + yo] = S[py * sw + jz];
-    }
-}
-
-// ---------------------------------------------------------------------------
 // 64-point FFT of one line by 8 threads (radix 8 x 8, registers + one
 // exchange through the line's own shared-memory storage).  n = 8 n2 + n1,
 // k = k1 + 8 k2:  Y[n1][k1] = w64^(n1 k1) sum_n2 x[8 n2 + n1] w8^(n2 k1),
@@ -648,9 +557,6 @@ __device__ __forceinline__ void fft64_lines(C *base, int nlines, int lstride, in
 // Row pitch of the 64-point line buffers: 68 (4 mod 16) for FP32, 65 for FP64
 // (both conflict-free for the line loads and stores).
 template <typename R> struct Pitch64 { static constexpr int P = sizeof(R) == 4 ? 68 : 65; };
-// Lines exchange through a separate padded buffer (FP32 and double-float
-// complex entries); plain FP64 lines exchange in place.
-template <typename R> struct UseXs { static constexpr bool v = !std::is_same<R, double>::value; };
 
 // First radix-8 butterfly of a line whose inputs 3..7 are zero (the forward
 // passes, whose n+1 <= 24 nonzero samples sit at positions 8 n2 + t, n2 < 3):
@@ -707,135 +613,6 @@ __device__ __forceinline__ void line64_regs(C (&v)[8], int t, const C (&wt)[8], 
     __syncwarp();
     dft8<C, R>(v, inv);
 }
-
-// Fused slab for M = 64 (same contract as k_slab), radix 8 x 8 over 8-thread
-// line groups: the FP64 tier runs it with R = dfl (double-float arithmetic on
-// FP64 data); the split tier uses k_slab64r instead.  The slab is S[z][y]
-// (row pitch P).  Passes: forward y on the nin nonzero z rows; per y column,
-// forward z, product with the real kernel spectrum and inverse z in registers
-// (only the z rows the inverse-x step reads are stored back); inverse y on
-// those rows only.  Requires nin <= 24.
-template <typename R>
-__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2) k_slab64(SlabArgs a) {
-    using C = typename Cx<R>::T;
-    constexpr int M = 64, MH = 33, P = Pitch64<R>::P;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    C *tw64 = (C *)smem_raw;  // 64 twiddles exp(-2 pi i j / 64)
-    C *S = tw64 + M;
-    C *xs = S + M * P;        // blockDim/8 x 72 exchange entries
-    int *rowoff = (int *)(xs + 32 * 72);
-    const int nin = a.nin, W = a.nout;
-    const C *tw = (const C *)a.tw;  // M/2 entries; extend by w^(j+32) = -w^j
-    for (int j = threadIdx.x; j < M; j += blockDim.x) {
-        C w = tw[j & 31];
-        if (j >= 32) { w.x = -w.x; w.y = -w.y; }
-        tw64[j] = w;
-    }
-    // output z rows as slab rows (the field box starts at out_off, wrapped mod M)
-    unsigned long long rowmask = 0;
-    for (int j = 0; j < a.nz; ++j) {
-        int pz = (a.out_off + a.zrow[j]) % M;
-        if (pz < 0) pz += M;
-        rowmask |= 1ull << pz;
-        if (threadIdx.x == 0) rowoff[j] = pz * P;
-    }
-    const int grp = threadIdx.x >> 3, t = threadIdx.x & 7, ngrp = blockDim.x >> 3;
-    C *gx = xs + grp * 72;
-    // blockDim.x steps in (row, column) of the nin x nin input and nz x W output blocks
-    const int d_in_z = blockDim.x / nin, d_in_y = blockDim.x - d_in_z * nin;
-    const int d_out_z = blockDim.x / W, d_out_y = blockDim.x - d_out_z * W;
-    __syncthreads();
-    C wt[8];
-#pragma unroll
-    for (int k1 = 0; k1 < 8; ++k1) wt[k1] = tw64[(t * k1) & 63];
-    const C zero = Cx<R>::mk(0, 0);
-    // one slab per CTA, or (persistent launch) a grid-stride loop over slabs
-    const int nunits = a.it.nitems * MH;
-    for (int unit = blockIdx.x; unit < nunits; unit += gridDim.x) {
-        const int kx = unit % MH;
-        int p;
-        const PlanPtrs &PP = item_plan(a.it, unit / MH, p);
-        const long q = unit / MH;  // scratch slot
-        const C *in = (const C *)a.it.a1 + (q * MH + kx) * nin * nin;
-        // (zi, yi) of element e stepped incrementally (one division per thread)
-        for (int e = threadIdx.x, zi = e / nin, yi = e - zi * nin; e < nin * nin; e += blockDim.x) {
-            S[zi * P + yi] = in[e];
-            yi += d_in_y;
-            zi += d_in_z;
-            if (yi >= nin) { yi -= nin; ++zi; }
-        }
-        __syncthreads();
-        // forward y on the nin nonzero z rows
-        for (int l0 = 0; l0 < nin; l0 += ngrp) {
-            const int l = l0 + grp;
-            const bool valid = l < nin;
-            C *line = S + (valid ? l * P : 0);
-            C v[8];
-#pragma unroll
-            for (int n2 = 0; n2 < 8; ++n2) {
-                const int pos = 8 * n2 + t;
-                v[n2] = (n2 < 3 && valid && pos < nin) ? line[pos] : zero;
-            }
-            line64_regs<C, R, true>(v, t, wt, false, gx);
-#pragma unroll
-            for (int k2 = 0; k2 < 8; ++k2)
-                if (valid) line[t + 8 * k2] = v[k2];
-        }
-        __syncthreads();
-        // per y column: forward z, kernel product, inverse z (64 columns)
-        const R *khat = (const R *)PP.khat + (long)kx * MH * MH;
-        for (int ky0 = grp; ky0 < M; ky0 += ngrp) {
-            C *col = S + ky0;
-            C v[8];
-#pragma unroll
-            for (int n2 = 0; n2 < 8; ++n2) {
-                const int pos = 8 * n2 + t;
-                v[n2] = (n2 < 3 && pos < nin) ? col[pos * P] : zero;
-            }
-            line64_regs<C, R, true>(v, t, wt, false, gx);
-            const R *kk = khat + (ky0 < M - ky0 ? ky0 : M - ky0) * MH;
-#pragma unroll
-            for (int k2 = 0; k2 < 8; ++k2) {
-                const int kz0 = t + 8 * k2;
-                const R k = kk[kz0 < M - kz0 ? kz0 : M - kz0];
-                v[k2].x *= k;
-                v[k2].y *= k;
-            }
-            // the kernel products are nearly normalised already (residual ~2^-24 |p|)
-            line64_regs<C, R, false, false>(v, t, wt, true, gx);
-#pragma unroll
-            for (int k2 = 0; k2 < 8; ++k2) {
-                const int z = t + 8 * k2;
-                if ((rowmask >> z) & 1ull) col[z * P] = v[k2];
-            }
-        }
-        __syncthreads();
-        // inverse y on the output z rows
-        for (int l0 = 0; l0 < a.nz; l0 += ngrp) {
-            const int l = l0 + grp;
-            const bool valid = l < a.nz;
-            C *line = S + (valid ? rowoff[l] : 0);
-            C v[8];
-#pragma unroll
-            for (int n2 = 0; n2 < 8; ++n2) v[n2] = valid ? line[8 * n2 + t] : zero;
-            line64_regs<C, R, false>(v, t, wt, true, gx);
-#pragma unroll
-            for (int k2 = 0; k2 < 8; ++k2)
-                if (valid) line[t + 8 * k2] = v[k2];
-        }
-        __syncthreads();
-        C *out = (C *)a.it.a4 + q * a.nz * a.blk + kx * W;
-        for (int e = threadIdx.x, jz = e / W, yo = e - jz * W; jz < a.nz; e += blockDim.x) {
-            out[(long)jz * a.blk + yo] = S[rowoff[jz] + ((a.out_off + yo) & (M - 1))];
-            yo += d_out_y;
-            jz += d_out_z;
-            if (yo >= W) { yo -= W; ++jz; }
-        }
-        __syncthreads();  // S is rewritten by the next unit
-    }
-}
-
-
 
 // ---------------------------------------------------------------------------
 // Split tier slab with one 64-point line per thread: the whole transform of a
@@ -934,7 +711,7 @@ __host__ __device__ constexpr int brev6(int i) {
     return ((i & 1) << 5) | ((i & 2) << 3) | ((i & 4) << 1) | ((i & 8) >> 1) | ((i & 16) >> 3) | ((i & 32) >> 5);
 }
 
-// Same contract as k_slab64, for the split tier (FP32; 64 threads: one line each).  Passes:
+// Same contract as k_slab, for M = 64 (64 threads: one line each).  Passes:
 // forward y on the nin nonzero z rows; per y column, forward z (bit-reversed
 // result), product with the real kernel spectrum, inverse z back to natural
 // order, all in registers, storing only the z rows read later; inverse y on
@@ -1222,15 +999,6 @@ __global__ void __launch_bounds__(256, 2) k_slab128r(SlabArgs a) {
 __device__ __forceinline__ float2 shfl8(float2 v, int src) {
     return make_float2(__shfl_sync(0xffffffffu, v.x, src, 8), __shfl_sync(0xffffffffu, v.y, src, 8));
 }
-__device__ __forceinline__ double2 shfl8(double2 v, int src) {
-    return make_double2(__shfl_sync(0xffffffffu, v.x, src, 8), __shfl_sync(0xffffffffu, v.y, src, 8));
-}
-__device__ __forceinline__ dcx shfl8(dcx v, int src) {
-    dcx r;
-    r.x = dfl(__shfl_sync(0xffffffffu, v.x.hi, src, 8), __shfl_sync(0xffffffffu, v.x.lo, src, 8));
-    r.y = dfl(__shfl_sync(0xffffffffu, v.y.hi, src, 8), __shfl_sync(0xffffffffu, v.y.lo, src, 8));
-    return r;
-}
 
 // Forward real transform along x of the patch charges for M = 64 (the first
 // pass of the local convolution): one CTA per patch.  The chi-weighted
@@ -1373,7 +1141,7 @@ __global__ void __launch_bounds__(256) k_inv_x_pruned(InvXPArgs a) {
     C *tw = (C *)smem_raw;        // M twiddles
     C *raw = tw + M;              // MH x W (block of a.blk entries, 16-byte aligned)
     C *buf = raw + a.blk;         // up to a.maxfft lines of LP
-    C *xs = (LOG2M == 6 && UseXs<R>::v) ? buf + a.maxfft * LP : nullptr;
+    C *xs = LOG2M == 6 ? buf + a.maxfft * LP : nullptr;
     const int jz = blockIdx.x % a.nz, zi = a.zrow[jz];
     int p;
     const PlanPtrs &PP = item_plan(a.it, blockIdx.x / a.nz, p);
@@ -2995,38 +2763,24 @@ inline size_t fft_smem_bytes(int M, int lines, int ls) {
     return ((size_t)(M / 2) + (size_t)lines * ls) * 2 * sizeof(R);
 }
 
-// Local-convolution (patch) kernels in working precision R.
-// Largest dynamic shared memory of the 16-byte-entry M = 128 slab and
-// inverse-x launches: the 227 KB opt-in limit of an sm_100-class SM less room
-// for the kernels' static shared memory (the attribute cannot exceed the
-// difference).
-constexpr size_t kSlabRowsSmem = 225 * 1024;
+// Largest dynamic shared memory of the M = 128 launches: the 227 KB opt-in
+// limit less room for the kernels' static shared memory (the attribute cannot
+// exceed the difference).
+constexpr size_t kPatchSmem = 225 * 1024;
 
-template <int LOG2M, typename R>
+template <int LOG2M>
 void set_patch_attrs() {
     const int big = 200 * 1024;
-    if constexpr (LOG2M == 7 && !std::is_same<R, float>::value) {
-        cudaFuncSetAttribute(k_slab_rows<LOG2M, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSlabRowsSmem);
-        cudaFuncSetAttribute(k_inv_x_pruned<LOG2M, R, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSlabRowsSmem);
-        cudaFuncSetAttribute(k_fwd_x<LOG2M, double, true, R, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
-        return;
-    }
-    cudaFuncSetAttribute(k_fwd_x<LOG2M, double, true, R, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
-    cudaFuncSetAttribute(k_fwd_x<LOG2M, float, true, R, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
-    cudaFuncSetAttribute(k_slab<LOG2M, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
-    if constexpr (!std::is_same<R, float>::value)
-        cudaFuncSetAttribute(k_slab64<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
-    cudaFuncSetAttribute(k_slab64r<17>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
-    cudaFuncSetAttribute(k_slab64r<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
-    cudaFuncSetAttribute(k_inv_x_pruned<LOG2M, R, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
-    cudaFuncSetAttribute(k_inv_x64<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
+    cudaFuncSetAttribute(k_fwd_x<LOG2M, float, true, float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
+    cudaFuncSetAttribute(k_inv_x_pruned<LOG2M, float, float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         LOG2M == 7 ? (int)kPatchSmem : big);
 }
 
 // Local convolutions of a set of patches: forward x (real), fused slab (y,
 // z, kernel spectrum, inverse z, inverse y), pruned inverse x.  3 launches.
-template <int LOG2M, typename R>
-cudaError_t run_patch_conv_t(const mlc_plan_s *pl, const Items &it, bool f32, const void *tw,
-                             cudaStream_t st) {
+template <int LOG2M>
+cudaError_t run_patch_conv_t(const mlc_plan_s *pl, const Items &it, const void *tw, cudaStream_t st) {
+    using R = float;
     constexpr int M = 1 << LOG2M, MH = M / 2 + 1;
     const Geom &g = pl->g;
     const int nin = g.nb, W = g.W, nb = it.nitems;
@@ -3034,13 +2788,11 @@ cudaError_t run_patch_conv_t(const mlc_plan_s *pl, const Items &it, bool f32, co
     {
         FwdXArgs a{nullptr, nullptr, 0, g.n, 0, nin, nin, tw, it};
         if (LOG2M == 6 && nin <= 24) {  // register transform of line pairs
-            if (f32) k_fwd_x64<float, R><<<nb, 256, 0, st>>>(a);
-            else k_fwd_x64<double, R><<<nb, 256, 0, st>>>(a);
+            k_fwd_x64<float, R><<<nb, 256, 0, st>>>(a);
         } else {
             dim3 grid(nb * nin, 1);
             size_t sm = fft_smem_bytes<R>(M, nin, M + 1);
-            if (f32) k_fwd_x<LOG2M, float, true, R, true><<<grid, 256, sm, st>>>(a);
-            else k_fwd_x<LOG2M, double, true, R, true><<<grid, 256, sm, st>>>(a);
+            k_fwd_x<LOG2M, float, true, R, true><<<grid, 256, sm, st>>>(a);
         }
     }
     int nz = 0, zrow[128];
@@ -3052,57 +2804,28 @@ cudaError_t run_patch_conv_t(const mlc_plan_s *pl, const Items &it, bool f32, co
     {
         SlabArgs a{tw, nin, W, -g.s, it, nz, {}, g.a4blk};
         for (int j = 0; j < nz; ++j) a.zrow[j] = zrow[j];
-        if (LOG2M == 6) {
-            int dev = 0, nsm = 0, occ = 0;
-            if (it.persist) {  // one wave of resident CTAs walking all slabs
-                cudaGetDevice(&dev);
-                cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-            }
-            if constexpr (std::is_same<R, float>::value) {  // split tier: one line per thread
-                const size_t smr = (size_t)M * 65 * sizeof(float2);
-                int gr = nb * MH;
-                if (it.persist) {
-                    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_slab64r<32>, 64, smr);
-                    const int wave = nsm * (occ > 0 ? occ : 1);
-                    gr = gr < wave ? gr : wave;
-                }
-                if (nin <= 17) k_slab64r<17><<<gr, 64, smr, st>>>(a);
-                else k_slab64r<32><<<gr, 64, smr, st>>>(a);
-            } else if (nin > 24) {  // k_slab64's sparse forward passes take nin <= 24 (n = 24)
-                k_slab<LOG2M, R><<<nb * MH, 256, fft_smem_bytes<R>(M, M, M + 1), st>>>(a);
-            } else {  // FP64 and double-float: radix 8 x 8 over 8-thread groups
-                const size_t sm = (size_t)(M + M * Pitch64<R>::P + 32 * 72) * sizeof(typename Cx<R>::T) + 64 * sizeof(int);
-                int grid = nb * MH;
-                if (it.persist) {
-                    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_slab64<R>, 256, sm);
-                    const int wave = nsm * (occ > 0 ? occ : 1);
-                    grid = grid < wave ? grid : wave;
-                }
-                k_slab64<R><<<grid, 256, sm, st>>>(a);
-            }
+        int dev = 0, nsm = 0, occ = 0, gr = nb * MH;
+        if (it.persist && LOG2M > 5) {  // one wave of resident CTAs walking all slabs
+            cudaGetDevice(&dev);
+            cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
         }
-        else {
-            if constexpr (LOG2M == 7 && std::is_same<R, float>::value) {  // FP32: register lines
-                const size_t sm = ((size_t)144 + 32 * 152 + (size_t)std::max(nin, nz) * (M + 1)) * sizeof(float2);
-                int gr = nb * MH;
-                if (it.persist) {
-                    int dev = 0, nsm = 0, occ = 0;
-                    cudaGetDevice(&dev);
-                    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-                    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_slab128r, 256, sm);
-                    const int wave = nsm * (occ > 0 ? occ : 1);
-                    gr = gr < wave ? gr : wave;
-                }
-                k_slab128r<<<gr, 256, sm, st>>>(a);
-            } else if constexpr (LOG2M == 7 && sizeof(R) == 8) {  // 16-byte entries: row-streamed slab
-                const int sw = std::max(nin, nz);
-                const size_t csz = 2 * sizeof(R), fixed = ((size_t)M / 2 + (size_t)M * sw) * csz;
-                const int rb = (int)std::min<size_t>(M, (kSlabRowsSmem - fixed) / ((M + 1) * csz));
-                if (rb < 1) return cudaErrorInvalidValue;
-                k_slab_rows<LOG2M, R><<<nb * MH, 256, fixed + (size_t)rb * (M + 1) * csz, st>>>(a, sw, rb);
-            } else {
-                k_slab<LOG2M, R><<<nb * MH, 256, fft_smem_bytes<R>(M, M, M + 1), st>>>(a);
+        if constexpr (LOG2M == 5) {
+            k_slab<LOG2M, R><<<gr, 256, fft_smem_bytes<R>(M, M, M + 1), st>>>(a);
+        } else if constexpr (LOG2M == 6) {  // one line per thread
+            const size_t smr = (size_t)M * 65 * sizeof(float2);
+            if (it.persist) {
+                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_slab64r<32>, 64, smr);
+                gr = std::min(gr, nsm * (occ > 0 ? occ : 1));
             }
+            if (nin <= 17) k_slab64r<17><<<gr, 64, smr, st>>>(a);
+            else k_slab64r<32><<<gr, 64, smr, st>>>(a);
+        } else {  // register lines
+            const size_t sm = ((size_t)144 + 32 * 152 + (size_t)std::max(nin, nz) * (M + 1)) * sizeof(float2);
+            if (it.persist) {
+                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_slab128r, 256, sm);
+                gr = std::min(gr, nsm * (occ > 0 ? occ : 1));
+            }
+            k_slab128r<<<gr, 256, sm, st>>>(a);
         }
     }
     mark(pl, 3, st);
@@ -3134,17 +2857,15 @@ cudaError_t run_patch_conv_t(const mlc_plan_s *pl, const Items &it, bool f32, co
             a.maxfft = cnt > a.maxfft ? cnt : a.maxfft;
         }
         const int LPh = LOG2M == 6 ? Pitch64<R>::P : M + 1;
-        const size_t xsn = (LOG2M == 6 && UseXs<R>::v) ? 32 * 72 : 0;
+        const size_t xsn = LOG2M == 6 ? 32 * 72 : 0;
         // transformed rows per pass: all of them unless the line buffer would
         // not fit beside the staged block (16-byte entries at M = 128)
         const size_t fixed = ((size_t)M + (size_t)g.a4blk + xsn) * 2 * sizeof(R);
         const size_t line = (size_t)LPh * 2 * sizeof(R);
         a.rb = a.maxfft;
-        if (fixed + (size_t)a.rb * line > kSlabRowsSmem) a.rb = (int)((kSlabRowsSmem - fixed) / line);
+        if (fixed + (size_t)a.rb * line > kPatchSmem) a.rb = (int)((kPatchSmem - fixed) / line);
         if (a.rb < 1) return cudaErrorInvalidValue;
         const size_t sm = fixed + (size_t)a.rb * line;
-        // local fields leave in the working precision: FP32 (split tier) or
-        // double-float pairs (FP64 tier)
         if (LOG2M == 6 && !g.wide) {
             const int thr = 128;  // 16 line groups: one pass over the row pairs of a z row
             const size_t sm64 = ((size_t)M + (size_t)g.a4blk + (thr / 8) * 72) * sizeof(typename Cx<R>::T) +
@@ -3178,19 +2899,18 @@ cudaError_t launch_set_ptrs(PlanPtrs *d, const void *f, double *phi, cudaStream_
 }
 
 void configure_kernels() {
-    set_patch_attrs<5, dfl>();
-    set_patch_attrs<6, dfl>();
-    set_patch_attrs<5, float>();
-    set_patch_attrs<6, float>();
-    set_patch_attrs<5, double>();
-    set_patch_attrs<6, double>();
-    set_patch_attrs<7, float>();
-    cudaFuncSetAttribute(k_slab128r, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSlabRowsSmem);
-    set_patch_attrs<7, double>();
-    set_patch_attrs<7, dfl>();
+    set_patch_attrs<5>();
+    set_patch_attrs<6>();
+    set_patch_attrs<7>();
+    cudaFuncSetAttribute(k_inv_x64<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    cudaFuncSetAttribute(k_slab64r<17>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    cudaFuncSetAttribute(k_slab64r<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    cudaFuncSetAttribute(k_slab128r, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPatchSmem);
     set_cfft_attrs<dfl>();
     set_cfft_attrs<double>();
     configure_ring_gemm();
+    configure_limb();
+    configure_limb_conv();
     const int big = 200 * 1024;
 #define MLC_DIR_ATTR(NN)                                                                          \
     cudaFuncSetAttribute(k_dirichlet<double, NN, double>, cudaFuncAttributeMaxDynamicSharedMemorySize, big); \
@@ -3234,31 +2954,23 @@ cudaError_t launch_moments(const mlc_plan_s *pl, const Items &it, cudaStream_t s
     return cudaGetLastError();
 }
 
-// The three local-convolution launches for one launch group of items (its
-// scratch in it.a1 / it.a4).
+// The three local-convolution launches of the split tiers for one launch group
+// of items (its scratch in it.a1 / it.a4).
 cudaError_t launch_patch_conv_group(const mlc_plan_s *pl, const Items &it, cudaStream_t st) {
     NvtxRange nvtx("mlc:local_convolutions");
-    const Geom &g = pl->g;
-    const bool f32 = g.f32in;
-    if (g.conv == CONV_F32) {  // split tiers: FP32 (tables tw_f, khat_f)
-        if (g.log2M == 5) return run_patch_conv_t<5, float>(pl, it, f32, pl->tw_f, st);
-        if (g.log2M == 6) return run_patch_conv_t<6, float>(pl, it, f32, pl->tw_f, st);
-        if (g.log2M == 7) return run_patch_conv_t<7, float>(pl, it, f32, pl->tw_f, st);
-    } else if (g.conv == CONV_DF) {  // double-float (tables tw_df, khat_df)
-        if (g.log2M == 5) return run_patch_conv_t<5, dfl>(pl, it, f32, pl->tw_df, st);
-        if (g.log2M == 6) return run_patch_conv_t<6, dfl>(pl, it, f32, pl->tw_df, st);
-        if (g.log2M == 7) return run_patch_conv_t<7, dfl>(pl, it, f32, pl->tw_df, st);
-    } else {  // FP64 (tables tw, khat)
-        if (g.log2M == 5) return run_patch_conv_t<5, double>(pl, it, f32, pl->tw, st);
-        if (g.log2M == 6) return run_patch_conv_t<6, double>(pl, it, f32, pl->tw, st);
-        if (g.log2M == 7) return run_patch_conv_t<7, double>(pl, it, f32, pl->tw, st);
+    switch (pl->g.log2M) {
+        case 5: return run_patch_conv_t<5>(pl, it, pl->tw_f, st);
+        case 6: return run_patch_conv_t<6>(pl, it, pl->tw_f, st);
+        case 7: return run_patch_conv_t<7>(pl, it, pl->tw_f, st);
     }
     return cudaErrorInvalidValue;
 }
 
-// Local convolutions of all items, in launch groups of g.chunk items that
-// reuse one scratch (stream order keeps the groups apart).
+// Local convolutions of all items: FP32 transforms (split tiers) in launch
+// groups of g.chunk items that reuse one scratch (stream order keeps the groups
+// apart), or the exact-split products of limb_conv.cu (FP64, double-float).
 cudaError_t launch_patch_conv(const mlc_plan_s *pl, const Items &it, cudaStream_t st) {
+    if (pl->g.conv != CONV_F32) return launch_limb_conv(pl, it, st);
     const int chunk = it.chunk > 0 ? it.chunk : pl->g.chunk;
     for (int c0 = 0; c0 < it.nitems; c0 += chunk) {
         Items ic = it;

@@ -1,0 +1,542 @@
+// Local convolutions phi^{i,h} = G^h * f^{i,h} (eq. initiallocalproblemsmlcII)
+// of the FP64 and double-float tiers as one exact-split tensor-core product
+// (limb.h) of the folded Green's function with the folded patch charges:
+//
+//   k_limb_fold     charge -> even / odd parts along the three axes -> digits
+//   k_limb_gemm     per parity class, outputs x inputs by inputs x patches
+//   k_limb_unfold   even / odd outputs -> the coarse lattice of the field box
+//                   and the face planes (Q = 10: and the planes next to them)
+//
+// Only the values the later steps read are formed: a quarter of the field box
+// per axis for the lattice and a few planes of the inner box, 5947 of 117649
+// nodes for n = 16, s = 16, Q = 6.  Against those an FFT pays for whole lines
+// on the FP64 pipe (2 lanes per SM and cycle); the product is 7.4 MFLOP per patch
+// after folding, times 28 digit pairs on FP16 tensor cores.  256^3, FP64, in ms,
+// transforms before and fold + product + unfold now:
+//   n = 16, s = 16, Q = 6 (4096 patches)   53.9   0.53 + 1.19 + 0.19
+//   n = 32, s = 28, Q = 6 (512 patches)    91.0   0.90 + 6.00 + 0.16
+// and 8^3 patches of a 32^3 problem 0.17 -> 0.077, so no size is left to the
+// transforms.  The error against long double sums is below that of the FP64
+// transforms for smooth, constant and random charges (n = 16, s = 16: 9e-17,
+// 2e-17 and 1.5e-16 of the largest value, against 2.7e-16, 6.4e-16 and 5.1e-16).
+#include <algorithm>
+#include <cmath>
+#include <map>
+#include <mutex>
+#include <tuple>
+#include <vector>
+
+#include <cuda_fp16.h>
+
+#include "limb.h"
+#include "mlc_internal.h"
+
+namespace mlc {
+namespace {
+
+constexpr int kBias = 55;  // |X| <= 2^55
+
+// Seven balanced base-256 digits of X: byte 6 - i of the result is d_i + 128
+// (d_0 = 128, at the very top of the range, carries into bit 56).
+__device__ __forceinline__ unsigned long long digit_bytes(long long X) {
+    return (unsigned long long)(X + 0x0080808080808080ll);
+}
+
+// X = rint(x 2^(55 - e)) for |x| < 2^e, from the bits (round half up; emax: biased
+// exponent of the block's largest magnitude, so e = emax - 1022).
+__device__ __forceinline__ long long to_limb_int(double x, int emax) {
+    const long long b = __double_as_longlong(x);
+    const int ex = (int)((b >> 52) & 0x7ff);
+    long long m = (b & 0xfffffffffffffll) | (ex ? 1ll << 52 : 0);
+    const int sh = emax - (ex ? ex : 1);  // >= 0
+    // at the largest exponent 53 bits become 55
+    m = sh <= 2 ? m << (2 - sh) : (sh > 55 ? 0 : (m >> (sh - 2)) + ((m >> (sh - 3)) & 1));
+    return b < 0 ? -m : m;
+}
+
+// The same digit (0 = leading) of eight numbers as four half2.
+__device__ __forceinline__ uint4 digit_chunk(const unsigned long long (&Y)[8], int i) {
+    uint4 r;
+    unsigned *w = &r.x;
+    const __half2 off = __half2half2(__ushort_as_half(0x6480));  // 1024 + 128
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const unsigned mask = i == 0 ? 0x1ff : 0xff;
+        const unsigned a = (unsigned)(Y[2 * j] >> (8 * (6 - i))) & mask, b = (unsigned)(Y[2 * j + 1] >> (8 * (6 - i))) & mask;
+        const unsigned pk = 0x64006400u + a + (b << 16);  // 1024 + byte, exactly
+        __half2 h = *(const __half2 *)&pk;
+        h = __hsub2(h, off);
+        w[j] = *(const unsigned *)&h;
+    }
+    return r;
+}
+
+__device__ __forceinline__ int biased_exp(double x) { return (int)((__double_as_longlong(x) >> 52) & 0x7ff); }
+
+// ---------------------------------------------------------------------------
+// Tables: one CTA per row of one table.  Entry (row, k) is the Green's function
+// (h = 1) between the row's point and the column's, folded along each axis:
+// 1/8 sum over the mirror images of the input point, negative along odd axes.
+// ---------------------------------------------------------------------------
+__global__ void __launch_bounds__(256) k_limb_table(LimbConvGeom g, int u, const double *G1, int L, unsigned char *A,
+                                                    double *rf) {
+    extern __shared__ double val[];  // kst x 16
+    __shared__ int smax;
+    const int row = blockIdx.x, K = g.K[u], kpad = g.kst[u] * 16, n = g.n;
+    if (threadIdx.x == 0) smax = 0;
+    __syncthreads();
+    int mx = 0;
+    if (row < g.rows[u]) {
+        int x[3];
+        limb_row_point(g, u, row, x);
+        for (int k = threadIdx.x; k < kpad; k += blockDim.x) {
+            double v = 0.0;
+            if (k < K) {
+                int m[3];
+                limb_col_point(g, u, k, m);
+#pragma unroll
+                for (int c = 0; c < 8; ++c) {
+                    long idx = 0;
+                    bool neg = false;
+#pragma unroll
+                    for (int d = 0; d < 3; ++d) {
+                        const bool mir = (c >> d) & 1;
+                        const int lag = abs(x[d] - (mir ? n - m[d] : m[d]));
+                        idx = idx * (L + 1) + lag;
+                        neg ^= mir && limb_odd(u, d);
+                    }
+                    const double q = G1[idx];
+                    v += neg ? -q : q;
+                }
+                v *= 0.125;
+            }
+            val[k] = v;
+            mx = max(mx, biased_exp(v));
+        }
+    } else {
+        for (int k = threadIdx.x; k < kpad; k += blockDim.x) val[k] = 0.0;
+    }
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    if ((threadIdx.x & 31) == 0) atomicMax(&smax, mx);
+    __syncthreads();
+    const int e = smax;
+    // |v| < 2^(e - 1022); value = X 2^(e - 1022 - 55), and the sums come as X Y / 2^48
+    if (threadIdx.x == 0) rf[g.rf_off[u] + row] = e ? ldexp(1.0, e - 1022 - 2 * kBias + 48) : 0.0;
+    unsigned char *At = A + g.a_off[u] + (long)(row / kLimbM) * g.kst[u] * kLimbAStep;
+    for (int q = threadIdx.x; q < kpad / 8; q += blockDim.x) {
+        unsigned long long Y[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) Y[j] = digit_bytes(e ? to_limb_int(val[8 * q + j], e) : 0);
+        unsigned char *p = At + limb_chunk_off(row % kLimbM, q, kLimbABlk);
+#pragma unroll
+        for (int i = 0; i < kLimbs; ++i) *(uint4 *)(p + i * kLimbABlk) = digit_chunk(Y, i);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Folded charges.  One CTA per patch: the chi-weighted closed-patch charge is
+// folded along axis 0 while it is read (one parity at a time, so that the array
+// of (n/2 + 1) (n + 1)^2 values fits shared memory for every patch size) and
+// along axes 1 and 2 in place; each class is then scaled by its own largest
+// magnitude and written as digits, columns in the operand layout.  The bytes
+// written (14 per charge) bound it at large n; at n = 16 the FP64 pipe does:
+// three sums per value.
+// ---------------------------------------------------------------------------
+struct FoldArgs {
+    Items it;
+    unsigned char *B;
+    double *cf;       // [class][cols_pad]
+    int n, ctiles;
+    LimbConvGeom g;
+};
+
+__global__ void __launch_bounds__(256) k_limb_fold(const __grid_constant__ FoldArgs a) {
+    extern __shared__ double S[];  // [m0][m1][m2], m0 <= n/2; odd parts at the mirrored index
+    __shared__ int smax[4];
+    int p;
+    const PlanPtrs &PP = item_plan(a.it, blockIdx.x, p);
+    const int n = a.n, nb = n + 1, h = n / 2, N = PP.N, np = PP.np;
+    const int i2 = p % np, i1 = (p / np) % np, i0 = p / (np * np);
+    const double *f = (const double *)PP.f;
+    const int col = blockIdx.x, ct = col / kLimbN, cl = col % kLimbN;
+    auto charge = [&](int m0, int m1, int m2) -> double {
+        const int z = i0 * n + m0, y = i1 * n + m1, x = i2 * n + m2;
+        if (z >= N || y >= N || x >= N) return 0.0;
+        const int faces = (m0 == 0 || m0 == n) + (m1 == 0 || m1 == n) + (m2 == 0 || m2 == n);
+        const double w = faces == 0 ? 1.0 : (faces == 1 ? 0.5 : (faces == 2 ? 0.25 : 0.125));
+        return w * f[((long)z * N + y) * N + x];
+    };
+    for (int p0 = 0; p0 < 2; ++p0) {
+        const int d0 = a.g.hin[p0];
+        for (int e = threadIdx.x; e < d0 * nb * nb; e += blockDim.x) {
+            const int m2 = e % nb, m1 = (e / nb) % nb, m0 = e / (nb * nb);
+            double v = charge(m0, m1, m2);
+            if (m0 != h) {
+                const double w = charge(n - m0, m1, m2);
+                v = p0 ? v - w : v + w;
+            }
+            S[e] = v;
+        }
+        if (threadIdx.x < 4) smax[threadIdx.x] = 0;
+        __syncthreads();
+        for (int e = threadIdx.x; e < d0 * h * nb; e += blockDim.x) {  // axis 1
+            const int m2 = e % nb, m1 = (e / nb) % h, m0 = e / (nb * h);
+            double *u = S + (m0 * nb + m1) * nb + m2, *w = S + (m0 * nb + n - m1) * nb + m2;
+            const double x = *u, y = *w;
+            *u = x + y;
+            *w = x - y;
+        }
+        __syncthreads();
+        // axis 2, and the largest exponent of each class (p1, p2)
+        int mx[4] = {0, 0, 0, 0};
+        for (int e = threadIdx.x; e < d0 * nb * (h + 1); e += blockDim.x) {
+            const int m2 = e % (h + 1), r = e / (h + 1), m1 = r % nb;
+            double *u = S + r * nb + m2;
+            const int c = m1 > h ? 2 : 0;
+            if (m2 < h) {
+                double *w = S + r * nb + n - m2;
+                const double x = *u, y = *w;
+                const double s = x + y, d = x - y;
+                *u = s;
+                *w = d;
+                if (c) { mx[2] = max(mx[2], biased_exp(s)); mx[3] = max(mx[3], biased_exp(d)); }
+                else { mx[0] = max(mx[0], biased_exp(s)); mx[1] = max(mx[1], biased_exp(d)); }
+            } else {
+                const int ex = biased_exp(*u);
+                if (c) mx[2] = max(mx[2], ex);
+                else mx[0] = max(mx[0], ex);
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int v = __reduce_max_sync(0xffffffffu, mx[q]);
+            if ((threadIdx.x & 31) == 0 && v) atomicMax(&smax[q], v);
+        }
+        __syncthreads();
+        for (int q = 0; q < 4; ++q) {
+            const int c = 4 * p0 + q, u = limb_table(a.g.share, c), e = smax[q];
+            const bool live = e != 0 && e != 0x7ff;
+            // infinities and NaN make the patch's whole local field NaN, as the transforms of one do
+            if (threadIdx.x == 0)
+                a.cf[(long)c * a.ctiles * kLimbN + col] =
+                    e == 0x7ff ? __longlong_as_double(0x7ff8000000000000ll) : (live ? ldexp(PP.h2, e - 1022) : 0.0);
+            unsigned char *Bt = a.B + a.g.b_step[c] * a.ctiles + (long)ct * a.g.kst[u] * kLimbBStep;
+            const int K = a.g.K[u];
+            const int q0 = limb_perm(a.g.share, c, 0), q1 = limb_perm(a.g.share, c, 1), q2 = limb_perm(a.g.share, c, 2);
+            // step of S along each table axis and its start: odd reps run down from the mirrored end
+            const int st[3] = {nb * nb, nb, 1};
+            const int o1 = (q & 2) ? n * nb : 0, o2 = (q & 1) ? n : 0, base = o1 + o2;
+            auto step = [&](int ax) { return ax == 0 ? st[0] : (ax == 1 ? ((q & 2) ? -nb : nb) : ((q & 1) ? -1 : 1)); };
+            const int s0 = step(q0), s1 = step(q1), s2 = step(q2);
+            const int d1 = a.g.hin[limb_odd(u, 1)], d2 = a.g.hin[limb_odd(u, 2)];
+            for (int w = threadIdx.x; w < a.g.kst[u] * 2; w += blockDim.x) {
+                unsigned long long Y[8];
+                int k = 8 * w, t2 = k % d2, t1 = (k / d2) % d1, t0 = k / (d2 * d1);
+#pragma unroll
+                for (int j = 0; j < 8; ++j, ++k) {
+                    Y[j] = digit_bytes(live && k < K ? to_limb_int(S[base + t0 * s0 + t1 * s1 + t2 * s2], e) : 0);
+                    if (++t2 == d2) {
+                        t2 = 0;
+                        if (++t1 == d1) { t1 = 0; ++t0; }
+                    }
+                }
+                unsigned char *o = Bt + limb_chunk_off(cl, w, kLimbBBlk);
+#pragma unroll
+                for (int i = 0; i < kLimbs; ++i) *(uint4 *)(o + i * kLimbBBlk) = digit_chunk(Y, i);
+            }
+        }
+        __syncthreads();
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Unfold: one CTA per patch.  Each representative output point reads its value
+// in the eight classes (those odd along an axis on which it is the centre are
+// zero) and gives the values at its up to eight mirror images.
+// ---------------------------------------------------------------------------
+struct UnfoldArgs {
+    Items it;
+    const double *V;
+    int cols;
+    int base[2][3][8];  // first row of the planes of (kind, axis) in each class's table
+    LimbConvGeom g;
+};
+
+template <typename TO> __device__ __forceinline__ TO limb_out(double v);
+template <> __device__ __forceinline__ double limb_out<double>(double v) { return v; }
+template <> __device__ __forceinline__ float2 limb_out<float2>(double v) {
+    const float hi = (float)v;
+    return make_float2(hi, (float)(v - (double)hi));
+}
+
+// Values at the mirror images: bit d of the index set: axis d mirrored.
+__device__ __forceinline__ void unfold8(double (&v)[8]) {
+#pragma unroll
+    for (int b = 1; b < 8; b <<= 1)
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            if (!(i & b)) {
+                const double x = v[i], y = v[i | b];
+                v[i] = x + y;
+                v[i | b] = x - y;
+            }
+}
+
+template <typename TO, bool SHARE>
+__global__ void __launch_bounds__(256) k_limb_unfold(const __grid_constant__ UnfoldArgs a) {
+    int p;
+    const PlanPtrs &PP = item_plan(a.it, blockIdx.x, p);
+    const LimbConvGeom &g = a.g;
+    const long item = blockIdx.x;
+    auto class_row = [&](int c) -> const double * {
+        return a.V + g.v_step[c] * a.cols + item * g.rows[limb_table(SHARE, c)];
+    };
+    // class values of the point with reps i[3] whose per-axis centre reps are cen[3] (-1: none);
+    // row(u, j0, j1, j2): the table row, in table axes
+    auto gather = [&](const int (&i)[3], const int (&cen)[3], auto &&row, double (&v)[8]) {
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+            bool zero = false;
+#pragma unroll
+            for (int d = 0; d < 3; ++d) zero |= limb_odd(c, d) && i[d] == cen[d];
+            // value index: bit d = odd along axis d
+            const int b = (limb_odd(c, 0) ? 1 : 0) | (limb_odd(c, 1) ? 2 : 0) | (limb_odd(c, 2) ? 4 : 0);
+            v[b] = zero ? 0.0 : class_row(c)[row(c, limb_table(SHARE, c), i[limb_perm(SHARE, c, 0)], i[limb_perm(SHARE, c, 1)],
+                                                   i[limb_perm(SHARE, c, 2)])];
+        }
+        unfold8(v);
+    };
+    const int n = g.n, nc = g.nc, wa = g.wa;
+    {   // coarse lattice
+        TO *cl = (TO *)PP.cl + (long)p * nc * nc * nc;
+        const int d = g.hl[0], centre = g.hl[0] > g.hl[1] ? g.hl[1] : -1;
+        const int cen[3] = {centre, centre, centre};
+        for (int e = threadIdx.x; e < d * d * d; e += blockDim.x) {
+            const int i[3] = {e / (d * d), (e / d) % d, e % d};
+            double v[8];
+            gather(i, cen, [&](int, int u, int k0, int k1, int k2) { return limb_lat_row(g, u, k0, k1, k2); }, v);
+#pragma unroll
+            for (int b = 0; b < 8; ++b) {
+                if (((b & 1) && i[0] == centre) || ((b & 2) && i[1] == centre) || ((b & 4) && i[2] == centre)) continue;
+                const int k0 = (b & 1) ? nc - 1 - i[0] : i[0], k1 = (b & 2) ? nc - 1 - i[1] : i[1],
+                          k2 = (b & 4) ? nc - 1 - i[2] : i[2];
+                cl[((long)k0 * nc + k1) * nc + k2] = limb_out<TO>(v[b]);
+            }
+        }
+    }
+    for (int kind = 0; kind < 2; ++kind) {  // face planes, then the planes next to them
+        const LimbPlanes &pl = kind ? g.off : g.face;
+        if (!pl.nrep) continue;
+        TO *fp = (TO *)(kind ? PP.fp2 : PP.fp) + (long)p * 3 * pl.per_axis * wa * wa;
+        const int hp = g.hp[0], centre = n / 2 + g.ga;
+        for (int ax = 0; ax < 3; ++ax) {
+            const int cen[3] = {ax == 0 ? -1 : centre, ax == 1 ? -1 : centre, ax == 2 ? -1 : centre};
+            for (int e = threadIdx.x; e < pl.nrep * hp * hp; e += blockDim.x) {
+                const int v2 = e % hp, u2 = (e / hp) % hp, r = e / (hp * hp);
+                const int i[3] = {ax == 0 ? r : u2, ax == 1 ? r : (ax == 0 ? u2 : v2), ax == 2 ? r : v2};
+                double v[8];
+                gather(i, cen,
+                       [&](int c, int u, int k0, int k1, int k2) {
+                           const int ta = limb_perm(SHARE, c, 0) == ax ? 0 : (limb_perm(SHARE, c, 1) == ax ? 1 : 2);
+                           const int kr = ta == 0 ? k0 : (ta == 1 ? k1 : k2);
+                           const int j1 = ta == 0 ? k1 : k0, j2 = ta == 2 ? k1 : k2;
+                           const int w1 = g.hp[limb_odd(u, ta == 0 ? 1 : 0)], w2 = g.hp[limb_odd(u, ta == 2 ? 1 : 2)];
+                           return a.base[kind][ax][c] + (kr * w1 + j1) * w2 + j2;
+                       },
+                       v);
+                const int bu = ax == 0 ? 2 : 1, bv = ax == 2 ? 2 : 4, ba = 1 << ax;  // mirror bits of the axes
+#pragma unroll
+                for (int b = 0; b < 8; ++b) {
+                    if (((b & bu) && u2 == centre) || ((b & bv) && v2 == centre)) continue;
+                    const int slot = ax * pl.per_axis + ((b & ba) ? pl.mslot[r] : pl.slot[r]);
+                    const int uu = (b & bu) ? wa - 1 - u2 : u2, vv = (b & bv) ? wa - 1 - v2 : v2;
+                    fp[((long)slot * wa + uu) * wa + vv] = limb_out<TO>(v[b]);
+                }
+            }
+        }
+    }
+}
+
+struct TabKey {
+    int device, n, s, ga, wide;
+    const double *dgf;
+    bool operator<(const TabKey &o) const {
+        return std::tie(device, n, s, ga, wide, dgf) < std::tie(o.device, o.n, o.s, o.ga, o.wide, o.dgf);
+    }
+};
+std::mutex g_tab_mu;
+std::map<TabKey, std::weak_ptr<LimbConvTables>> g_tabs;
+
+}  // namespace
+
+LimbConvTables::~LimbConvTables() {
+    cudaFree(A);
+    cudaFree(rf);
+}
+
+bool limb_conv_geometry(const Geom &G, bool share, LimbConvGeom &c) {
+    c = LimbConvGeom{};
+    c.share = share;
+    const int n = G.n, s = G.s, ga = G.ga;
+    c.n = n; c.s = s; c.ga = ga; c.nc = G.nc; c.wa = G.wa;
+    c.hin[0] = n / 2 + 1; c.hin[1] = n / 2;
+    c.hl[0] = (n / 2 + s) / 4 + 1;
+    c.hl[1] = c.hl[0] - ((n / 2 + s) % 4 == 0 ? 1 : 0);
+    c.hp[0] = n / 2 + ga + 1; c.hp[1] = n / 2 + ga;
+    c.face.per_axis = G.npa;
+    c.off.per_axis = 2 * G.npa;
+    for (int j = 0; j < G.npa; ++j) {
+        const int x = G.pl0 + j * n;
+        if (2 * x < n) {
+            if (c.face.nrep >= 24) return false;
+            const int r = c.face.nrep++;
+            c.face.c[r] = x; c.face.slot[r] = j; c.face.mslot[r] = G.npa - 1 - j;
+        }
+        if (!G.wide) continue;
+        for (int sd = 0; sd < 2; ++sd) {
+            const int y = x + (sd ? 1 : -1);
+            if (y < -ga || y > n + ga || 2 * y >= n) continue;
+            if (c.off.nrep >= 24) return false;
+            const int r = c.off.nrep++;
+            c.off.c[r] = y; c.off.slot[r] = 2 * j + sd; c.off.mslot[r] = 2 * (G.npa - 1 - j) + (1 - sd);
+        }
+    }
+    for (int u = 0; u < 8; ++u) {
+        if (limb_table(share, u) != u) continue;
+        c.K[u] = c.hin[limb_odd(u, 0)] * c.hin[limb_odd(u, 1)] * c.hin[limb_odd(u, 2)];
+        c.kst[u] = (c.K[u] + 15) / 16;
+        c.rows[u] = limb_lat_rows(c, u);
+        for (int a = 0; a < 3; ++a) c.rows[u] += limb_plane_rows(c, u, c.face, a) + limb_plane_rows(c, u, c.off, a);
+        c.tiles[u] = (c.rows[u] + kLimbM - 1) / kLimbM;
+        c.a_off[u] = c.a_bytes;
+        c.rf_off[u] = c.rf_rows;
+        c.a_bytes += (long)c.tiles[u] * c.kst[u] * kLimbAStep;
+        c.rf_rows += (long)c.tiles[u] * kLimbM;
+    }
+    for (int k = 0; k < 8; ++k) {
+        const int u = limb_table(share, k);
+        c.b_step[k] = c.b_total;
+        c.v_step[k] = c.v_total;
+        c.b_total += (long)c.kst[u] * kLimbBStep;
+        c.v_total += c.rows[u];
+    }
+    return true;
+}
+
+cudaError_t limb_conv_tables(int device, const Geom &G, bool share, const double *dgf, int dgf_L,
+                             std::shared_ptr<LimbConvTables> *out) {
+    std::lock_guard<std::mutex> lk(g_tab_mu);
+    const TabKey key{device, G.n, G.s, G.ga, G.wide ? 1 : 0, dgf};
+    if (auto have = g_tabs[key].lock()) {
+        *out = have;
+        return cudaSuccess;
+    }
+    auto t = std::make_shared<LimbConvTables>();
+    if (!limb_conv_geometry(G, share, t->g)) return cudaErrorInvalidValue;
+    cudaError_t e = cudaMalloc((void **)&t->A, (size_t)t->g.a_bytes);
+    if (e == cudaSuccess) e = cudaMalloc((void **)&t->rf, (size_t)t->g.rf_rows * sizeof(double));
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return e;
+    }
+    for (int u = 0; u < 8; ++u)
+        if (t->g.tiles[u])
+            k_limb_table<<<t->g.tiles[u] * kLimbM, 256, (size_t)t->g.kst[u] * 16 * sizeof(double)>>>(t->g, u, dgf, dgf_L,
+                                                                                                 t->A, t->rf);
+    e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaDeviceSynchronize();
+    if (e != cudaSuccess) return e;
+    g_tabs[key] = t;
+    *out = t;
+    return cudaSuccess;
+}
+
+void configure_limb_conv() {
+    const int big = 160 * 1024;
+    cudaFuncSetAttribute(k_limb_fold, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
+}
+
+// Patches per launch group: as many as the scratch holds, in groups of one size.
+static long limb_group(const Geom &g, size_t cap, long items) {
+    long m = 0;
+    for (long ct = limb_ctiles(items); ct > 0 && m == 0; --ct) {
+        if (ct * g.limb_tile_bytes >= cap) continue;
+        const long fit = std::min({items, ct * kLimbN, (long)((cap - ct * g.limb_tile_bytes) / g.limb_item_bytes)});
+        if (fit > (ct - 1) * kLimbN) m = fit;
+    }
+    if (m <= 0) return 0;
+    const long groups = (items + m - 1) / m, even = (items + groups - 1) / groups;
+    return std::min(m, limb_ctiles(even) * kLimbN);
+}
+
+// Local convolutions of one launch group: three launches.
+static cudaError_t limb_conv_group(const mlc_plan_s *pl, const Items &it, cudaStream_t st) {
+    NvtxRange nvtx("mlc:local_convolutions");
+    const LimbConvTables &T = *pl->limb_tabs;
+    const LimbConvGeom &g = T.g;
+    const long items = it.nitems, ct = limb_ctiles(items);
+    unsigned char *B = (unsigned char *)it.a1;
+    double *cf = (double *)(B + ct * g.b_total);
+    double *V = cf + 8 * ct * kLimbN;
+    mark(pl, 1, st);
+    FoldArgs fa{it, B, cf, g.n, (int)ct, g};
+    k_limb_fold<<<(unsigned)items, 256, (size_t)(g.n / 2 + 1) * (g.n + 1) * (g.n + 1) * sizeof(double), st>>>(fa);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    mark(pl, 2, st);
+    LimbJob job{};
+    job.nparts = 8;
+    int t0 = 0;
+    for (int c = 0; c < 8; ++c) {
+        const int u = limb_table(g.share, c);
+        job.part[c] = LimbPart{T.A + g.a_off[u], T.rf + g.rf_off[u], g.b_step[c], g.v_step[c], g.kst[u], g.rows[u], g.tiles[u], t0};
+        t0 += g.tiles[u] * (int)ct;
+    }
+    job.B = B;
+    job.cf = cf;
+    job.V = V;
+    job.cols = (int)items;
+    job.ctiles = (int)ct;
+    job.ntiles = t0;
+    job.wait_tries = 1 << 22;
+    if (pl->fault == 1) {  // test hook: the waits must run out, quickly
+        job.skip_copy = 1;
+        job.wait_tries = 64;
+    }
+    e = launch_limb_gemm(job, it, st);
+    if (e != cudaSuccess) return e;
+    mark(pl, 3, st);
+    UnfoldArgs ua{it, V, (int)items, {}, g};
+    for (int kind = 0; kind < 2; ++kind)
+        for (int ax = 0; ax < 3; ++ax)
+            for (int c = 0; c < 8; ++c) {
+                int ta = 0;
+                while (limb_perm(g.share, c, ta) != ax) ++ta;
+                ua.base[kind][ax][c] = limb_plane_base(g, limb_table(g.share, c), kind, ta);
+            }
+    const bool df = pl->g.conv == CONV_DF;
+    if (g.share) {
+        if (df) k_limb_unfold<float2, true><<<(unsigned)items, 256, 0, st>>>(ua);
+        else k_limb_unfold<double, true><<<(unsigned)items, 256, 0, st>>>(ua);
+    } else {
+        if (df) k_limb_unfold<float2, false><<<(unsigned)items, 256, 0, st>>>(ua);
+        else k_limb_unfold<double, false><<<(unsigned)items, 256, 0, st>>>(ua);
+    }
+    return cudaGetLastError();
+}
+
+cudaError_t launch_limb_conv(const mlc_plan_s *pl, const Items &it, cudaStream_t st) {
+    const long group = limb_group(pl->g, it.cap, it.nitems);
+    if (group <= 0) return cudaErrorInvalidValue;
+    for (long c0 = 0; c0 < it.nitems; c0 += group) {
+        Items ic = it;
+        ic.nitems = (int)std::min<long>(group, it.nitems - c0);
+        if (it.items) ic.items = it.items + c0;
+        else ic.first = it.first + (int)c0;
+        const cudaError_t e = limb_conv_group(pl, ic, st);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
+}  // namespace mlc

@@ -1,0 +1,280 @@
+// The exact-split matrix product of limb.h as a persistent, warp-specialised
+// tcgen05 kernel.
+//
+// A work tile is 128 table rows x 64 columns of one block.  Its seven level
+// accumulators (7 x 64 FP32 columns) fill TMEM's 512 columns, so one CTA runs
+// per SM.  Per k-step of 16 a producer thread brings the seven digits of the
+// rows and of the columns into shared memory with two bulk copies (28 + 14 KB,
+// laid out in global memory as the canonical K-major core matrices, so a copy
+// is one contiguous run), five steps deep; one thread issues the 28 MMAs of
+// digit pairs i + j < 7; after every 16 steps eight warps read the levels,
+// combine them into two 64-bit integers per output (exact) and hand the
+// accumulators back.  The FP64 conversion of a finished tile therefore runs
+// beside the next tile's MMAs.  It is kept to four operations per output, since
+// GB300 issues FP64 on two lanes per SM and cycle.
+//
+// Bound: shared-memory reads of the MMAs (M = 128, N = 64 reads 6 KB per 128 x
+// 64 x 16 products: about 48 cycles of SMEM bandwidth against 32 of tensor
+// work); a wider N does not fit seven accumulators.
+#include "limb.h"
+#include "mlc_internal.h"
+
+namespace mlc {
+namespace {
+
+constexpr int kStages = 5;
+constexpr int kStageBytes = kLimbAStep + kLimbBStep;
+constexpr int kEpiWarps = 8;
+constexpr int kThreads = (kEpiWarps + 2) * 32;
+constexpr int kSmem = kStages * kStageBytes + 1024;
+
+__device__ __forceinline__ uint32_t s32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void mb_init(uint64_t *b, unsigned count) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(s32(b)), "r"(count) : "memory");
+}
+__device__ __forceinline__ void mb_expect(uint64_t *b, unsigned bytes) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(s32(b)), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void mb_arrive(uint64_t *b) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(s32(b)) : "memory");
+}
+__device__ __forceinline__ bool mb_wait(uint64_t *b, unsigned parity, int tries) {
+    for (int i = 0; i < tries; ++i) {
+        unsigned ok;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok)
+            : "r"(s32(b)), "r"(parity)
+            : "memory");
+        if (ok) return true;
+    }
+    return false;
+}
+__device__ __forceinline__ void bulk_in(void *dst, const void *src, unsigned bytes, uint64_t *bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                     s32(dst)),
+                 "l"(src), "r"(bytes), "r"(s32(bar))
+                 : "memory");
+}
+// canonical K-major layout without swizzle: core matrices 128 bytes apart along
+// K, 256 along M / N (descriptor version 1)
+__device__ __forceinline__ uint64_t mat_desc(uint32_t addr) {
+    return (uint64_t)((addr >> 4) & 0x3FFFu) | (uint64_t)(128 >> 4) << 16 | (uint64_t)(256 >> 4) << 32 |
+           (uint64_t)1 << 46;
+}
+// kind::f16: FP32 accumulator, FP16 A and B, both K-major
+constexpr uint32_t kIdesc = (1u << 4) | ((uint32_t)(kLimbN >> 3) << 17) | ((uint32_t)(kLimbM >> 4) << 24);
+
+__device__ __forceinline__ void mma_f16(uint32_t d, uint64_t a, uint64_t b, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
+        "l"(a), "l"(b), "r"(kIdesc), "r"(accumulate)
+        : "memory");
+}
+__device__ __forceinline__ void commit(uint64_t *bar) {
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(s32(bar))
+                 : "memory");
+}
+__device__ __forceinline__ void tmem_ld16(uint32_t t, uint32_t (&r)[16]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
+        "%15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(t));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+
+__device__ __forceinline__ const LimbPart &part_of(const LimbJob &job, int t) {
+    int p = 0;
+#pragma unroll
+    for (int i = 1; i < kLimbMaxParts; ++i)
+        if (i < job.nparts && t >= job.part[i].tile0) p = i;
+    return job.part[p];
+}
+
+__global__ void __launch_bounds__(kThreads, 1) k_limb_gemm(const __grid_constant__ LimbJob job, Items it) {
+    extern __shared__ __align__(1024) unsigned char sm[];
+    __shared__ uint64_t full[kStages], empty[kStages], acc_full, acc_empty;
+    __shared__ uint32_t tmem_slot;
+    __shared__ int failed;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < kStages; ++i) {
+            mb_init(&full[i], 1);
+            mb_init(&empty[i], 1);
+        }
+        mb_init(&acc_full, 1);
+        mb_init(&acc_empty, kEpiWarps * 32);
+        failed = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(s32(&tmem_slot)),
+                     "r"(512)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem = tmem_slot;
+    const int tries = job.wait_tries;
+
+    if (warp == kEpiWarps) {  // producer
+        if (lane == 0) {
+            int step = 0;
+            bool ok = true;
+            for (int t = blockIdx.x; ok && t < job.ntiles; t += gridDim.x) {
+                const LimbPart &P = part_of(job, t);
+                const int local = t - P.tile0, rt = local / job.ctiles, ct = local - rt * job.ctiles;
+                const unsigned char *a = P.A + (long)rt * P.kst * kLimbAStep;
+                const unsigned char *b = job.B + P.b_off * job.ctiles + (long)ct * P.kst * kLimbBStep;
+                for (int k = 0; k < P.kst; ++k, ++step) {
+                    const int s = step % kStages;
+                    if (!mb_wait(&empty[s], ((step / kStages) & 1) ^ 1, tries) || atomicAdd(&failed, 0)) {
+                        ok = false;
+                        break;
+                    }
+                    mb_expect(&full[s], kStageBytes);
+                    if (!job.skip_copy) {
+                        bulk_in(sm + s * kStageBytes, a + (long)k * kLimbAStep, kLimbAStep, &full[s]);
+                        bulk_in(sm + s * kStageBytes + kLimbAStep, b + (long)k * kLimbBStep, kLimbBStep, &full[s]);
+                    }
+                }
+            }
+            if (!ok) {
+                atomicExch(&failed, 1);
+                // the copies in flight land in shared memory: wait (again bounded) for each stage last filled
+                for (int i = 0; i < kStages && i < step; ++i) {
+                    const int q = step - 1 - i;
+                    mb_wait(&full[q % kStages], (q / kStages) & 1, tries);
+                }
+            }
+        }
+    } else if (warp == kEpiWarps + 1) {  // MMA issue
+        if (lane == 0) {
+            int step = 0, chunk = 0;
+            bool ok = true;
+            for (int t = blockIdx.x; ok && t < job.ntiles; t += gridDim.x) {
+                const LimbPart &P = part_of(job, t);
+                for (int k = 0; k < P.kst; ++k, ++step) {
+                    const int s = step % kStages;
+                    const bool first = k % kLimbChunk == 0;
+                    if (first) {
+                        if (!mb_wait(&acc_empty, (chunk & 1) ^ 1, tries) || atomicAdd(&failed, 0)) {
+                            ok = false;
+                            break;
+                        }
+                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    }
+                    if (!mb_wait(&full[s], (step / kStages) & 1, tries)) {
+                        ok = false;
+                        break;
+                    }
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    const uint32_t a0 = s32(sm + s * kStageBytes), b0 = a0 + kLimbAStep;
+#pragma unroll
+                    for (int i = 0; i < kLimbs; ++i) {
+                        const uint64_t da = mat_desc(a0 + i * kLimbABlk);
+#pragma unroll
+                        for (int j = 0; i + j < kLimbLevels && j < kLimbs; ++j)
+                            mma_f16(tmem + (uint32_t)((i + j) * kLimbN), da, mat_desc(b0 + j * kLimbBBlk),
+                                    (first && i == 0) ? 0u : 1u);
+                    }
+                    commit(&empty[s]);
+                    if (k % kLimbChunk == kLimbChunk - 1 || k == P.kst - 1) {
+                        commit(&acc_full);
+                        ++chunk;
+                    }
+                }
+            }
+            if (!ok) {
+                atomicExch(&failed, 1);
+                // MMAs in flight: a commit of everything issued so far completes the stage's barrier phase
+                if (step > 0) {
+                    const int q = step - 1;
+                    mb_wait(&empty[q % kStages], (q / kStages) & 1, tries);
+                }
+            }
+        }
+    } else {  // eight warps read the accumulators: warp w has lanes 32 (w % 4).., columns 32 (w / 4)..
+        const int sub = warp & 3, half = warp >> 2;
+        const uint32_t tl = tmem + ((uint32_t)(sub * 32) << 16) + (uint32_t)(half * 32);
+        int chunk = 0;
+        bool ok = true;
+        for (int t = blockIdx.x; ok && t < job.ntiles; t += gridDim.x) {
+            const LimbPart &P = part_of(job, t);
+            const int local = t - P.tile0, rt = local / job.ctiles, ct = local - rt * job.ctiles;
+            long long hi[32], lo[32];  // sum = hi 2^32 + lo
+#pragma unroll
+            for (int j = 0; j < 32; ++j) hi[j] = lo[j] = 0;
+            for (int k = 0; k < P.kst; k += kLimbChunk, ++chunk) {
+                const bool got = mb_wait(&acc_full, chunk & 1, tries);
+                if (!__all_sync(0xffffffffu, got)) {
+                    ok = false;
+                    break;
+                }
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll
+                for (int q = 0; q < 2 * kLimbLevels; ++q) {
+                    const int l = q >> 1, j0 = (q & 1) * 16;
+                    uint32_t r[16];
+                    tmem_ld16(tl + (uint32_t)(l * kLimbN + j0), r);
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) {
+                        const long long v = __float2int_rn(__uint_as_float(r[j]));
+                        if (l < 3) hi[j0 + j] += v * (1ll << (16 - 8 * l));
+                        else lo[j0 + j] += v * (1ll << (48 - 8 * l));
+                    }
+                }
+                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                mb_arrive(&acc_empty);
+            }
+            if (!ok) break;
+            const int row = rt * kLimbM + sub * 32 + lane, c0 = ct * kLimbN + half * 32;
+            const double rf = P.rf[row];
+            const double *cf = job.cf + (long)(&P - job.part) * job.ctiles * kLimbN + c0;
+            double *v = job.V + P.v_off * job.cols + (long)c0 * P.rows + row;
+            if (row < P.rows) {
+#pragma unroll
+                for (int j = 0; j < 32; ++j)
+                    if (c0 + j < job.cols)
+                        v[(long)j * P.rows] = fma((double)hi[j], 4294967296.0, (double)lo[j]) * rf * cf[j];
+            }
+        }
+        if (!ok) {
+            atomicExch(&failed, 1);
+            if (threadIdx.x == 0)  // every plan with a column in this launch
+                for (int c = 0; c < job.cols; ++c) {
+                    const PlanPtrs &rec = it.plans[it.items ? it.items[c].x : 0];
+                    atomicExch(rec.err, 1);
+                    if (!it.items) break;
+                }
+        }
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (warp == 0)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+}
+
+}  // namespace
+
+void configure_limb() {
+    cudaFuncSetAttribute(k_limb_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+}
+
+cudaError_t launch_limb_gemm(const LimbJob &job, const Items &it, cudaStream_t st) {
+    if (job.ntiles <= 0) return cudaSuccess;
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    k_limb_gemm<<<job.ntiles < sms ? job.ntiles : sms, kThreads, kSmem, st>>>(job, it);
+    return cudaGetLastError();
+}
+
+}  // namespace mlc

@@ -10,6 +10,7 @@
 #include <vector>
 
 #include "../../include/mlc.h"
+#include "limb.h"
 
 namespace mlc {
 
@@ -97,14 +98,23 @@ struct Geom {
     bool wide;                       // Q = 10 (s = 2): a second boundary layer one node off the
                                      // face planes (fp2, resid2, phiB2 below); R18
     size_t scr_a1, scr_a4;           // scratch bytes per patch: x-transformed charges, slab outputs
+    // FP64 and double-float tiers: scratch of the exact-split products (limb.h)
+    size_t limb_tile_bytes, limb_item_bytes;  // per 64 patches: digits and factors; per patch: products
 };
 // Local-convolution scratch for `items` patches: the a1 part, then (from a
 // 256-byte boundary) the a4 part.
 inline size_t conv_scratch_a4_offset(const Geom &g, long items) {
     return ((size_t)items * g.scr_a1 + 255) & ~(size_t)255;
 }
+// The exact-split products of the FP64 and double-float tiers take less than
+// transforms would (118 KB against 954 KB per patch of 16^3, s = 16), so a
+// scratch of that size holds more patches than conv_chunk at once; only a few
+// patches, whose columns fill a tile of 64, can need more.
 inline size_t conv_scratch_bytes(const Geom &g, long items) {
-    return conv_scratch_a4_offset(g, items) + (size_t)items * g.scr_a4;
+    const size_t fft = conv_scratch_a4_offset(g, items) + (size_t)items * g.scr_a4;
+    if (g.conv == CONV_F32) return fft;
+    const size_t limb = (size_t)limb_ctiles(items) * g.limb_tile_bytes + (size_t)items * g.limb_item_bytes;
+    return limb > fft ? limb : fft;
 }
 
 // Per-plan pointers and sizes read by the per-patch kernels.  A single solve
@@ -114,7 +124,7 @@ inline size_t conv_scratch_bytes(const Geom &g, long items) {
 struct PlanPtrs {
     const void *f;        // charge, N^3 (FP64 or FP32 by tier)
     void *cl, *fp;        // local fields on the coarse lattice / alpha face planes
-    const void *khat;     // patch kernel spectrum octant (working precision)
+    const void *khat;     // split tiers: patch kernel spectrum octant (FP32)
     const void *momw;     // 1D moment weights a_k(m) = w_m q_k(2m/n - 1), P x (n+1), FP64
     double mom_scale;     // R^{-3/2}
     double *mom;
@@ -126,6 +136,7 @@ struct PlanPtrs {
     const void *lam;      // Dirichlet inverse eigenvalues (2/n)^3 h^2 / lambda (FP64 or double-float)
     int N, np;
     double c2h2, inv_h2;  // h^2 / 12, 1 / h^2
+    double h2;            // h^2
     void *dscr;           // Dirichlet workspace (n > 24): [patch][(n-1)^3] in the fine precision
     int *err;             // the plan's error word
     // Q = 10 (R18): local fields and residuals on the planes one node off the
@@ -148,7 +159,23 @@ struct Items {
     int chunk = 0;        // items per local-convolution launch group (0: the plan's conv_chunk)
     void *a1 = nullptr;   // scratch: x-transformed charges, scr_a1 bytes per item
     void *a4 = nullptr;   // scratch: slab outputs, scr_a4 bytes per item
+    size_t cap = 0;       // scratch bytes from a1 on (FP64 and double-float tiers)
 };
+
+#ifdef __CUDACC__
+// Plan record and local patch index of a work item.
+// Item `item` of a launch covers patch p of its plan; the item index itself
+// is the slot of the item in the launch's local-convolution scratch.
+__device__ __forceinline__ const PlanPtrs &item_plan(const Items &it, int item, int &p) {
+    if (it.items) {
+        const int2 v = it.items[item];
+        p = v.y;
+        return it.plans[v.x];
+    }
+    p = item + it.first;
+    return it.plans[0];
+}
+#endif
 
 }  // namespace mlc
 
@@ -164,20 +191,18 @@ struct mlc_plan_s {
     // tables (device)
     const double *dgf;       // shared octant table (L_dgf+1)^3, owned by the device cache
     int dgf_L;
-    double *khat;            // patch kernel spectrum octant (Mh^3), scaled by h^2/M^3
+    double *khat;            // split tiers: patch kernel spectrum octant (Mh^3), scaled by h^2/M^3
     double *khat_c;          // coarse kernel spectrum octant (Mhc^3), scaled by H^2/Mc^3
     double *momw;            // P x nb 1D moment weights (Boole weight x orthonormal Legendre)
     // Legendre ring tables: D [axis][plane][u][v][npad] (dense over the beta
     // box face planes, zero rows off the ring), T [coarse cell][npoly], in the
     // ring precision of the tier (FP32 split tiers, double-float pairs, FP64)
     void *Dtab, *Ttab;
-    double2 *tw, *tw_c;      // FFT twiddles exp(-2 pi i t / M), t < M/2 (FP64 tier)
+    double2 *tw_c;           // coarse FFT twiddles exp(-2 pi i t / Mc), t < Mc/2 (FP64)
     float *khat_f;           // split tiers: FP32 copies of the patch spectrum and twiddles
     float2 *tw_f;
     float2 *khat_c_df;       // coarse spectrum and twiddles as double-float (hi, lo) pairs
     float4 *tw_c_df;
-    float2 *khat_df;         // double-float tier: patch spectrum and twiddles as double-float pairs
-    float4 *tw_df;
     void *sinm;              // (n-1) x n/2 half DST-I matrix sin(pi k t / n), fine precision
     void *lam;               // (n-1)^3 (2/n)^3 h^2 / stencil eigenvalue, fine precision
     // workspace (device)
@@ -206,6 +231,7 @@ struct mlc_plan_s {
     double *tpl2 = nullptr;    // 3 (np+1) 2 no (N+1): I^H(phi^H) on those planes summed along v
     void *D2tab = nullptr;     // [axis][npb][2][wbx][wbx][npad] ring rows of the off-face nodes
     void *f_stage, *phi_stage;  // device staging for mlc_solve_host
+    std::shared_ptr<mlc::LimbConvTables> limb_tabs;  // FP64 and double-float tiers: folded Green's function
     int *err;                // device error word: nonzero if a bounded wait in a kernel gave up
     size_t ws_bytes;
     std::vector<void *> owned;  // device allocations to free
@@ -250,6 +276,8 @@ inline void mark(const mlc_plan_s *pl, int k, cudaStream_t st);
 // plans with the geometry of `pl`).
 cudaError_t launch_moments(const mlc_plan_s *pl, const Items &it, cudaStream_t st);
 cudaError_t launch_patch_conv(const mlc_plan_s *pl, const Items &it, cudaStream_t st);
+// limb_conv.cu: the local convolutions of the FP64 and double-float tiers
+cudaError_t launch_limb_conv(const mlc_plan_s *pl, const Items &it, cudaStream_t st);
 cudaError_t launch_resid(const mlc_plan_s *pl, const Items &it, cudaStream_t st);
 cudaError_t launch_dirichlet(const mlc_plan_s *pl, const Items &it, cudaStream_t st);
 cudaError_t launch_assemble(const mlc_plan_s *pl, cudaStream_t st);
@@ -330,6 +358,7 @@ struct BatchLayout {
         int item0, nitems;      // the group's range of the item table
         void *a1 = nullptr, *a4 = nullptr;  // the group's local-convolution scratch
                                             // (min(chunk, nitems) patches; set by the owner)
+        size_t cap = 0;                     // its bytes
     };
     std::vector<int> order, plan_group;
     std::vector<Group> groups;

@@ -78,6 +78,7 @@ extern "C" mlc_status mlc_solve_noalloc(mlc_plan_t pl, const void *f, void *phi,
     Items it{nullptr, addr.record, pl->g.NP};
     it.a1 = addr.scratch;
     it.a4 = addr.scratch + conv_scratch_a4_offset(pl->g, items);
+    it.cap = kNoAllocScratchBytes;
     if (launch_moments(pl, it, st) != cudaSuccess) return MLC_ERR_CUDA;
     if (launch_patch_conv(pl, it, st) != cudaSuccess) return MLC_ERR_CUDA;
     if (launch_resid(pl, it, st) != cudaSuccess) return MLC_ERR_CUDA;

@@ -268,7 +268,17 @@ mlc_status derive_geometry(const mlc_params &pp, Geom &g) {
         g.scr_a4 = (size_t)g.nzr * g.a4blk * cb;
         g.chunk = pp.conv_chunk > 0 ? pp.conv_chunk : 1024;
     }
+    // face planes of the patch lattice inside Omega_alpha (relative x = pl0 + j n)
+    g.pl0 = g.n * ceildiv(-g.ga, g.n);
+    g.npa = 0;
+    for (int c = g.pl0; c <= g.n + g.ga; c += g.n) ++g.npa;
     g.wa = g.n + 2 * g.ga + 1;
+    if (g.conv != CONV_F32) {
+        LimbConvGeom lc;
+        if (!limb_conv_geometry(g, true, lc)) return MLC_ERR_UNSUPPORTED;
+        g.limb_tile_bytes = (size_t)lc.b_total + 8 * kLimbN * sizeof(double);
+        g.limb_item_bytes = (size_t)lc.v_total * sizeof(double);
+    }
     g.wbx = g.n + 2 * g.gb + 1;
     g.plane_n = (g.N + 1) * (g.N + 1);
     g.n_planes_total = 3L * (g.np + 1) * (long)g.plane_n;
@@ -313,10 +323,6 @@ mlc_status build_tables(mlc_plan_s *pl) {
         for (int m = 0; m < nb; ++m) a1d[(size_t)k * nb + m] = bw[m] * leg[(size_t)k * nb + m];
     TRY(dev_upload(pl, &pl->momw, a1d));
 
-    // face planes of the patch lattice inside Omega_alpha (relative x = pl0 + j n)
-    g.pl0 = g.n * ceildiv(-g.ga, g.n);
-    g.npa = 0;
-    for (int c = g.pl0; c <= n + g.ga; c += n) ++g.npa;
     // every interpolation stencil of a face node of Omega_alpha stays in the field box
     if (4 * (-g.ga / 4 - g.b) < -g.s || 4 * ((n + g.ga) / 4 + g.b) > n + g.s) return MLC_ERR_INVALID_ARG;
     (void)W;
@@ -568,7 +574,6 @@ mlc_status build_tables(mlc_plan_s *pl) {
         }
         return tw;
     };
-    TRY(dev_upload(pl, &pl->tw, twiddles(g.M)));
     if (g.levels <= 2) TRY(dev_upload(pl, &pl->tw_c, twiddles(g.Mc)));  // coarse Hockney solve
 
     // Dirichlet tables: half DST-I matrix and eigenvalues of the stencil / h^2
@@ -740,10 +745,14 @@ mlc_status create_plan(const mlc_params *params, const double *dgf_host, int dgf
         st = get_dgf(pl->device, G.Q, G.nD, G.zeta, Lneed, &pl->dgf, &pl->dgf_L);
     }
     if (st == MLC_OK) st = build_tables(pl);
+    if (st == MLC_OK && G.conv != CONV_F32)
+        st = to_status(limb_conv_tables(pl->device, G, dgf_host == nullptr, pl->dgf, pl->dgf_L, &pl->limb_tabs));
     auto alloc_all = [&]() -> mlc_status {
-        TRY(dev_alloc(pl, &pl->khat, (size_t)G.Mh * G.Mh * G.Mh, false));
-        TRY_CUDA(build_even_spectrum(pl->dgf, pl->dgf_L, G.M, std::min(G.n + G.s, G.M / 2),
-                                     G.h * G.h / ((double)G.M * G.M * G.M), pl->khat));
+        if (G.conv == CONV_F32) {
+            TRY(dev_alloc(pl, &pl->khat, (size_t)G.Mh * G.Mh * G.Mh, false));
+            TRY_CUDA(build_even_spectrum(pl->dgf, pl->dgf_L, G.M, std::min(G.n + G.s, G.M / 2),
+                                         G.h * G.h / ((double)G.M * G.M * G.M), pl->khat));
+        }
         const bool hockney = G.levels <= 2;  // this plan runs the coarse Hockney solve itself
         if (hockney) {
             TRY(dev_alloc(pl, &pl->khat_c, (size_t)G.Mhc * G.Mhc * G.Mhc, false));
@@ -779,26 +788,6 @@ mlc_status create_plan(const mlc_params *params, const double *dgf_host, int dgf
         TRY(dev_alloc(pl, &bf, NP * 3 * (size_t)G.npa * G.wa * G.wa * rb));
         pl->cl = bc;
         pl->fpl = bf;
-        if (G.conv == CONV_DF) {
-            // double-float copies of the patch kernel spectrum and twiddles
-            auto split = [](double v) {
-                const float h = (float)v;
-                return make_float2(h, (float)(v - (double)h));
-            };
-            const size_t nk = (size_t)G.Mh * G.Mh * G.Mh;
-            std::vector<double> kd(nk);
-            TRY_CUDA(cudaMemcpy(kd.data(), pl->khat, nk * sizeof(double), cudaMemcpyDeviceToHost));
-            std::vector<float2> kf(nk);
-            for (size_t i = 0; i < nk; ++i) kf[i] = split(kd[i]);
-            TRY(dev_upload(pl, &pl->khat_df, kf));
-            std::vector<float4> tf(G.M / 2);
-            for (int t = 0; t < G.M / 2; ++t) {
-                const double a = 2.0 * M_PI * (double)t / (double)G.M;
-                const float2 re = split(std::cos(a)), im = split(-std::sin(a));
-                tf[t] = make_float4(re.x, re.y, im.x, im.y);
-            }
-            TRY(dev_upload(pl, &pl->tw_df, tf));
-        }
         if (G.conv == CONV_F32) {
             // FP32 copies of the patch kernel spectrum and twiddles
             const size_t nk = (size_t)G.Mh * G.Mh * G.Mh;
@@ -857,8 +846,7 @@ mlc_status create_plan(const mlc_params *params, const double *dgf_host, int dgf
         h.phi = nullptr;
         h.cl = pl->cl;
         h.fp = pl->fpl;
-        h.khat = G.conv == CONV_F32 ? (const void *)pl->khat_f
-                 : (G.conv == CONV_DF ? (const void *)pl->khat_df : (const void *)pl->khat);
+        h.khat = pl->khat_f;
         h.momw = pl->momw;
         h.mom_scale = std::pow(G.R, -1.5);
         h.mom = pl->mom;
@@ -871,6 +859,7 @@ mlc_status create_plan(const mlc_params *params, const double *dgf_host, int dgf
         h.np = G.np;
         h.c2h2 = correction ? stencil_c2(G.Q) * G.h * G.h : 0.0;
         h.inv_h2 = 1.0 / (G.h * G.h);
+        h.h2 = G.h * G.h;
         h.err = pl->err;
         h.dscr = pl->dscr;
         h.fp2 = pl->fp2;
@@ -1012,6 +1001,7 @@ mlc_status mlc_solve(mlc_plan_t pl, const void *f, void *phi, void *stream) {
     Items it{nullptr, pl->dptrs, pl->g.NP};
     it.a1 = scr;
     it.a4 = (char *)scr + conv_scratch_a4_offset(pl->g, std::min<long>(pl->g.chunk, pl->g.NP));
+    it.cap = conv_scratch_bytes(pl->g, std::min<long>(pl->g.chunk, pl->g.NP));
     if (!pl->timing) {
         // Two streams: the moments (they read only f) and, once the local
         // fields exist, the face-plane residuals run on a side stream beside

@@ -298,6 +298,7 @@ cudaError_t mlc_server_s::launch(Lane &ln) {
         }
         L.groups[g].a1 = ln.scratch[g];
         L.groups[g].a4 = (char *)ln.scratch[g] + conv_scratch_a4_offset(G, nit);
+        L.groups[g].cap = need;
     }
     return batch_enqueue(ln.plans, L, ln.d_items, ln.d_recs, ln.S, std::min(4, count), 0, ln.st);
 }

@@ -1,0 +1,154 @@
+"""The exact-split tensor-core convolutions of the FP64 and double-float tiers
+(limb.h) at the edges of their tiles, classes and scales: the local fields at
+the coarse points of the field box against direct sums in extended precision.
+
+Bound.  With charges |f| <= F on nb^3 nodes and |G| <= g, each folded entry is
+at most 8 F and each table entry at most g; both are rounded to 2^-55 of their
+block's largest magnitude and the digit pairs left out weigh at most 7 * 2^-56,
+so the sum over at most nb^3 terms is off by at most nb^3 * 8 F g * (2 * 2^-55 +
+7 * 2^-56) < 46 nb^3 F g 2^-54; FP64 roundings of the fold, the table and the
+unfolding add less than 16 nb^3 F g 2^-53.  Both together stay below
+80 nb^3 F g 2^-54 (about 1e-14 of a field of one sign).  A double-float result
+adds 2^-47 of itself."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def torch_cuda():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    return torch
+
+
+def _plan(torch, N, n, s, Q, tier, **kw):
+    from paper_1702_08111_gb300 import mlc
+    return mlc.Plan(N, n, s, 4, Q, tier=tier, **kw)
+
+
+def _reference(G, f, N, n, s, i, ks):
+    """h^2 sum_m G[|4 k - m|] chi(m) f[n i + m] at the lattice points k of patch i, in long double."""
+    np_ = N // n
+    o = np.array([i // (np_ * np_), (i // np_) % np_, i % np_]) * n
+    fp = np.zeros((n + 1,) * 3, dtype=np.longdouble)
+    hi = [min(n + 1, N - o[d]) for d in range(3)]
+    fp[:hi[0], :hi[1], :hi[2]] = f[o[0]:o[0] + hi[0], o[1]:o[1] + hi[1], o[2]:o[2] + hi[2]]
+    w = np.ones(n + 1)
+    w[0] = w[n] = 0.5
+    fp *= (w[:, None, None] * w[:, None] * w)
+    m = np.arange(n + 1)
+    out = []
+    for k in ks:
+        a, b, c = (np.abs(4 * kk - s - m) for kk in k)
+        out.append(np.sum(G[np.ix_(a, b, c)].astype(np.longdouble) * fp))
+    return np.array(out) / N ** 2
+
+
+def _check(plan, f, N, n, s, tier, patches, seed, G=None):
+    from paper_1702_08111_gb300 import mlc
+    if G is None:
+        G = plan.export(mlc.STAGE_DGF)
+    got = plan.export(mlc.STAGE_COARSE_SAMPLES)
+    nc = got.shape[1]
+    rng = np.random.default_rng(seed)
+    ks = [(0, 0, 0), (nc - 1, nc - 1, nc - 1), (0, nc - 1, nc // 2)] + [tuple(rng.integers(0, nc, 3)) for _ in range(5)]
+    lim = np.abs(G[:n + s + 1, :n + s + 1, :n + s + 1]).max()
+    for i in patches:
+        ref = _reference(G, f, N, n, s, i, ks)
+        v = np.array([got[(i,) + k] for k in ks])
+        tol = 80 * (n + 1) ** 3 * np.abs(f).max() * lim * 2.0 ** -54 / N ** 2
+        if tier == mlc.MLC_TIER_DF:
+            tol = tol + 2.0 ** -47 * np.abs(v)
+        assert np.all(np.abs((v - ref).astype(np.float64)) <= tol), (i, np.abs((v - ref).astype(np.float64)).max(), tol)
+
+
+@pytest.mark.parametrize("N,n,s,Q,kw", [
+    (4, 4, 8, 4, {}),              # one patch: one column of a tile of 64
+    (8, 4, 12, 4, {}),             # n/2 not a multiple of 4: no centre on the lattice
+    (20, 4, 20, 6, {"mode": 1}),   # 125 patches: two column tiles, the second ragged
+    (32, 8, 8, 4, {}),             # 64 patches: one full tile; inner box = patch
+    (40, 8, 16, 10, {}),           # the planes next to the face planes
+    (36, 12, 20, 6, {}),
+    (32, 16, 16, 6, {}),           # K = 729: three reads of the accumulators
+    (48, 24, 20, 4, {}),
+    (32, 32, 28, 6, {}),           # K = 4913, the longest sums
+    (64, 32, 12, 6, {"mode": 1}),
+])
+@pytest.mark.parametrize("tier", [0, 2])
+def test_local_fields_against_long_double(torch_cuda, N, n, s, Q, kw, tier):
+    torch = torch_cuda
+    if Q == 10 and tier == 2:
+        pytest.skip("Q = 10 has no double-float tier")
+    plan = _plan(torch, N, n, s, Q, tier, **kw)
+    rng = np.random.default_rng(N + n + s)
+    f = rng.uniform(-1, 1, (N,) * 3) + 0.3
+    plan.solve(torch.from_numpy(f).cuda())
+    NP = (N // n) ** 3
+    _check(plan, f, N, n, s, tier, sorted({0, NP // 2, NP - 1}), 7)
+
+
+@pytest.mark.parametrize("scale", [2.0 ** -400, 2.0 ** 300])
+def test_scales_and_empty_patches(torch_cuda, scale):
+    """Each patch has its own scale: huge and tiny charges side by side, and patches without charge."""
+    torch = torch_cuda
+    N, n, s = 32, 8, 12
+    plan = _plan(torch, N, n, s, 4, 0)
+    rng = np.random.default_rng(3)
+    f = np.zeros((N,) * 3)
+    f[1:8, 1:8, 1:8] = rng.uniform(-1, 1, (7,) * 3)                # patch 0
+    f[25:32, 25:32, 25:32] = rng.uniform(-1, 1, (7,) * 3) * scale  # patch 63
+    plan.solve(torch.from_numpy(f).cuda())
+    g = f.copy()
+    g[:16] = 0.0
+    _check(plan, f[:, :, :] * (np.abs(f) <= 1.0 if scale > 1 else 1.0), N, n, s, 0, [0], 1)
+    _check(plan, g, N, n, s, 0, [63], 1)
+    from paper_1702_08111_gb300 import mlc
+    assert np.all(plan.export(mlc.STAGE_COARSE_SAMPLES)[30] == 0.0)
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf, -np.inf])
+def test_not_finite_charge_stays_in_its_patches(torch_cuda, bad):
+    torch = torch_cuda
+    from paper_1702_08111_gb300 import mlc
+    N, n, s = 32, 8, 8
+    plan = _plan(torch, N, n, s, 4, 0)
+    f = np.random.default_rng(5).uniform(-1, 1, (N,) * 3)
+    f[4, 4, 4] = bad
+    phi = plan.solve(torch.from_numpy(f).cuda())
+    got = plan.export(mlc.STAGE_COARSE_SAMPLES)
+    assert not np.isfinite(got[0]).any() and np.isfinite(got[1:]).all()
+    assert not torch.isfinite(phi).any()
+
+
+def test_caller_table_without_axis_symmetry(torch_cuda):
+    """A caller's Green's function need not be the same along the axes; plans with it keep tables of
+    their own, also inside one batch."""
+    torch = torch_cuda
+    from paper_1702_08111_gb300 import mlc
+    N, n, s = 32, 8, 12
+    plan, other = _plan(torch, N, n, s, 4, 0), _plan(torch, N, n, s, 4, 0)
+    G = plan.export(mlc.STAGE_DGF)
+    L = G.shape[0] - 1
+    x = np.arange(L + 1)
+    T = G * (1.0 + 1e-3 * x[:, None, None] / L - 2e-3 * x[:, None] / L)
+    plan.set_dgf(T)
+    f = torch.from_numpy(np.random.default_rng(11).uniform(-1, 1, (N,) * 3)).cuda()
+    a, b = plan.solve(f).clone(), other.solve(f).clone()
+    _check(plan, f.cpu().numpy(), N, n, s, 0, [0, 21, 63], 2, G=T)
+    _check(other, f.cpu().numpy(), N, n, s, 0, [0, 21, 63], 2, G=G)
+    p, q = torch.empty_like(a), torch.empty_like(a)
+    mlc.batch_solve([plan, other], [f, f], [p, q])
+    assert torch.equal(p, a) and torch.equal(q, b)
+
+
+def test_results_do_not_depend_on_the_launch_groups(torch_cuda):
+    """conv_chunk bounds the scratch; 125 patches in one group or in several have the same bits."""
+    torch = torch_cuda
+    N, n, s = 40, 8, 12
+    f = torch.from_numpy(np.random.default_rng(2).uniform(-1, 1, (N,) * 3)).cuda()
+    ref = _plan(torch, N, n, s, 4, 0).solve(f)
+    for chunk in (1, 7, 64, 100):
+        assert torch.equal(_plan(torch, N, n, s, 4, 0, conv_chunk=chunk).solve(f), ref)
