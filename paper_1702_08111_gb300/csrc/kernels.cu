@@ -1721,6 +1721,7 @@ struct AsmArgs {
     double coefd[4];  // the same in FP64
     int wide;         // Q = 10: the 5 x 5 x 5 operator (stencil_coef), FP64 tiers only
     double invH2;     // 1 / H^2
+    RingView ring;    // LIMB: the ring terms (limb_ring.cu)
 };
 
 // Patches i (ascending linear index) whose coarse box C(Omega_beta(i)) holds
@@ -1750,7 +1751,9 @@ __device__ __forceinline__ void coarse_node_patches(const int k[3], int n, int n
 // F^H[k] = sum over patches i (ascending) of Delta^H phi^{i,h} on C(Omega_alpha(i))
 // or sum_p c_p^i Delta^H(G^h * Q^p) on C(Omega_beta(i)) \ C(Omega_alpha(i)).
 // TB: local-field storage, RT: ring tables, T: accumulation (FP64 or double-float).
-template <typename TB, typename RT, typename T>
+// LIMB: the ring sum comes from the ring products, and only the patches whose
+// C(Omega_alpha) holds k are visited.
+template <typename TB, typename RT, typename T, bool LIMB = false>
 __global__ void __launch_bounds__(128) k_assemble(AsmArgs a) {
     const long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
     const long tot = (long)a.nf * a.nf * a.nf;
@@ -1762,7 +1765,11 @@ __global__ void __launch_bounds__(128) k_assemble(AsmArgs a) {
     const int ncb = a.cb_hi - a.cb_lo + 1;
     const long nc = a.nc, kl = -a.s / 4;
     T acc = FT<T>::zero();
-    coarse_node_patches(k, a.n, a.np, a.ca_lo, a.ca_hi, a.cb_lo, a.cb_hi,
+    if (LIMB) {
+        const int q = a.n / 4, i0 = floordiv(k[0], q), i1 = floordiv(k[1], q), i2 = floordiv(k[2], q);
+        acc = FT<T>::of(a.ring.at(3, i0, i1, i2, q * q * q, ((k[0] - q * i0) * q + k[1] - q * i1) * q + k[2] - q * i2));
+    }
+    coarse_node_patches(k, a.n, a.np, a.ca_lo, a.ca_hi, LIMB ? a.ca_lo : a.cb_lo, LIMB ? a.ca_hi : a.cb_hi,
                         [&](long p, int r0, int r1, int r2, bool inA) {
                 if (inA && a.wide) {
                     const TB *bx = (const TB *)a.cl + p * nc * nc * nc;
@@ -1792,7 +1799,7 @@ __global__ void __launch_bounds__(128) k_assemble(AsmArgs a) {
                                 if (in_range(x0, nc, a.err) & in_range(x1, nc, a.err) & in_range(x2, nc, a.err))
                                     acc = FT<T>::fma(pick<T>(a.coef[nz], a.coefd[nz]), FT<T>::of(bx[(x0 * nc + x1) * nc + x2]), acc);
                             }
-                } else {
+                } else if (!LIMB) {
                     const long t = (((long)(r0 - a.cb_lo) * ncb + (r1 - a.cb_lo)) * ncb +
                                     (r2 - a.cb_lo)) * a.npoly;
                     if (in_range(r0 - a.cb_lo, ncb, a.err) & in_range(r1 - a.cb_lo, ncb, a.err) &
@@ -1897,6 +1904,7 @@ struct BndArgs {
     long ring_rows_pad;
     long idx0, idx1;           // face-plane nodes of this launch: [idx0, idx1)
     const void *mom, *D;       // ring tables in the ring precision RT
+    RingView view;             // RING = 2: the ring terms (limb_ring.cu)
     void *phiB;                // fine precision T
     int N, n, np, ga, gb, b, npoly, olo, no, wa, wbx, npa, pl0;
     int pb0, npb;     // face planes of Omega_beta (relative): pb0 + j n, j < npb
@@ -1908,9 +1916,11 @@ struct BndArgs {
 // phi^B at every face-plane node (axis, plane j, u, v).  RT: precision of the
 // Legendre ring sums (the local-convolution precision: FP32, double-float or
 // FP64); T: the interpolation and the accumulation (FP64 or double-float).
-// RING: the ring terms come from the ring GEMM (ringR) instead of per-node
-// dot products of the ring-table rows with the coefficients.
-template <typename RT, int NN, typename T, bool RING = false>
+// RING: 0, per-node dot products of the ring-table rows with the coefficients;
+// 1, the ring terms of each patch come from the ring GEMM (ringR); 2, their sum
+// comes from the ring products (view), and only the patches whose Omega_alpha
+// holds the node are visited.
+template <typename RT, int NN, typename T, int RING = 0>
 __global__ void __launch_bounds__(128, 6) k_boundary(BndArgs a) {
     constexpr int n = NN;  // patch size as a constant: the index divisions become multiplies
     const long idx = a.idx0 + (long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -1946,7 +1956,13 @@ __global__ void __launch_bounds__(128, 6) k_boundary(BndArgs a) {
     // local corrections of the patches whose Omega_beta holds g (ascending index);
     // the Legendre ring terms accumulate in the ring precision RT
     RT ring(0.0);
-    face_node_patches<NN>(g, a.np, a.ga, a.gb, [&](long p, int r0, int r1, int r2, bool inA) {
+    if constexpr (RING == 2) {
+        // a node on several planes takes the term of its first axis, so that it keeps one value
+        const int d = g[0] % n == 0 ? 0 : (g[1] % n == 0 ? 1 : 2);
+        const int u = d == 0 ? g[1] : g[0], v = d == 2 ? g[1] : g[2];
+        acc = acc + FT<T>::of(a.view.at(d, g[0] / n, g[1] / n, g[2] / n, n * n, (u % n) * n + v % n));
+    }
+    face_node_patches<NN>(g, a.np, a.ga, RING == 2 ? a.ga : a.gb, [&](long p, int r0, int r1, int r2, bool inA) {
                 if (inA) {
                     // the residual plane holding r: first axis on a face plane
                     int d, uu, vv;
@@ -1958,13 +1974,13 @@ __global__ void __launch_bounds__(128, 6) k_boundary(BndArgs a) {
                     if (in_range((rr - a.pl0) / n, a.npa, a.err) & in_range(uu + a.ga, a.wa, a.err) &
                         in_range(vv + a.ga, a.wa, a.err))
                         acc = acc + resid[((p * 3 * a.npa + slot) * a.wa + (uu + a.ga)) * a.wa + (vv + a.ga)];
-                } else {
+                } else if constexpr (RING != 2) {
                     // dense ring row of (axis, plane, u, v): no index map to read
                     const int ra = axis == 0 ? r0 : (axis == 1 ? r1 : r2);
                     const int ru = axis == 0 ? r1 : r0, rv = axis == 2 ? r1 : r2;
                     const bool ok = in_range((ra - a.pb0) / n, a.npb, a.err) & in_range(ru + a.gb, a.wbx, a.err) &
                                     in_range(rv + a.gb, a.wbx, a.err);
-                    if constexpr (RING) {
+                    if constexpr (RING == 1) {
                         const long row = ((long)((ra - a.pb0) / n) * a.wbx + (ru + a.gb)) * a.wbx + (rv + a.gb);
                         if (ok) ring += a.ringR[p * a.ring_rows_pad + row];
                     } else {
@@ -3057,6 +3073,11 @@ cudaError_t launch_assemble(const mlc_plan_s *pl, cudaStream_t st) {
     NvtxRange nvtx("mlc:coarse_charge");
     const Geom &g = pl->g;
     AsmArgs a{};
+    if (pl->limb_ring) {  // the ring terms of F^H and phi^B
+        const cudaError_t e = launch_limb_ring(pl, st);
+        if (e != cudaSuccess) return e;
+        a.ring = limb_ring_view(*pl->limb_ring);
+    }
     a.err = pl->err;
     a.cl = pl->cl; a.FH = pl->FH;
     a.mom = ring_moments(pl);
@@ -3077,9 +3098,11 @@ cudaError_t launch_assemble(const mlc_plan_s *pl, cudaStream_t st) {
         if (g.fine == FINE_F64) k_assemble<float, float, double><<<nbk, 128, 0, st>>>(a);
         else k_assemble<float, float, dfl><<<nbk, 128, 0, st>>>(a);
     } else if (g.conv == CONV_DF) {
-        k_assemble<dfl, dfl, dfl><<<nbk, 128, 0, st>>>(a);
+        if (pl->limb_ring) k_assemble<dfl, dfl, dfl, true><<<nbk, 128, 0, st>>>(a);
+        else k_assemble<dfl, dfl, dfl><<<nbk, 128, 0, st>>>(a);
     } else {
-        k_assemble<double, double, double><<<nbk, 128, 0, st>>>(a);
+        if (pl->limb_ring) k_assemble<double, double, double, true><<<nbk, 128, 0, st>>>(a);
+        else k_assemble<double, double, double><<<nbk, 128, 0, st>>>(a);
     }
     return cudaGetLastError();
 }
@@ -3175,6 +3198,8 @@ cudaError_t launch_boundary(const mlc_plan_s *pl, cudaStream_t st) {
     const long per_axis = (long)(g.np + 1) * g.plane_n;
     // split tiers with a Legendre ring: one ring GEMM and one boundary launch
     // per face-plane axis (the GEMM's output holds one axis at a time)
+    const bool limb = pl->limb_ring != nullptr;
+    if (limb) a.view = limb_ring_view(*pl->limb_ring);
     const bool gemm = g.conv == CONV_F32 && pl->ring_R != nullptr && pl->ring_aimg != nullptr;
     for (int axis = 0; axis < 3; ++axis) {
         if (!gemm && axis > 0) break;
@@ -3187,8 +3212,10 @@ cudaError_t launch_boundary(const mlc_plan_s *pl, cudaStream_t st) {
         const unsigned nbk = (unsigned)((a.idx1 - a.idx0 + 127) / 128);
 #define MLC_BND(NN)                                                                                        \
         case NN:                                                                                           \
-            if (gemm && g.fine == FINE_F64) k_boundary<float, NN, double, true><<<nbk, 128, 0, st>>>(a);   \
-            else if (gemm) k_boundary<float, NN, dfl, true><<<nbk, 128, 0, st>>>(a);                        \
+            if (limb && g.conv == CONV_DF) k_boundary<dfl, NN, dfl, 2><<<nbk, 128, 0, st>>>(a);             \
+            else if (limb) k_boundary<double, NN, double, 2><<<nbk, 128, 0, st>>>(a);                       \
+            else if (gemm && g.fine == FINE_F64) k_boundary<float, NN, double, 1><<<nbk, 128, 0, st>>>(a);  \
+            else if (gemm) k_boundary<float, NN, dfl, 1><<<nbk, 128, 0, st>>>(a);                           \
             else if (g.conv == CONV_F32 && g.fine == FINE_F64) k_boundary<float, NN, double><<<nbk, 128, 0, st>>>(a); \
             else if (g.conv == CONV_F32) k_boundary<float, NN, dfl><<<nbk, 128, 0, st>>>(a);                 \
             else if (g.conv == CONV_DF) k_boundary<dfl, NN, dfl><<<nbk, 128, 0, st>>>(a);                    \

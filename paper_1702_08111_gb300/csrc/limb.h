@@ -14,10 +14,12 @@
 // of the many steps of an FP64 transform.
 #pragma once
 
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
 #include <memory>
+#include <vector>
 
 namespace mlc {
 
@@ -30,27 +32,36 @@ constexpr int kLimbABlk = kLimbM * 16 * 2;   // bytes of one digit of a (tile, k
 constexpr int kLimbBBlk = kLimbN * 16 * 2;   // the same of the columns
 constexpr int kLimbAStep = kLimbs * kLimbABlk;
 constexpr int kLimbBStep = kLimbs * kLimbBBlk;
-constexpr int kLimbMaxParts = 8;
+constexpr int kLimbMaxParts = 32;
 
 // One block of a block-diagonal product: rows x K of the table by K x columns.
 struct LimbPart {
-    const unsigned char *A;  // digits: [row tile][k-step][digit][canonical core matrices]
+    const unsigned char *A;  // digits: [row tile][k-step][digit][k half][row][8 k]
+    long a_tile;             // bytes between row tiles
     const double *rf;        // row factors 2^(e_row - 62) (rows padded to the tile)
-    long b_off;              // bytes, per column tile, before this part in the column image
-    long v_off;              // rows of the parts before this one
+    const int *koff;         // shifted columns: per 8 k, the first column's place in the digit arrays
+    long b_off;              // contiguous columns: byte offset of the part in the column image
+    long v_off, cf_off;      // first element of the part in V and cf
     int kst;                 // k-steps of 16
-    int rows, tiles;         // rows and row tiles
-    int tile0;               // first work tile of this part (tiles x column tiles each)
+    int rows;                // rows (columns of V are this long)
+    int cols, ctiles;        // columns and column tiles
+    int tile0;               // first work tile (row tiles x column tiles each)
 };
 
-// V[part][column][row] = rf[row] cf[part][column] sum_k A[row][k] B[k][column].
+// V[part][column][row] = rf[row] cf[column] sum_k A[row][k] B[k][column].
+// Columns come in one of two forms.  Contiguous (koff null): an image
+// [column tile][k-step][digit][k half][column][8 k] per part.  Shifted: arrays
+// [digit][...][place][8 k] shared by all parts, where column c of k-group q is
+// the place koff[q] + c, so that columns which read the same numbers at
+// different offsets (the patches around a patch) need no copies of them.
 struct LimbJob {
     LimbPart part[kLimbMaxParts];
     int nparts;
-    const unsigned char *B;  // digits of the columns: [part][column tile][k-step][digit][...]
-    const double *cf;        // column factors, [part][cols_pad]
-    double *V;               // [part][column][row of the part]
-    int cols, ctiles;        // columns and column tiles
+    const unsigned char *B;
+    long b_digit;            // shifted columns: bytes between digits
+    const double *cf;        // column factors
+    int cf_step;             // 1, or 0: one factor for all columns
+    double *V;
     int ntiles;              // work tiles of all parts
     int wait_tries;          // limit of the bounded waits
     int skip_copy;           // test hook: issue no copies, so the bounded waits run out
@@ -63,11 +74,52 @@ cudaError_t launch_limb_gemm(const LimbJob &job, const Items &it, cudaStream_t s
 void configure_limb();
 
 // Byte offset of the 8 digits (of one limb) of row `r`, k in [8 q, 8 q + 8) in
-// an operand tile of `blk` bytes per digit and k-step: core matrices of 8 rows
-// x 16 bytes, the two of a k-step next to each other, rows in groups of 8.
+// an operand tile of `blk` bytes per digit and k-step: per half k-step, the rows
+// one after the other, 16 bytes each (core matrices of 8 rows, 128 bytes apart).
 __host__ __device__ inline long limb_chunk_off(int r, int q, int blk) {
-    return (long)(q >> 1) * (kLimbs * (long)blk) + (r >> 3) * 256 + (q & 1) * 128 + (r & 7) * 16;
+    return (long)(q >> 1) * (kLimbs * (long)blk) + (q & 1) * (blk / 2) + r * 16;
 }
+
+#ifdef __CUDACC__
+constexpr int kLimbBias = 55;  // |X| <= 2^55
+
+// Seven balanced base-256 digits of X: byte 6 - i of the result is d_i + 128
+// (d_0 = 128, at the very top of the range, carries into bit 56).
+__device__ __forceinline__ unsigned long long digit_bytes(long long X) {
+    return (unsigned long long)(X + 0x0080808080808080ll);
+}
+// X = rint(x 2^(55 - e)) for |x| < 2^e, from the bits (round half up; emax: biased
+// exponent of the block's largest magnitude, so e = emax - 1022).
+__device__ __forceinline__ long long to_limb_int(double x, int emax) {
+    const long long b = __double_as_longlong(x);
+    const int ex = (int)((b >> 52) & 0x7ff);
+    long long m = (b & 0xfffffffffffffll) | (ex ? 1ll << 52 : 0);
+    const int sh = emax - (ex ? ex : 1);  // >= 0
+    // at the largest exponent 53 bits become 55
+    m = sh <= 2 ? m << (2 - sh) : (sh > 55 ? 0 : (m >> (sh - 2)) + ((m >> (sh - 3)) & 1));
+    return b < 0 ? -m : m;
+}
+// The same digit (0 = leading) of eight numbers as eight FP16 values.
+__device__ __forceinline__ uint4 digit_chunk(const unsigned long long (&Y)[8], int i) {
+    uint4 r;
+    unsigned *w = &r.x;
+    const __half2 off = __half2half2(__ushort_as_half(0x6480));  // 1024 + 128
+    const unsigned mask = i == 0 ? 0x1ff : 0xff;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const unsigned a = (unsigned)(Y[2 * j] >> (8 * (6 - i))) & mask, b = (unsigned)(Y[2 * j + 1] >> (8 * (6 - i))) & mask;
+        const unsigned pk = 0x64006400u + a + (b << 16);  // 1024 + byte, exactly
+        __half2 h = *(const __half2 *)&pk;
+        h = __hsub2(h, off);
+        w[j] = *(const unsigned *)&h;
+    }
+    return r;
+}
+__device__ __forceinline__ int biased_exp(double x) { return (int)((__double_as_longlong(x) >> 52) & 0x7ff); }
+// Row factor of a table row whose largest magnitude has biased exponent e: an entry is
+// X 2^(e - 1022 - 55), and sums of X Y come divided by 2^48.
+__device__ __forceinline__ double limb_row_factor(int e) { return e ? ldexp(1.0, e - 1022 - 2 * kLimbBias + 48) : 0.0; }
+#endif
 
 // ---- parity classes ---------------------------------------------------------
 // The local field of a patch is a convolution with a kernel that is even along
@@ -187,5 +239,42 @@ cudaError_t limb_conv_tables(int device, const Geom &g, bool share, const double
                              std::shared_ptr<LimbConvTables> *out);
 inline long limb_ctiles(long items) { return (items + kLimbN - 1) / kLimbN; }
 void configure_limb_conv();
+
+// ---- ring products (limb_ring.cu) -------------------------------------------
+// Buffers and layout of one plan's ring products: parts 0..2 the face nodes of
+// an axis, part 3 the coarse nodes.
+struct LimbRing {
+    struct Part {
+        int rows, tiles, cols, ctiles, nq, kst;
+        int lo[3], cnt[3];       // patch offsets per axis
+        long first;              // place of the first column's cell
+        long a_off, rf_off, v_off, v_split;
+        int koff_off;
+    } part[4];
+    int np, nch, T, clo, chi, splits;
+    long origin, places;         // of the padded patch grid
+    long a_bytes = 0, rf_rows = 0, v_total = 0;
+    int nkoff = 0;
+    unsigned char *A = nullptr, *C = nullptr;  // table digits, coefficient digits
+    double *rf = nullptr, *cf = nullptr, *V = nullptr;
+    int *koff = nullptr;
+    ~LimbRing();
+};
+// What the boundary and coarse-charge kernels read: the ring term of row `row`
+// of cell (i0, i1, i2) in part p.
+struct RingView {
+    const double *V;
+    long off[4], step[4], first[4];
+    int T, splits;
+    __device__ __forceinline__ double at(int p, int i0, int i1, int i2, int rows, int row) const {
+        const double *v = V + off[p] + (((long)i0 * T + i1) * T + i2 - first[p]) * rows + row;
+        double s = 0.0;
+        for (int k = 0; k < splits; ++k) s += v[k * step[p]];
+        return s;
+    }
+};
+bool limb_ring_layout(const Geom &g, LimbRing &r);
+cudaError_t limb_ring_create(const Geom &g, const std::vector<double> &D, const std::vector<double> &T, LimbRing &r);
+RingView limb_ring_view(const LimbRing &r);
 
 }  // namespace mlc

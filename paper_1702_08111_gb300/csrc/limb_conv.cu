@@ -26,52 +26,11 @@
 #include <tuple>
 #include <vector>
 
-#include <cuda_fp16.h>
-
 #include "limb.h"
 #include "mlc_internal.h"
 
 namespace mlc {
 namespace {
-
-constexpr int kBias = 55;  // |X| <= 2^55
-
-// Seven balanced base-256 digits of X: byte 6 - i of the result is d_i + 128
-// (d_0 = 128, at the very top of the range, carries into bit 56).
-__device__ __forceinline__ unsigned long long digit_bytes(long long X) {
-    return (unsigned long long)(X + 0x0080808080808080ll);
-}
-
-// X = rint(x 2^(55 - e)) for |x| < 2^e, from the bits (round half up; emax: biased
-// exponent of the block's largest magnitude, so e = emax - 1022).
-__device__ __forceinline__ long long to_limb_int(double x, int emax) {
-    const long long b = __double_as_longlong(x);
-    const int ex = (int)((b >> 52) & 0x7ff);
-    long long m = (b & 0xfffffffffffffll) | (ex ? 1ll << 52 : 0);
-    const int sh = emax - (ex ? ex : 1);  // >= 0
-    // at the largest exponent 53 bits become 55
-    m = sh <= 2 ? m << (2 - sh) : (sh > 55 ? 0 : (m >> (sh - 2)) + ((m >> (sh - 3)) & 1));
-    return b < 0 ? -m : m;
-}
-
-// The same digit (0 = leading) of eight numbers as four half2.
-__device__ __forceinline__ uint4 digit_chunk(const unsigned long long (&Y)[8], int i) {
-    uint4 r;
-    unsigned *w = &r.x;
-    const __half2 off = __half2half2(__ushort_as_half(0x6480));  // 1024 + 128
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const unsigned mask = i == 0 ? 0x1ff : 0xff;
-        const unsigned a = (unsigned)(Y[2 * j] >> (8 * (6 - i))) & mask, b = (unsigned)(Y[2 * j + 1] >> (8 * (6 - i))) & mask;
-        const unsigned pk = 0x64006400u + a + (b << 16);  // 1024 + byte, exactly
-        __half2 h = *(const __half2 *)&pk;
-        h = __hsub2(h, off);
-        w[j] = *(const unsigned *)&h;
-    }
-    return r;
-}
-
-__device__ __forceinline__ int biased_exp(double x) { return (int)((__double_as_longlong(x) >> 52) & 0x7ff); }
 
 // ---------------------------------------------------------------------------
 // Tables: one CTA per row of one table.  Entry (row, k) is the Green's function
@@ -120,8 +79,7 @@ __global__ void __launch_bounds__(256) k_limb_table(LimbConvGeom g, int u, const
     if ((threadIdx.x & 31) == 0) atomicMax(&smax, mx);
     __syncthreads();
     const int e = smax;
-    // |v| < 2^(e - 1022); value = X 2^(e - 1022 - 55), and the sums come as X Y / 2^48
-    if (threadIdx.x == 0) rf[g.rf_off[u] + row] = e ? ldexp(1.0, e - 1022 - 2 * kBias + 48) : 0.0;
+    if (threadIdx.x == 0) rf[g.rf_off[u] + row] = limb_row_factor(e);
     unsigned char *At = A + g.a_off[u] + (long)(row / kLimbM) * g.kst[u] * kLimbAStep;
     for (int q = threadIdx.x; q < kpad / 8; q += blockDim.x) {
         unsigned long long Y[8];
@@ -489,14 +447,14 @@ static cudaError_t limb_conv_group(const mlc_plan_s *pl, const Items &it, cudaSt
     int t0 = 0;
     for (int c = 0; c < 8; ++c) {
         const int u = limb_table(g.share, c);
-        job.part[c] = LimbPart{T.A + g.a_off[u], T.rf + g.rf_off[u], g.b_step[c], g.v_step[c], g.kst[u], g.rows[u], g.tiles[u], t0};
+        job.part[c] = LimbPart{T.A + g.a_off[u], (long)g.kst[u] * kLimbAStep, T.rf + g.rf_off[u], nullptr, g.b_step[c] * ct, g.v_step[c] * items,
+                               c * ct * kLimbN, g.kst[u], g.rows[u], (int)items, (int)ct, t0};
         t0 += g.tiles[u] * (int)ct;
     }
     job.B = B;
     job.cf = cf;
+    job.cf_step = 1;
     job.V = V;
-    job.cols = (int)items;
-    job.ctiles = (int)ct;
     job.ntiles = t0;
     job.wait_tries = 1 << 22;
     if (pl->fault == 1) {  // test hook: the waits must run out, quickly

@@ -3,10 +3,10 @@
 //
 // A work tile is 128 table rows x 64 columns of one block.  Its seven level
 // accumulators (7 x 64 FP32 columns) fill TMEM's 512 columns, so one CTA runs
-// per SM.  Per k-step of 16 a producer thread brings the seven digits of the
-// rows and of the columns into shared memory with two bulk copies (28 + 14 KB,
-// laid out in global memory as the canonical K-major core matrices, so a copy
-// is one contiguous run), five steps deep; one thread issues the 28 MMAs of
+// per SM.  Per k-step of 16 a producer warp brings the seven digits of the rows
+// and of the columns into shared memory with bulk copies (28 + 14 KB, laid out in
+// global memory as the canonical K-major core matrices, so a copy is one
+// contiguous run; shifted columns in fourteen runs of 1 KB), five steps deep; one thread issues the 28 MMAs of
 // digit pairs i + j < 7; after every 16 steps eight warps read the levels,
 // combine them into two 64-bit integers per output (exact) and hand the
 // accumulators back.  The FP64 conversion of a finished tile therefore runs
@@ -58,9 +58,9 @@ __device__ __forceinline__ void bulk_in(void *dst, const void *src, unsigned byt
                  : "memory");
 }
 // canonical K-major layout without swizzle: core matrices 128 bytes apart along
-// K, 256 along M / N (descriptor version 1)
-__device__ __forceinline__ uint64_t mat_desc(uint32_t addr) {
-    return (uint64_t)((addr >> 4) & 0x3FFFu) | (uint64_t)(128 >> 4) << 16 | (uint64_t)(256 >> 4) << 32 |
+// M / N, half a k-step's rows apart along K (descriptor version 1)
+__device__ __forceinline__ uint64_t mat_desc(uint32_t addr, uint32_t khalf) {
+    return (uint64_t)((addr >> 4) & 0x3FFFu) | (uint64_t)(khalf >> 4) << 16 | (uint64_t)(128 >> 4) << 32 |
            (uint64_t)1 << 46;
 }
 // kind::f16: FP32 accumulator, FP16 A and B, both K-major
@@ -89,9 +89,8 @@ __device__ __forceinline__ void tmem_ld16(uint32_t t, uint32_t (&r)[16]) {
 
 __device__ __forceinline__ const LimbPart &part_of(const LimbJob &job, int t) {
     int p = 0;
-#pragma unroll
-    for (int i = 1; i < kLimbMaxParts; ++i)
-        if (i < job.nparts && t >= job.part[i].tile0) p = i;
+    for (int i = 1; i < job.nparts; ++i)
+        if (t >= job.part[i].tile0) p = i;
     return job.part[p];
 }
 
@@ -124,34 +123,42 @@ __global__ void __launch_bounds__(kThreads, 1) k_limb_gemm(const __grid_constant
     const int tries = job.wait_tries;
 
     if (warp == kEpiWarps) {  // producer
-        if (lane == 0) {
-            int step = 0;
-            bool ok = true;
-            for (int t = blockIdx.x; ok && t < job.ntiles; t += gridDim.x) {
-                const LimbPart &P = part_of(job, t);
-                const int local = t - P.tile0, rt = local / job.ctiles, ct = local - rt * job.ctiles;
-                const unsigned char *a = P.A + (long)rt * P.kst * kLimbAStep;
-                const unsigned char *b = job.B + P.b_off * job.ctiles + (long)ct * P.kst * kLimbBStep;
-                for (int k = 0; k < P.kst; ++k, ++step) {
-                    const int s = step % kStages;
-                    if (!mb_wait(&empty[s], ((step / kStages) & 1) ^ 1, tries) || atomicAdd(&failed, 0)) {
-                        ok = false;
-                        break;
-                    }
-                    mb_expect(&full[s], kStageBytes);
-                    if (!job.skip_copy) {
-                        bulk_in(sm + s * kStageBytes, a + (long)k * kLimbAStep, kLimbAStep, &full[s]);
-                        bulk_in(sm + s * kStageBytes + kLimbAStep, b + (long)k * kLimbBStep, kLimbBStep, &full[s]);
+        int step = 0;
+        bool ok = true;
+        for (int t = blockIdx.x; ok && t < job.ntiles; t += gridDim.x) {
+            const LimbPart &P = part_of(job, t);
+            const int local = t - P.tile0, rt = local / P.ctiles, ct = local - rt * P.ctiles;
+            const unsigned char *a = P.A + (long)rt * P.a_tile;
+            const unsigned char *b = job.B + P.b_off + (long)ct * P.kst * kLimbBStep;
+            // shifted columns: lane 2 d + half copies its half k-step of digit d
+            const unsigned char *bs = job.B + (lane >> 1) * job.b_digit + (long)ct * kLimbN * 16;
+            for (int k = 0; k < P.kst; ++k, ++step) {
+                const int s = step % kStages;
+                const int at = P.koff && lane < 2 * kLimbs ? P.koff[2 * k + (lane & 1)] : 0;
+                if (lane == 0) {
+                    ok = mb_wait(&empty[s], ((step / kStages) & 1) ^ 1, tries) && !atomicAdd(&failed, 0);
+                    if (ok) mb_expect(&full[s], kStageBytes);
+                }
+                ok = __shfl_sync(0xffffffffu, ok, 0);
+                if (!ok) break;
+                unsigned char *dst = sm + s * kStageBytes;
+                if (!job.skip_copy) {
+                    if (lane == 0) bulk_in(dst, a + (long)k * kLimbAStep, kLimbAStep, &full[s]);
+                    dst += kLimbAStep;
+                    if (P.koff) {
+                        if (lane < 2 * kLimbs) bulk_in(dst + lane * (kLimbBBlk / 2), bs + (long)at * 16, kLimbBBlk / 2, &full[s]);
+                    } else if (lane == 0) {
+                        bulk_in(dst, b + (long)k * kLimbBStep, kLimbBStep, &full[s]);
                     }
                 }
             }
-            if (!ok) {
-                atomicExch(&failed, 1);
-                // the copies in flight land in shared memory: wait (again bounded) for each stage last filled
-                for (int i = 0; i < kStages && i < step; ++i) {
-                    const int q = step - 1 - i;
-                    mb_wait(&full[q % kStages], (q / kStages) & 1, tries);
-                }
+        }
+        if (!ok && lane == 0) {
+            atomicExch(&failed, 1);
+            // the copies in flight land in shared memory: wait (again bounded) for each stage last filled
+            for (int i = 0; i < kStages && i < step; ++i) {
+                const int q = step - 1 - i;
+                mb_wait(&full[q % kStages], (q / kStages) & 1, tries);
             }
         }
     } else if (warp == kEpiWarps + 1) {  // MMA issue
@@ -178,10 +185,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_limb_gemm(const __grid_constant
                     const uint32_t a0 = s32(sm + s * kStageBytes), b0 = a0 + kLimbAStep;
 #pragma unroll
                     for (int i = 0; i < kLimbs; ++i) {
-                        const uint64_t da = mat_desc(a0 + i * kLimbABlk);
+                        const uint64_t da = mat_desc(a0 + i * kLimbABlk, kLimbABlk / 2);
 #pragma unroll
                         for (int j = 0; i + j < kLimbLevels && j < kLimbs; ++j)
-                            mma_f16(tmem + (uint32_t)((i + j) * kLimbN), da, mat_desc(b0 + j * kLimbBBlk),
+                            mma_f16(tmem + (uint32_t)((i + j) * kLimbN), da, mat_desc(b0 + j * kLimbBBlk, kLimbBBlk / 2),
                                     (first && i == 0) ? 0u : 1u);
                     }
                     commit(&empty[s]);
@@ -207,7 +214,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_limb_gemm(const __grid_constant
         bool ok = true;
         for (int t = blockIdx.x; ok && t < job.ntiles; t += gridDim.x) {
             const LimbPart &P = part_of(job, t);
-            const int local = t - P.tile0, rt = local / job.ctiles, ct = local - rt * job.ctiles;
+            const int local = t - P.tile0, rt = local / P.ctiles, ct = local - rt * P.ctiles;
             long long hi[32], lo[32];  // sum = hi 2^32 + lo
 #pragma unroll
             for (int j = 0; j < 32; ++j) hi[j] = lo[j] = 0;
@@ -236,21 +243,20 @@ __global__ void __launch_bounds__(kThreads, 1) k_limb_gemm(const __grid_constant
             if (!ok) break;
             const int row = rt * kLimbM + sub * 32 + lane, c0 = ct * kLimbN + half * 32;
             const double rf = P.rf[row];
-            const double *cf = job.cf + (long)(&P - job.part) * job.ctiles * kLimbN + c0;
-            double *v = job.V + P.v_off * job.cols + (long)c0 * P.rows + row;
+            const double *cf = job.cf + P.cf_off + (long)c0 * job.cf_step;
+            double *v = job.V + P.v_off + (long)c0 * P.rows + row;
             if (row < P.rows) {
 #pragma unroll
                 for (int j = 0; j < 32; ++j)
-                    if (c0 + j < job.cols)
-                        v[(long)j * P.rows] = fma((double)hi[j], 4294967296.0, (double)lo[j]) * rf * cf[j];
+                    if (c0 + j < P.cols)
+                        v[(long)j * P.rows] = fma((double)hi[j], 4294967296.0, (double)lo[j]) * rf * cf[j * job.cf_step];
             }
         }
         if (!ok) {
             atomicExch(&failed, 1);
-            if (threadIdx.x == 0)  // every plan with a column in this launch
-                for (int c = 0; c < job.cols; ++c) {
-                    const PlanPtrs &rec = it.plans[it.items ? it.items[c].x : 0];
-                    atomicExch(rec.err, 1);
+            if (threadIdx.x == 0)  // every plan with an item in this launch
+                for (int c = 0; c < it.nitems; ++c) {
+                    atomicExch(it.plans[it.items ? it.items[c].x : 0].err, 1);
                     if (!it.items) break;
                 }
         }

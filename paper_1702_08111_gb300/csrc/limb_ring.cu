@@ -1,0 +1,298 @@
+// The Legendre ring terms of the FP64 and double-float tiers as exact-split
+// tensor-core products (limb.h): for every face-plane node the sum over the
+// patches around it of c_q (B_q - I^H B_q) (eq. philocmlcII), and for every
+// coarse node the ring part of F^H (eq. FDLD).
+//
+// Nodes come in cells of one patch's size.  All nodes of a cell see the same
+// patches, up to their offset from the cell, so the terms are one product: rows
+// the n^2 nodes of a cell's lower face (per axis) or its (n/4)^3 coarse nodes,
+// K the coefficients of the patches around a cell (Q = 6: 4 x 5 x 5 patches for
+// a face, 5^3 for coarse nodes), columns the cells.  The columns read the digits
+// of the patches' coefficients in place, shifted by the patch offset: patches
+// and cells lie on a grid whose rows are padded with zeros, so that the cells of
+// a column tile stay consecutive under every shift, and each k-group of a tile
+// is one run of 1 KB.  One FP64 value per node leaves the product.
+//
+// Before, each node formed its own dot products of npoly coefficients, up to 64
+// of them, on the FP64 pipe.  256^3, FP64, boundary values + coarse charge with
+// the products: n = 16, Q = 6 (125 patches around a cell) 5.35 + 0.80 -> 0.16 +
+// 1.43 ms; n = 32 2.19 + 0.78 -> 0.11 + 1.19 ms; 32^3, n = 8: 0.088 + 0.082 ->
+// 0.014 + 0.056 ms; double-float 128^3, n = 16, Q = 4: 0.257 + 0.109 -> 0.037 +
+// 0.201 ms.  The table (31 MB at n = 16) is read from L2.
+#include <cooperative_groups.h>
+
+#include <algorithm>
+#include <climits>
+#include <cmath>
+#include <vector>
+
+#include "limb.h"
+#include "mlc_internal.h"
+
+namespace mlc {
+namespace {
+
+int fdiv(int a, int b) { return a >= 0 ? a / b : -((-a + b - 1) / b); }
+int cdiv(int a, int b) { return -fdiv(-a, b); }
+
+constexpr int kDigitCtas = 8;  // one cluster
+
+struct DigitArgs {
+    const double *mom;  // [NP][npad]
+    unsigned char *C;   // [digit][k-group][place][8 k]
+    double *cf;         // the common column factor
+    int NP, np, npoly, npad, nch;
+    int T;
+    long origin, places;
+};
+
+// Coefficients to digits under one scale, the largest magnitude of the problem
+// (every value of the potential is of that order).  One cluster, so that the
+// scale and the digits take one launch: a few loads and stores per thread.
+__global__ void __cluster_dims__(kDigitCtas, 1, 1) __launch_bounds__(1024) k_ring_digits(DigitArgs a) {
+    __shared__ int smax;
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    const int gt = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
+    if (threadIdx.x == 0) smax = 0;
+    cl.sync();
+    int mx = 0;
+    for (long e = gt; e < (long)a.NP * a.npoly; e += nt) {
+        const long p = e / a.npoly;
+        mx = max(mx, biased_exp(a.mom[p * a.npad + (e - p * a.npoly)]));
+    }
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    if ((threadIdx.x & 31) == 0 && mx)
+        for (int r = 0; r < kDigitCtas; ++r) atomicMax(cl.map_shared_rank(&smax, r), mx);
+    cl.sync();
+    const int e = smax;
+    const bool live = e != 0 && e != 0x7ff;
+    if (gt == 0) *a.cf = e == 0x7ff ? __longlong_as_double(0x7ff8000000000000ll) : (live ? ldexp(1.0, e - 1022) : 0.0);
+    for (long w = gt; w < (long)a.NP * a.nch; w += nt) {
+        const int p = (int)(w % a.NP), q = (int)(w / a.NP);
+        const int i2 = p % a.np, i1 = (p / a.np) % a.np, i0 = p / (a.np * a.np);
+        unsigned long long Y[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const int k = 8 * q + j;
+            Y[j] = digit_bytes(live && k < a.npoly ? to_limb_int(a.mom[(long)p * a.npad + k], e) : 0);
+        }
+        const long place = ((long)i0 * a.T + i1) * a.T + i2 + a.origin;
+#pragma unroll
+        for (int i = 0; i < kLimbs; ++i)
+            *(uint4 *)(a.C + (((long)i * a.nch + q) * a.places + place) * 16) = digit_chunk(Y, i);
+    }
+}
+
+// Table rows of one part (axis 0..2: face nodes; 3: coarse nodes) from the dense
+// ring tables D [axis][plane][u][v][npad], T [coarse cell][npoly], whose entries
+// are zero off the ring.
+struct TabArgs {
+    const double *D, *T;
+    int n, gb, wbx, pb0, npb, npoly, npad, nch;
+    int cb_lo, ncb;
+    int axis, rows, nq, kst;       // k-groups in all
+    int lo[3], cnt[3];             // patch offsets delta = lo + [0, cnt) per axis (row-major)
+    unsigned char *A;
+    double *rf;
+};
+
+__global__ void __launch_bounds__(256) k_ring_table(TabArgs a) {
+    __shared__ int smax;
+    const int row = blockIdx.x;
+    if (threadIdx.x == 0) smax = 0;
+    __syncthreads();
+    auto entry = [&](int q, int j) -> double {
+        const int p = 8 * (q % a.nch) + j;
+        int r = q / a.nch;
+        if (row >= a.rows || q >= a.nq || p >= a.npoly) return 0.0;
+        int del[3];
+        del[2] = a.lo[2] + r % a.cnt[2];
+        r /= a.cnt[2];
+        del[1] = a.lo[1] + r % a.cnt[1];
+        del[0] = a.lo[0] + r / a.cnt[1];
+        if (a.axis == 3) {
+            const int c = a.n / 4;
+            const int r0 = row / (c * c) - c * del[0] - a.cb_lo, r1 = (row / c) % c - c * del[1] - a.cb_lo,
+                      r2 = row % c - c * del[2] - a.cb_lo;
+            if (r0 < 0 || r1 < 0 || r2 < 0 || r0 >= a.ncb || r1 >= a.ncb || r2 >= a.ncb) return 0.0;
+            return a.T[(((long)r0 * a.ncb + r1) * a.ncb + r2) * a.npoly + p];
+        }
+        const int iu = a.axis == 0 ? 1 : 0, iv = a.axis == 2 ? 1 : 2;
+        const int pl = -a.n * del[a.axis] - a.pb0, u = row / a.n - a.n * del[iu] + a.gb, v = row % a.n - a.n * del[iv] + a.gb;
+        if (pl < 0 || pl / a.n >= a.npb || u < 0 || v < 0 || u >= a.wbx || v >= a.wbx) return 0.0;
+        return a.D[((((long)a.axis * a.npb + pl / a.n) * a.wbx + u) * a.wbx + v) * a.npad + p];
+    };
+    int mx = 0;
+    for (int e = threadIdx.x; e < a.nq * 8; e += blockDim.x) mx = max(mx, biased_exp(entry(e >> 3, e & 7)));
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    if ((threadIdx.x & 31) == 0) atomicMax(&smax, mx);
+    __syncthreads();
+    const int e = smax;
+    if (threadIdx.x == 0) a.rf[row] = limb_row_factor(e);
+    unsigned char *At = a.A + (long)(row / kLimbM) * a.kst * kLimbAStep;
+    for (int q = threadIdx.x; q < a.kst * 2; q += blockDim.x) {
+        unsigned long long Y[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) Y[j] = digit_bytes(e ? to_limb_int(entry(q, j), e) : 0);
+        unsigned char *p = At + limb_chunk_off(row % kLimbM, q, kLimbABlk);
+#pragma unroll
+        for (int i = 0; i < kLimbs; ++i) *(uint4 *)(p + i * kLimbABlk) = digit_chunk(Y, i);
+    }
+}
+
+}  // namespace
+
+LimbRing::~LimbRing() {
+    for (void *p : {(void *)A, (void *)rf, (void *)koff, (void *)C, (void *)cf, (void *)V}) cudaFree(p);
+}
+
+// The layout of the ring products of a plan, or false where the per-node sums
+// stay: more patches around a cell than kRingPatches, whose table would not pay
+// (a caller's g_beta of many patch sizes on a small problem).
+bool limb_ring_layout(const Geom &g, LimbRing &r) {
+    constexpr int kRingPatches = 216;
+    r.np = g.np;
+    r.nch = (g.npoly + 7) / 8;
+    const int n = g.n, c = n / 4;
+    // cells and patch offsets per axis: of a face's normal, its in-plane axes, coarse nodes
+    const int norm_lo = cdiv(-n - g.gb, n), norm_hi = fdiv(g.gb, n);
+    const int in_lo = cdiv(-n - g.gb, n), in_hi = fdiv(n - 1 + g.gb, n);
+    const int co_lo = cdiv(-g.cb_hi, c), co_hi = fdiv(c - 1 - g.cb_lo, c);
+    r.clo = fdiv(g.flo, c);
+    r.chi = fdiv(g.fhi, c);
+    const long around = (long)(co_hi - co_lo + 1) * (co_hi - co_lo + 1) * (co_hi - co_lo + 1);
+    if (around > kRingPatches) return false;
+    int qlo = std::min(std::min(norm_lo, in_lo), r.clo + co_lo), qhi = std::max(g.np + std::max(norm_hi, in_hi), r.chi + co_hi);
+    // rows of T places: patches first, then zeros that serve as the margin on both sides
+    r.T = std::max({g.np - qlo, qhi + 1, r.chi - r.clo + 1, g.np + 1});
+    const long T = r.T;
+    long lowest = LONG_MAX, highest = 0;
+    for (int ax = 0; ax < 4; ++ax) {
+        LimbRing::Part &p = r.part[ax];
+        p = LimbRing::Part{};
+        p.rows = ax < 3 ? n * n : c * c * c;
+        p.tiles = (p.rows + kLimbM - 1) / kLimbM;
+        const int c0 = ax < 3 ? 0 : r.clo, c1 = ax < 3 ? g.np : r.chi;
+        p.first = ((long)c0 * T + c0) * T + c0;
+        p.cols = (int)(((long)c1 * T + c1) * T + c1 - p.first + 1);
+        p.ctiles = (p.cols + kLimbN - 1) / kLimbN;
+        int nb = 1;
+        for (int d = 0; d < 3; ++d) {
+            p.lo[d] = ax == 3 ? co_lo : (d == ax ? norm_lo : in_lo);
+            p.cnt[d] = (ax == 3 ? co_hi : (d == ax ? norm_hi : in_hi)) - p.lo[d] + 1;
+            nb *= p.cnt[d];
+        }
+        p.nq = nb * r.nch;
+        p.kst = (p.nq + 1) / 2;
+        const long dlo = ((long)p.lo[0] * T + p.lo[1]) * T + p.lo[2];
+        const long dhi = ((long)(p.lo[0] + p.cnt[0] - 1) * T + (p.lo[1] + p.cnt[1] - 1)) * T + (p.lo[2] + p.cnt[2] - 1);
+        lowest = std::min(lowest, p.first + dlo);
+        highest = std::max(highest, p.first + dhi + (long)p.ctiles * kLimbN);
+    }
+    r.origin = std::max(0l, -lowest);
+    r.places = std::max(highest, ((long)(g.np - 1) * T + g.np - 1) * T + g.np) + r.origin;
+    // a small problem has few tiles: split the sums so that they fill the SMs
+    long tiles = 0, steps = LONG_MAX;
+    for (auto &p : r.part) {
+        tiles += (long)p.tiles * p.ctiles;
+        steps = std::min<long>(steps, p.kst);
+    }
+    r.splits = (int)std::max(1l, std::min({(long)kLimbMaxParts / 4, 152 / tiles, steps}));
+    for (auto &p : r.part) {
+        p.a_off = r.a_bytes;
+        p.rf_off = r.rf_rows;
+        p.koff_off = r.nkoff;
+        p.v_off = r.v_total;
+        p.v_split = (long)p.cols * p.rows;
+        r.a_bytes += (long)p.tiles * p.kst * kLimbAStep;
+        r.rf_rows += (long)p.tiles * kLimbM;
+        r.nkoff += 2 * p.kst;
+        r.v_total += r.splits * p.v_split;
+    }
+    return true;
+}
+
+// Tables and buffers of a plan's ring products from the dense ring tables (host).
+cudaError_t limb_ring_create(const Geom &g, const std::vector<double> &D, const std::vector<double> &T, LimbRing &r) {
+    auto up = [](auto **dst, const auto &v) -> cudaError_t {
+        const size_t b = v.size() * sizeof(v[0]);
+        cudaError_t e = cudaMalloc((void **)dst, b);
+        return e == cudaSuccess ? cudaMemcpy((void *)*dst, v.data(), b, cudaMemcpyHostToDevice) : e;
+    };
+    std::vector<int> ko(r.nkoff, 0);
+    for (auto &p : r.part)
+        for (int q = 0; q < 2 * p.kst; ++q) {
+            const int qq = std::min(q, p.nq - 1);  // a last odd half k-step meets zero table digits
+            int nb = qq / r.nch;
+            const int d2 = p.lo[2] + nb % p.cnt[2], d1 = p.lo[1] + (nb / p.cnt[2]) % p.cnt[1],
+                      d0 = p.lo[0] + nb / (p.cnt[2] * p.cnt[1]);
+            ko[p.koff_off + q] = (int)((qq % r.nch) * r.places + r.origin + p.first + ((long)d0 * r.T + d1) * r.T + d2);
+        }
+    double *dD = nullptr, *dT = nullptr;
+    cudaError_t e = up(&dD, D);
+    if (e == cudaSuccess) e = up(&dT, T);
+    if (e == cudaSuccess) e = up(&r.koff, ko);
+    const size_t cbytes = (size_t)kLimbs * r.nch * r.places * 16;
+    if (e == cudaSuccess) e = cudaMalloc((void **)&r.A, (size_t)r.a_bytes);
+    if (e == cudaSuccess) e = cudaMalloc((void **)&r.rf, (size_t)r.rf_rows * sizeof(double));
+    if (e == cudaSuccess) e = cudaMalloc((void **)&r.C, cbytes);
+    if (e == cudaSuccess) e = cudaMemset(r.C, 0, cbytes);  // the margins stay zero
+    if (e == cudaSuccess) e = cudaMalloc((void **)&r.cf, sizeof(double));
+    if (e == cudaSuccess) e = cudaMalloc((void **)&r.V, (size_t)r.v_total * sizeof(double));
+    for (int ax = 0; ax < 4 && e == cudaSuccess; ++ax) {
+        const LimbRing::Part &p = r.part[ax];
+        TabArgs a{dD, dT, g.n, g.gb, g.wbx, g.pb0, g.npb, g.npoly, g.npad, r.nch, g.cb_lo, g.cb_hi - g.cb_lo + 1,
+                  ax, p.rows, p.nq, p.kst, {p.lo[0], p.lo[1], p.lo[2]}, {p.cnt[0], p.cnt[1], p.cnt[2]},
+                  r.A + p.a_off, r.rf + p.rf_off};
+        k_ring_table<<<p.tiles * kLimbM, 256>>>(a);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaDeviceSynchronize();
+    cudaFree(dD);
+    cudaFree(dT);
+    return e;
+}
+
+RingView limb_ring_view(const LimbRing &r) {
+    RingView v{};
+    v.V = r.V;
+    v.T = r.T;
+    v.splits = r.splits;
+    for (int i = 0; i < 4; ++i) {
+        v.off[i] = r.part[i].v_off;
+        v.step[i] = r.part[i].v_split;
+        v.first[i] = r.part[i].first;
+    }
+    return v;
+}
+
+cudaError_t launch_limb_ring(const mlc_plan_s *pl, cudaStream_t st) {
+    const LimbRing &r = *pl->limb_ring;
+    const Geom &g = pl->g;
+    DigitArgs d{pl->mom, r.C, r.cf, g.NP, g.np, g.npoly, g.npad, r.nch, r.T, r.origin, r.places};
+    k_ring_digits<<<kDigitCtas, 1024, 0, st>>>(d);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    LimbJob job{};
+    int t0 = 0, np = 0;
+    for (const auto &p : r.part)
+        for (int s = 0; s < r.splits; ++s) {
+            const int k0 = (int)((long)p.kst * s / r.splits), k1 = (int)((long)p.kst * (s + 1) / r.splits);
+            job.part[np++] = LimbPart{r.A + p.a_off + (long)k0 * kLimbAStep, (long)p.kst * kLimbAStep, r.rf + p.rf_off, r.koff + p.koff_off + 2 * k0, 0,
+                                      p.v_off + s * p.v_split, 0, k1 - k0, p.rows, p.cols, p.ctiles, t0};
+            t0 += p.tiles * p.ctiles;
+        }
+    job.nparts = np;
+    job.B = r.C;
+    job.b_digit = (long)r.nch * r.places * 16;
+    job.cf = r.cf;
+    job.cf_step = 0;
+    job.V = r.V;
+    job.ntiles = t0;
+    job.wait_tries = 1 << 22;
+    Items it{nullptr, pl->dptrs, 1};
+    return launch_limb_gemm(job, it, st);
+}
+
+}  // namespace mlc

@@ -232,6 +232,7 @@ struct mlc_plan_s {
     void *D2tab = nullptr;     // [axis][npb][2][wbx][wbx][npad] ring rows of the off-face nodes
     void *f_stage, *phi_stage;  // device staging for mlc_solve_host
     std::shared_ptr<mlc::LimbConvTables> limb_tabs;  // FP64 and double-float tiers: folded Green's function
+    std::shared_ptr<mlc::LimbRing> limb_ring;        // and ring products (null: no ring, or per-node sums)
     int *err;                // device error word: nonzero if a bounded wait in a kernel gave up
     size_t ws_bytes;
     std::vector<void *> owned;  // device allocations to free
@@ -278,6 +279,8 @@ cudaError_t launch_moments(const mlc_plan_s *pl, const Items &it, cudaStream_t s
 cudaError_t launch_patch_conv(const mlc_plan_s *pl, const Items &it, cudaStream_t st);
 // limb_conv.cu: the local convolutions of the FP64 and double-float tiers
 cudaError_t launch_limb_conv(const mlc_plan_s *pl, const Items &it, cudaStream_t st);
+// limb_ring.cu: their Legendre ring terms (after the moments, before F^H and phi^B)
+cudaError_t launch_limb_ring(const mlc_plan_s *pl, cudaStream_t st);
 cudaError_t launch_resid(const mlc_plan_s *pl, const Items &it, cudaStream_t st);
 cudaError_t launch_dirichlet(const mlc_plan_s *pl, const Items &it, cudaStream_t st);
 cudaError_t launch_assemble(const mlc_plan_s *pl, cudaStream_t st);

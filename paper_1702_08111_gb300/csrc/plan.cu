@@ -544,8 +544,18 @@ mlc_status build_tables(mlc_plan_s *pl) {
             pl->D2tab = d;
         }
     }
-    // ring tables in the ring precision: the local-convolution arithmetic
-    if (g.conv == CONV_F32) {
+    // ring tables: digits for the ring products (FP64, double-float), else in the
+    // ring precision, the local-convolution arithmetic
+    if (ring && g.conv != CONV_F32) {
+        auto r = std::make_shared<LimbRing>();
+        if (limb_ring_layout(g, *r)) {
+            TRY_CUDA(limb_ring_create(g, Dtab, Ttab, *r));
+            pl->limb_ring = r;
+        }
+    }
+    if (pl->limb_ring) {
+        // the digits replace them
+    } else if (g.conv == CONV_F32) {
         float *d = nullptr, *t = nullptr;
         TRY(dev_upload(pl, &d, std::vector<float>(Dtab.begin(), Dtab.end())));
         TRY(dev_upload(pl, &t, std::vector<float>(Ttab.begin(), Ttab.end())));

@@ -10,6 +10,8 @@ so the sum over at most nb^3 terms is off by at most nb^3 * 8 F g * (2 * 2^-55 +
 unfolding add less than 16 nb^3 F g 2^-53.  Both together stay below
 80 nb^3 F g 2^-54 (about 1e-14 of a field of one sign).  A double-float result
 adds 2^-47 of itself."""
+import functools
+
 import numpy as np
 import pytest
 
@@ -152,3 +154,42 @@ def test_results_do_not_depend_on_the_launch_groups(torch_cuda):
     ref = _plan(torch, N, n, s, 4, 0).solve(f)
     for chunk in (1, 7, 64, 100):
         assert torch.equal(_plan(torch, N, n, s, 4, 0, conv_chunk=chunk).solve(f), ref)
+
+
+@functools.lru_cache(maxsize=None)
+def _oracle_stages(N, n, s, Q, P, g_beta):
+    from oracle import mlc_oracle as O
+    from paper_1702_08111_gb300 import inputs as I
+    f = I.sample_bumps(N, I.draw_bumps(3, 70 + N + P))
+    prm = O.Params(N=N, n=n, s=s, P=P, Q=Q, beta=(1 + 2 * g_beta / n) if g_beta else None)
+    st = {}
+    O.mlc_solve(prm, O.pad_charge(f), stages=st)
+    return f, prm, st
+
+
+@pytest.mark.parametrize("N,n,s,Q,P,g_beta", [
+    (8, 4, 8, 4, 4, 0),       # 16 face nodes and one coarse node of a tile of 128; split sums
+    (12, 4, 12, 6, 6, 0),     # 56 coefficients in seven groups of 8
+    (24, 8, 12, 6, 1, 0),     # one coefficient of a group of 8
+    (16, 8, 12, 4, 6, 11),    # an outer radius that is no multiple of 4
+    (24, 12, 16, 6, 5, 0),    # two ragged row tiles per axis
+    (32, 16, 16, 4, 2, 0),    # two patches per axis: most patches around a cell do not exist
+    (8, 4, 8, 4, 4, 16),      # too many patches around a cell: per-node sums
+])
+@pytest.mark.parametrize("tier", [0, 2])
+def test_ring_products_against_the_oracle(torch_cuda, N, n, s, Q, P, g_beta, tier):
+    """F^H and phi^B with the Legendre ring as one product over the patches around a cell, at its
+    edges, against the oracle's literal sums.  Tolerance: the parity bar of these stages, 1e-12 of
+    the largest value (the products' error is below 1e-15 of it; double-float steps keep 1e-13)."""
+    from paper_1702_08111_gb300 import mlc
+    f, prm, st = _oracle_stages(N, n, s, Q, P, g_beta)
+    plan = mlc.Plan(N, n, s, P, Q, tier=tier, **({"g_beta": g_beta} if g_beta else {}))
+    plan.solve(torch_cuda.from_numpy(f).cuda())
+    assert prm.g_beta == plan.info.g_beta
+    FH, B = plan.export(mlc.STAGE_FH), plan.export(mlc.STAGE_PHIB)
+    assert np.abs(FH - st["FH"]).max() <= 1e-12 * np.abs(st["FH"]).max()
+    g = st["face_nodes"]
+    for ax in range(3):
+        on = g[:, ax] % n == 0
+        u, v = (g[on, e] for e in range(3) if e != ax)
+        assert np.abs(B[ax, g[on, ax] // n, u, v] - st["phiB"][on]).max() <= 1e-12 * np.abs(st["phiB"]).max()
