@@ -165,6 +165,8 @@ cudaError_t batch_enqueue(const std::vector<mlc_plan_t> &plans, const BatchLayou
     for (int g = 0; g < G; ++g) {
         const BatchLayout::Group &gr = L.groups[g];
         Items it{d_items + gr.item0, d_recs, gr.nitems};
+        it.a1 = gr.a1;
+        it.cap = gr.cap;
         for (int b = 0; b < nb; ++b) TRYE(cudaStreamWaitEvent(S.conv[g], ev_br(b), 0));
         TRYE(launch_dirichlet(gr.rep, it, S.conv[g]));
         TRYE(cudaEventRecord(ev_dir(g), S.conv[g]));

@@ -116,6 +116,19 @@ __device__ __forceinline__ uint4 digit_chunk(const unsigned long long (&Y)[8], i
     return r;
 }
 __device__ __forceinline__ int biased_exp(double x) { return (int)((__double_as_longlong(x) >> 52) & 0x7ff); }
+// Even and odd parts (bit d of the index: odd along axis d) to the values at the
+// mirror images (bit d: mirrored along axis d), and, up to a factor 8, back.
+__device__ __forceinline__ void unfold8(double (&v)[8]) {
+#pragma unroll
+    for (int b = 1; b < 8; b <<= 1)
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            if (!(i & b)) {
+                const double x = v[i], y = v[i | b];
+                v[i] = x + y;
+                v[i | b] = x - y;
+            }
+}
 // Row factor of a table row whose largest magnitude has biased exponent e: an entry is
 // X 2^(e - 1022 - 55), and sums of X Y come divided by 2^48.
 __device__ __forceinline__ double limb_row_factor(int e) { return e ? ldexp(1.0, e - 1022 - 2 * kLimbBias + 48) : 0.0; }
@@ -239,6 +252,21 @@ cudaError_t limb_conv_tables(int device, const Geom &g, bool share, const double
                              std::shared_ptr<LimbConvTables> *out);
 inline long limb_ctiles(long items) { return (items + kLimbN - 1) / kLimbN; }
 void configure_limb_conv();
+// Columns per launch group: as many as `cap` bytes of scratch hold (per 64
+// columns tile_bytes, per column item_bytes), in groups of one size; 0 if none.
+inline long limb_group(size_t cap, long items, size_t tile_bytes, size_t item_bytes) {
+    long m = 0;
+    for (long ct = limb_ctiles(items); ct > 0 && m == 0; --ct) {
+        if (ct * tile_bytes >= cap) continue;
+        long fit = (long)((cap - ct * tile_bytes) / item_bytes);
+        fit = fit < ct * kLimbN ? fit : ct * kLimbN;
+        fit = fit < items ? fit : items;
+        if (fit > (ct - 1) * kLimbN) m = fit;
+    }
+    if (m <= 0) return 0;
+    const long groups = (items + m - 1) / m, even = limb_ctiles((items + groups - 1) / groups) * kLimbN;
+    return m < even ? m : even;
+}
 
 // ---- ring products (limb_ring.cu) -------------------------------------------
 // Buffers and layout of one plan's ring products: parts 0..2 the face nodes of

@@ -227,19 +227,6 @@ template <> __device__ __forceinline__ float2 limb_out<float2>(double v) {
     return make_float2(hi, (float)(v - (double)hi));
 }
 
-// Values at the mirror images: bit d of the index set: axis d mirrored.
-__device__ __forceinline__ void unfold8(double (&v)[8]) {
-#pragma unroll
-    for (int b = 1; b < 8; b <<= 1)
-#pragma unroll
-        for (int i = 0; i < 8; ++i)
-            if (!(i & b)) {
-                const double x = v[i], y = v[i | b];
-                v[i] = x + y;
-                v[i | b] = x - y;
-            }
-}
-
 template <typename TO, bool SHARE>
 __global__ void __launch_bounds__(256) k_limb_unfold(const __grid_constant__ UnfoldArgs a) {
     int p;
@@ -414,19 +401,6 @@ void configure_limb_conv() {
     cudaFuncSetAttribute(k_limb_fold, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
 }
 
-// Patches per launch group: as many as the scratch holds, in groups of one size.
-static long limb_group(const Geom &g, size_t cap, long items) {
-    long m = 0;
-    for (long ct = limb_ctiles(items); ct > 0 && m == 0; --ct) {
-        if (ct * g.limb_tile_bytes >= cap) continue;
-        const long fit = std::min({items, ct * kLimbN, (long)((cap - ct * g.limb_tile_bytes) / g.limb_item_bytes)});
-        if (fit > (ct - 1) * kLimbN) m = fit;
-    }
-    if (m <= 0) return 0;
-    const long groups = (items + m - 1) / m, even = (items + groups - 1) / groups;
-    return std::min(m, limb_ctiles(even) * kLimbN);
-}
-
 // Local convolutions of one launch group: three launches.
 static cudaError_t limb_conv_group(const mlc_plan_s *pl, const Items &it, cudaStream_t st) {
     NvtxRange nvtx("mlc:local_convolutions");
@@ -484,7 +458,7 @@ static cudaError_t limb_conv_group(const mlc_plan_s *pl, const Items &it, cudaSt
 }
 
 cudaError_t launch_limb_conv(const mlc_plan_s *pl, const Items &it, cudaStream_t st) {
-    const long group = limb_group(pl->g, it.cap, it.nitems);
+    const long group = limb_group(it.cap, it.nitems, pl->g.limb_tile_bytes, pl->g.limb_item_bytes);
     if (group <= 0) return cudaErrorInvalidValue;
     for (long c0 = 0; c0 < it.nitems; c0 += group) {
         Items ic = it;

@@ -100,6 +100,7 @@ struct Geom {
     size_t scr_a1, scr_a4;           // scratch bytes per patch: x-transformed charges, slab outputs
     // FP64 and double-float tiers: scratch of the exact-split products (limb.h)
     size_t limb_tile_bytes, limb_item_bytes;  // per 64 patches: digits and factors; per patch: products
+    size_t wide_tile_bytes, wide_item_bytes;  // Q = 10: the same of the Dirichlet step's layer operator
 };
 // Local-convolution scratch for `items` patches: the a1 part, then (from a
 // 256-byte boundary) the a4 part.
@@ -112,9 +113,9 @@ inline size_t conv_scratch_a4_offset(const Geom &g, long items) {
 // patches, whose columns fill a tile of 64, can need more.
 inline size_t conv_scratch_bytes(const Geom &g, long items) {
     const size_t fft = conv_scratch_a4_offset(g, items) + (size_t)items * g.scr_a4;
-    if (g.conv == CONV_F32) return fft;
     const size_t limb = (size_t)limb_ctiles(items) * g.limb_tile_bytes + (size_t)items * g.limb_item_bytes;
-    return limb > fft ? limb : fft;
+    const size_t wide = (size_t)limb_ctiles(items) * g.wide_tile_bytes + (size_t)items * g.wide_item_bytes;
+    return limb > fft ? (wide > limb ? wide : limb) : (wide > fft ? wide : fft);
 }
 
 // Per-plan pointers and sizes read by the per-patch kernels.  A single solve
@@ -137,7 +138,8 @@ struct PlanPtrs {
     int N, np;
     double c2h2, inv_h2;  // h^2 / 12, 1 / h^2
     double h2;            // h^2
-    void *dscr;           // Dirichlet workspace (n > 24): [patch][(n-1)^3] in the fine precision
+    void *dscr;           // Dirichlet workspace (n > 24: [patch][(n-1)^3] in the fine precision; Q = 10:
+                          // [patch][1 or, n > 16, 2][(n-1)^3] FP64)
     int *err;             // the plan's error word
     // Q = 10 (R18): local fields and residuals on the planes one node off the
     // alpha face planes, [patch][axis][j][side][u][v] (side 0: plane - 1,
@@ -159,7 +161,7 @@ struct Items {
     int chunk = 0;        // items per local-convolution launch group (0: the plan's conv_chunk)
     void *a1 = nullptr;   // scratch: x-transformed charges, scr_a1 bytes per item
     void *a4 = nullptr;   // scratch: slab outputs, scr_a4 bytes per item
-    size_t cap = 0;       // scratch bytes from a1 on (FP64 and double-float tiers)
+    size_t cap = 0;       // scratch bytes from a1 on
 };
 
 #ifdef __CUDACC__
@@ -223,7 +225,7 @@ struct mlc_plan_s {
     double *tpl;             // 3 (np+1) no (N+1): I^H(phi^H) summed along v per plane and coarse row
     float *ring_aimg;        // split tiers: ring table as the tensor-core GEMM operand (TF32 hi/lo image)
     float *ring_R;           // split tiers: [patch][ring_rows_pad] ring terms of one face-plane axis
-    void *dscr = nullptr;    // n > 24: Dirichlet workspace [patch][(n-1)^3] (fine precision)
+    void *dscr = nullptr;    // n > 24 or Q = 10: Dirichlet workspace (PlanPtrs::dscr)
     // Q = 10 (R18): the second boundary layer
     void *fp2 = nullptr;     // NP x 3 npa 2 x wa^2 local fields one node off the alpha face planes
     double *resid2 = nullptr;  // NP x 3 npa 2 x wa^2 their residuals (FP64)
@@ -233,6 +235,8 @@ struct mlc_plan_s {
     void *f_stage, *phi_stage;  // device staging for mlc_solve_host
     std::shared_ptr<mlc::LimbConvTables> limb_tabs;  // FP64 and double-float tiers: folded Green's function
     std::shared_ptr<mlc::LimbRing> limb_ring;        // and ring products (null: no ring, or per-node sums)
+    const unsigned char *wide_A = nullptr;  // Q = 10: the layer operator (shared, wide.cuh)
+    const double *wide_rf = nullptr;
     int *err;                // device error word: nonzero if a bounded wait in a kernel gave up
     size_t ws_bytes;
     std::vector<void *> owned;  // device allocations to free
@@ -291,6 +295,8 @@ cudaError_t launch_boundary(const mlc_plan_s *pl, cudaStream_t st);
 cudaError_t launch_resid_outer(const mlc_plan_s *pl, const Items &it, cudaStream_t st);
 cudaError_t launch_boundary_outer(const mlc_plan_s *pl, cudaStream_t st);
 cudaError_t launch_dirichlet_wide(const mlc_plan_s *pl, const Items &it, cudaStream_t st);
+cudaError_t wide_tables(int device, int n, const double *sinm, const unsigned char **A, const double **rf);
+void wide_scratch(int n, size_t *tile_bytes, size_t *item_bytes);
 void configure_wide();
 // Lagrange weights of I^H (R4) for g mod 4 = r, row r, 2b+2 <= 12 entries.
 void lagrange_rows(int b, double lw[4][12]);

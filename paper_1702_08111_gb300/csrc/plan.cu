@@ -279,6 +279,7 @@ mlc_status derive_geometry(const mlc_params &pp, Geom &g) {
         g.limb_tile_bytes = (size_t)lc.b_total + 8 * kLimbN * sizeof(double);
         g.limb_item_bytes = (size_t)lc.v_total * sizeof(double);
     }
+    if (g.wide) wide_scratch(g.n, &g.wide_tile_bytes, &g.wide_item_bytes);
     g.wbx = g.n + 2 * g.gb + 1;
     g.plane_n = (g.N + 1) * (g.N + 1);
     g.n_planes_total = 3L * (g.np + 1) * (long)g.plane_n;
@@ -840,11 +841,13 @@ mlc_status create_plan(const mlc_params *params, const double *dgf_host, int dgf
             TRY(dev_alloc(pl, &pl->phiB2, 2 * (size_t)G.n_planes_total));
             TRY(dev_alloc(pl, &pl->tpl2, 6 * (size_t)(G.np + 1) * G.no * (G.N + 1)));
         }
-        if (G.n > 24 || (G.wide && G.n > 16)) {  // Dirichlet workspace of patches too large for shared memory
-            double *d = nullptr;                     // (Q = 10: right-hand side, iterate and work array)
-            TRY(dev_alloc(pl, &d, NP * (G.wide ? 3 : 1) * (size_t)(G.n - 1) * (G.n - 1) * (G.n - 1)));
+        if (G.n > 24 || G.wide) {  // Dirichlet workspace of patches too large for shared memory
+            double *d = nullptr;       // (Q = 10: right-hand side and, above n = 16, work array)
+            TRY(dev_alloc(pl, &d, NP * (G.wide && G.n > 16 ? 2 : 1) * (size_t)(G.n - 1) * (G.n - 1) * (G.n - 1)));
             pl->dscr = d;
         }
+        if (G.wide)
+            TRY_CUDA(wide_tables(pl->device, G.n, (const double *)pl->sinm, &pl->wide_A, &pl->wide_rf));
         TRY(dev_alloc(pl, &pl->err, 1, false));
         TRY_CUDA(cudaMemset(pl->err, 0, sizeof(int)));
         return MLC_OK;

@@ -213,47 +213,175 @@ __global__ void __launch_bounds__(128) k_boundary_outer(BndOutArgs a) {
 // stencil with the odd continuation across the faces (diagonal in DST-I), and
 // E u(g) = sum over the offsets that leave the layer next to a face through
 // it of a_s u(mirror(g + s)) (L reads zero there, L_odd minus the mirrored
-// value).  u_0 = L_odd^-1 b, u_{k+1} = L_odd^-1 (b - E u_k).  One CTA per
-// patch; b, u and the work array in shared memory up to n = 16, in the
-// plan's workspace above; each DST pass gives a line of m = n-1 values to one
-// thread (n = 16: the split-radix 15-point DST; n = 32: the split 31-point
-// DST; other n: dense m x m sums with the matrix in shared memory).
+// value).  E reads and writes only the layers next to the faces, so the solution
+// is u = L_odd^-1 (b - w) with w on those layers,
+//   w = S t,  t = E L_odd^-1 b,  S = (1 + E L_odd^-1)^-1 restricted to them:
+// two DST-I solves around one fixed linear map, where iterating on E takes
+// eleven solves to FP64 accuracy (256^3, n = 32: 28.2 -> 8.0 ms for 512
+// patches).  S is 5402 x 5402 at n = 32; folded by parity along the axes it is
+// eight blocks of about 690, the same for every h, applied to all patches as an
+// exact-split product (limb.h):
+//   k_wide_first   b, L_odd^-1 b, t folded to digits
+//   k_limb_gemm    w, folded
+//   k_wide_last    L_odd^-1 (b - w), phi
+// One CTA per patch; the work array in shared memory up to n = 16, in the plan's
+// workspace (L2) above, b always there; each DST pass gives a line of m = n-1
+// values to one thread (n = 16: the split-radix 15-point DST; n = 32: the split
+// 31-point DST; other n: dense m x m sums with the matrix in shared memory).
+// Bound by the FP64 pipe in the DST passes.
+
+// Layer nodes of one parity block: reps (i0, i1, i2), i_d < d_d, at least one
+// of them 0 (the node next to the low face), numbered by the first axis that is.
+__host__ __device__ inline int surf_count(int d0, int d1, int d2) { return d0 * d1 * d2 - (d0 - 1) * (d1 - 1) * (d2 - 1); }
+__host__ __device__ inline int surf_index(int d0, int d1, int d2, int i0, int i1, int i2) {
+    if (i0 == 0) return i1 * d2 + i2;
+    if (i1 == 0) return d1 * d2 + (i0 - 1) * d2 + i2;
+    return d1 * d2 + (d0 - 1) * d2 + (i0 - 1) * (d1 - 1) + (i1 - 1);
+}
+__host__ __device__ inline void surf_rep(int d0, int d1, int d2, int k, int i[3]) {
+    if (k < d1 * d2) { i[0] = 0; i[1] = k / d2; i[2] = k % d2; return; }
+    k -= d1 * d2;
+    if (k < (d0 - 1) * d2) { i[0] = 1 + k / d2; i[1] = 0; i[2] = k % d2; return; }
+    k -= (d0 - 1) * d2;
+    i[0] = 1 + k / (d1 - 1); i[1] = 1 + k % (d1 - 1); i[2] = 0;
+}
+
+// E u at the layer node (q0, q1, q2) of the interior (1..m): the offsets that
+// leave through a face are (-+2, 0, 0) and (-+2, +-1, 0), (-+2, 0, +-1) along its
+// normal; their mirror images lie in the same layer, at the node itself and its
+// four in-layer neighbours (zero on the faces).
+template <int m>
+__device__ __forceinline__ double wide_E(const double *U, int q0, int q1, int q2, double e200, double e210) {
+    auto at = [&](int a, int b, int c) -> double {
+        return (a < 1 || a > m || b < 1 || b > m || c < 1 || c > m) ? 0.0 : U[((a - 1) * m + (b - 1)) * m + (c - 1)];
+    };
+    double r = 0.0;
+    const double u = at(q0, q1, q2);
+    const double s0 = at(q0 - 1, q1, q2) + at(q0 + 1, q1, q2), s1 = at(q0, q1 - 1, q2) + at(q0, q1 + 1, q2),
+                 s2 = at(q0, q1, q2 - 1) + at(q0, q1, q2 + 1);
+    if (q0 == 1 || q0 == m) r = fma(e200, u, fma(e210, s1 + s2, r));
+    if (q1 == 1 || q1 == m) r = fma(e200, u, fma(e210, s0 + s2, r));
+    if (q2 == 1 || q2 == m) r = fma(e200, u, fma(e210, s0 + s1, r));
+    return r;
+}
+
+// X <- L_odd^-1 X: three DST-I passes, the eigenvalue scaling (lam holds
+// (2/n)^3 h^2 / lambda), three more passes.  S: dense DST-I matrix (other n).
+template <int NN>
+__device__ void wide_solve(double *X, const double *S, const double *lam, const double *sinm) {
+    constexpr int m = NN - 1;
+    double sv16[9];  // n = 16: sin(pi i / 16), i = 0..8
+    sv16[0] = 0.0;
+#pragma unroll
+    for (int i = 1; i <= 8; ++i) sv16[i] = NN == 16 ? sinm[i - 1] : 0.0;
+    double sv32[17];  // n = 32: sin(pi i / 32), i = 0..16
+    sv32[0] = 0.0;
+#pragma unroll
+    for (int i = 1; i <= 16; ++i) sv32[i] = NN == 32 ? sinm[i - 1] : 0.0;
+#pragma unroll 1
+    for (int pass = 0; pass < 6; ++pass) {
+        const int axis = 2 - (pass % 3);
+        for (int l = threadIdx.x; l < m * m; l += blockDim.x) {
+            const int qa = l / m, qb = l % m;
+            int base, str;
+            if (axis == 2) { base = (qa * m + qb) * m; str = 1; }
+            else if (axis == 1) { base = qa * m * m + qb; str = m; }
+            else { base = qa * m + qb; str = m * m; }
+            double x[m];
+#pragma unroll
+            for (int t = 0; t < m; ++t) x[t] = X[base + t * str];
+            if constexpr (NN == 16 || NN == 32) {  // the split-radix 15-point / split 31-point DST-I
+                if constexpr (NN == 16) dst15_fast(x, sv16);
+                else dst31_fast(x, sv32);
+#pragma unroll
+                for (int k = 0; k < m; ++k) X[base + k * str] = pass == 2 ? x[k] * lam[base + k * str] : x[k];
+            } else {
+#pragma unroll
+                for (int k = 0; k < m; ++k) {
+                    double acc = 0.0;
+#pragma unroll
+                    for (int t = 0; t < m; ++t) acc = fma(S[k * m + t], x[t], acc);
+                    if (pass == 2) acc *= lam[base + k * str];
+                    X[base + k * str] = acc;
+                }
+            }
+        }
+        __syncthreads();
+    }
+}
+template <int NN>
+__device__ __forceinline__ void wide_dense_dst(double *S, const double *sinm) {
+    constexpr int n = NN, m = n - 1, h = n / 2;
+    for (int e = threadIdx.x; e < m * m && NN != 16 && NN != 32; e += blockDim.x) {
+        const int k = e / m, T = e % m + 1;
+        // sin(pi K (n - T') / n) = (-1)^(K+1) sin(pi K T' / n), K = k + 1
+        S[e] = T <= h ? sinm[k * h + (T - 1)] : ((k & 1) ? -1.0 : 1.0) * sinm[k * h + (n - T - 1)];
+    }
+}
+
+// Folded layer operator of a patch size: reps per axis (even, odd) and, per
+// parity class or its table (limb.h), sizes and offsets.
+struct WideGeom {
+    int d[2];
+    int K[8], kst[8], tiles[8];     // per table
+    long a_off[8], rf_off[8], a_bytes, rf_rows;
+    long b_step[8], v_step[8], b_total, v_total;  // per class
+};
+inline WideGeom wide_geometry(int n) {
+    WideGeom g{};
+    g.d[0] = n / 2;       // interior 1..n-1: the centre n/2 included
+    g.d[1] = n / 2 - 1;
+    for (int c = 0; c < 8; ++c) {
+        const int u = limb_table(true, c);
+        if (u == c) {
+            g.K[u] = surf_count(g.d[limb_odd(u, 0)], g.d[limb_odd(u, 1)], g.d[limb_odd(u, 2)]);
+            g.kst[u] = (g.K[u] + 15) / 16;
+            g.tiles[u] = (g.K[u] + kLimbM - 1) / kLimbM;
+            g.a_off[u] = g.a_bytes;
+            g.rf_off[u] = g.rf_rows;
+            g.a_bytes += (long)g.tiles[u] * g.kst[u] * kLimbAStep;
+            g.rf_rows += (long)g.tiles[u] * kLimbM;
+        }
+    }
+    for (int c = 0; c < 8; ++c) {
+        const int u = limb_table(true, c);
+        g.b_step[c] = g.b_total;
+        g.v_step[c] = g.v_total;
+        g.b_total += (long)g.kst[u] * kLimbBStep;
+        g.v_total += g.K[u];
+    }
+    return g;
+}
+
 struct DirWArgs {
     Items it;
     const double *sinm;  // (n-1) x n/2 half DST-I matrix sin(pi k t / n), t in [1, n/2]
-    int iters;           // fixed-point steps after the first solve
+    WideGeom g;
+    unsigned char *Bd;   // digits of t, [class][column tile][k-step]...
+    double *cf;          // [class][cols_pad]
+    const double *V;     // w, [class][column][layer rep]
+    int cols, ctiles;
 };
 
 template <typename TF, int NN>
-__global__ void __launch_bounds__(256) k_dirichlet_wide(DirWArgs a) {
-    constexpr int n = NN, m = n - 1, m3 = m * m * m, h = n / 2;
-    constexpr bool BIG = NN > 16;  // the three arrays in the plan's global workspace (L2-resident)
+__global__ void __launch_bounds__(256) k_wide_first(const __grid_constant__ DirWArgs a) {
+    constexpr int n = NN, m = n - 1, m3 = m * m * m;
+    constexpr bool BIG = NN > 16;  // the work array in the plan's workspace (L2-resident)
     extern __shared__ double smw[];
+    __shared__ int smax[8];
     int p;
     const PlanPtrs &PP = item_plan(a.it, blockIdx.x, p);
-    double *B, *U, *X, *S;  // right-hand side, current iterate, transform work array, DST-I matrix
-    if constexpr (BIG) {
-        B = (double *)PP.dscr + (long)p * 3 * m3;
-        U = B + m3;
-        X = U + m3;
-        S = smw;
-    } else {
-        B = smw;
-        U = B + m3;
-        X = U + m3;
-        S = X + m3;
-    }
+    double *B = (double *)PP.dscr + (long)p * (BIG ? 2 : 1) * m3;
+    double *X = BIG ? B + m3 : smw;
+    double *S = BIG ? smw : smw + m3;           // dense DST-I matrix
+    double *FV = S + (NN == 16 || NN == 32 ? 0 : m * m);  // folded t, class after class
     const int N = PP.N, np = PP.np;
     const int i0 = p / (np * np), i1 = (p / np) % np, i2 = p % np;
     const int o0 = i0 * n, o1 = i1 * n, o2 = i2 * n;
     const TF *f = (const TF *)PP.f;
     const double ih2 = PP.inv_h2;
-    const double *lam = (const double *)PP.lam;
-    for (int e = threadIdx.x; e < m * m && NN != 16 && NN != 32; e += blockDim.x) {  // dense lines only
-        const int k = e / m, T = e % m + 1;
-        // sin(pi K (n - T') / n) = (-1)^(K+1) sin(pi K T' / n), K = k + 1
-        S[e] = T <= h ? a.sinm[k * h + (T - 1)] : ((k & 1) ? -1.0 : 1.0) * a.sinm[k * h + (n - T - 1)];
-    }
+    wide_dense_dst<NN>(S, a.sinm);
+    if (threadIdx.x < 8) smax[threadIdx.x] = 0;
     // boundary value at the relative node q (a face node, or one coordinate -1 or n+1)
     auto bval = [&](int q0, int q1, int q2) -> double {
         const int G[3] = {o0 + q0, o1 + q1, o2 + q2}, q[3] = {q0, q1, q2}, ip[3] = {i0, i1, i2};
@@ -282,96 +410,199 @@ __global__ void __launch_bounds__(256) k_dirichlet_wide(DirWArgs a) {
                         if (c == 0.0) continue;
                         const int t0 = q0 + s0, t1 = q1 + s1, t2 = q2 + s2;
                         if (t0 >= 1 && t0 <= m && t1 >= 1 && t1 <= m && t2 >= 1 && t2 <= m) continue;
-                        r -= c * ih2 * bval(t0, t1, t2);
+                        r = fma(-c * ih2, bval(t0, t1, t2), r);
                     }
         }
         B[e] = r;
+        X[e] = r;
     }
     __syncthreads();
-    // X <- L_odd^-1 X: three DST-I passes, the eigenvalue scaling (lam holds
-    // (2/n)^3 h^2 / lambda), three more passes
-    double sv16[9];  // n = 16: sin(pi i / 16), i = 0..8
-    sv16[0] = 0.0;
+    wide_solve<NN>(X, S, (const double *)PP.lam, a.sinm);
+    // t = E X at the mirror images of each layer rep, folded
+    const double e200 = stencil_coef(10, 2, 0, 0) * ih2, e210 = stencil_coef(10, 2, 1, 0) * ih2;
+    const int d = a.g.d[0], cen = d - 1;
+    int mx[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    for (int k = threadIdx.x; k < surf_count(d, d, d); k += blockDim.x) {
+        int i[3];
+        surf_rep(d, d, d, k, i);
+        double v[8];
 #pragma unroll
-    for (int i = 1; i <= 8; ++i) sv16[i] = NN == 16 ? a.sinm[i - 1] : 0.0;
-    double sv32[17];  // n = 32: sin(pi i / 32), i = 0..16
-    sv32[0] = 0.0;
-#pragma unroll
-    for (int i = 1; i <= 16; ++i) sv32[i] = NN == 32 ? a.sinm[i - 1] : 0.0;
-    auto solve = [&]() {
-        for (int pass = 0; pass < 6; ++pass) {
-            const int axis = 2 - (pass % 3);
-            for (int l = threadIdx.x; l < m * m; l += blockDim.x) {
-                const int qa = l / m, qb = l % m;
-                int base, str;
-                if (axis == 2) { base = (qa * m + qb) * m; str = 1; }
-                else if (axis == 1) { base = qa * m * m + qb; str = m; }
-                else { base = qa * m + qb; str = m * m; }
-                double x[m];
-#pragma unroll
-                for (int t = 0; t < m; ++t) x[t] = X[base + t * str];
-                if constexpr (NN == 16 || NN == 32) {  // the split-radix 15-point / split 31-point DST-I
-                    if constexpr (NN == 16) dst15_fast(x, sv16);
-                    else dst31_fast(x, sv32);
-#pragma unroll
-                    for (int k = 0; k < m; ++k) X[base + k * str] = pass == 2 ? x[k] * lam[base + k * str] : x[k];
-                } else {
-#pragma unroll
-                    for (int k = 0; k < m; ++k) {
-                        double acc = 0.0;
-#pragma unroll
-                        for (int t = 0; t < m; ++t) acc = fma(S[k * m + t], x[t], acc);
-                        if (pass == 2) acc *= lam[base + k * str];
-                        X[base + k * str] = acc;
-                    }
-                }
-            }
-            __syncthreads();
+        for (int b = 0; b < 8; ++b) {
+            const bool dup = ((b & 1) && i[0] == cen) || ((b & 2) && i[1] == cen) || ((b & 4) && i[2] == cen);
+            v[b] = dup ? 0.0
+                       : wide_E<m>(X, (b & 1) ? m - i[0] : 1 + i[0], (b & 2) ? m - i[1] : 1 + i[1],
+                                   (b & 4) ? m - i[2] : 1 + i[2], e200, e210);
         }
-    };
+        unfold8(v);  // sums and differences along each axis
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+            if ((limb_odd(c, 0) && i[0] == cen) || (limb_odd(c, 1) && i[1] == cen) || (limb_odd(c, 2) && i[2] == cen)) continue;
+            const int b = (limb_odd(c, 0) ? 1 : 0) | (limb_odd(c, 1) ? 2 : 0) | (limb_odd(c, 2) ? 4 : 0);
+            const int u = limb_table(true, c);
+            FV[a.g.v_step[c] + surf_index(a.g.d[limb_odd(u, 0)], a.g.d[limb_odd(u, 1)], a.g.d[limb_odd(u, 2)],
+                                          i[limb_perm(true, c, 0)], i[limb_perm(true, c, 1)], i[limb_perm(true, c, 2)])] = v[b];
+            mx[c] = max(mx[c], biased_exp(v[b]));
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+        const int v = __reduce_max_sync(0xffffffffu, mx[c]);
+        if ((threadIdx.x & 31) == 0 && v) atomicMax(&smax[c], v);
+    }
+    __syncthreads();
+    const int col = blockIdx.x, ct = col / kLimbN, cl = col % kLimbN;
+    for (int c = 0; c < 8; ++c) {
+        const int u = limb_table(true, c), e = smax[c], K = a.g.K[u];
+        const bool live = e != 0 && e != 0x7ff;
+        if (threadIdx.x == 0)
+            a.cf[(long)c * a.ctiles * kLimbN + col] =
+                e == 0x7ff ? __longlong_as_double(0x7ff8000000000000ll) : (live ? ldexp(1.0, e - 1022) : 0.0);
+        unsigned char *Bt = a.Bd + a.g.b_step[c] * a.ctiles + (long)ct * a.g.kst[u] * kLimbBStep;
+        for (int w = threadIdx.x; w < a.g.kst[u] * 2; w += blockDim.x) {
+            unsigned long long Y[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+                Y[j] = digit_bytes(live && 8 * w + j < K ? to_limb_int(FV[a.g.v_step[c] + 8 * w + j], e) : 0);
+            unsigned char *o = Bt + limb_chunk_off(cl, w, kLimbBBlk);
+#pragma unroll
+            for (int i = 0; i < kLimbs; ++i) *(uint4 *)(o + i * kLimbBBlk) = digit_chunk(Y, i);
+        }
+    }
+}
+
+template <typename TF, int NN>
+__global__ void __launch_bounds__(256) k_wide_last(const __grid_constant__ DirWArgs a) {
+    constexpr int n = NN, m = n - 1, m3 = m * m * m;
+    constexpr bool BIG = NN > 16;
+    extern __shared__ double smw[];
+    int p;
+    const PlanPtrs &PP = item_plan(a.it, blockIdx.x, p);
+    const double *B = (const double *)PP.dscr + (long)p * (BIG ? 2 : 1) * m3;
+    double *X = BIG ? (double *)PP.dscr + (long)p * 2 * m3 + m3 : smw;
+    double *S = BIG ? smw : smw + m3;
+    const int N = PP.N, np = PP.np;
+    const int o0 = p / (np * np) * n, o1 = (p / np) % np * n, o2 = p % np * n;
+    const TF *f = (const TF *)PP.f;
+    wide_dense_dst<NN>(S, a.sinm);
     for (int e = threadIdx.x; e < m3; e += blockDim.x) X[e] = B[e];
     __syncthreads();
-    solve();
-    for (int e = threadIdx.x; e < m3; e += blockDim.x) U[e] = X[e];
-    __syncthreads();
-    // E u on the layer next to a face: the offsets that leave the interior
-    // through the face are (-+2, 0, 0) and (-+2, +-1, 0), (-+2, 0, +-1) along
-    // its normal; their mirror images lie in the same layer, at the node
-    // itself and its four in-layer neighbours (zero on the faces)
-    const double e200 = stencil_coef(10, 2, 0, 0) * ih2, e210 = stencil_coef(10, 2, 1, 0) * ih2;
-    auto Uin = [&](int q0, int q1, int q2) -> double {
-        return (q0 < 1 || q0 > m || q1 < 1 || q1 > m || q2 < 1 || q2 > m) ? 0.0
-                                                                         : U[((q0 - 1) * m + (q1 - 1)) * m + (q2 - 1)];
-    };
-    for (int it = 0; it < a.iters; ++it) {
-        for (int e = threadIdx.x; e < m3; e += blockDim.x) {
-            const int q2 = e % m + 1, q1 = (e / m) % m + 1, q0 = e / (m * m) + 1;
-            double r = B[e];
-            if (q0 == 1 || q0 == m)
-                r -= e200 * U[e] + e210 * (Uin(q0, q1 - 1, q2) + Uin(q0, q1 + 1, q2) + Uin(q0, q1, q2 - 1) +
-                                           Uin(q0, q1, q2 + 1));
-            if (q1 == 1 || q1 == m)
-                r -= e200 * U[e] + e210 * (Uin(q0 - 1, q1, q2) + Uin(q0 + 1, q1, q2) + Uin(q0, q1, q2 - 1) +
-                                           Uin(q0, q1, q2 + 1));
-            if (q2 == 1 || q2 == m)
-                r -= e200 * U[e] + e210 * (Uin(q0 - 1, q1, q2) + Uin(q0 + 1, q1, q2) + Uin(q0, q1 - 1, q2) +
-                                           Uin(q0, q1 + 1, q2));
-        X[e] = r;
+    const int d = a.g.d[0], cen = d - 1;
+    for (int k = threadIdx.x; k < surf_count(d, d, d); k += blockDim.x) {
+        int i[3];
+        surf_rep(d, d, d, k, i);
+        double v[8];
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+            const bool zero = (limb_odd(c, 0) && i[0] == cen) || (limb_odd(c, 1) && i[1] == cen) || (limb_odd(c, 2) && i[2] == cen);
+            const int b = (limb_odd(c, 0) ? 1 : 0) | (limb_odd(c, 1) ? 2 : 0) | (limb_odd(c, 2) ? 4 : 0);
+            const int u = limb_table(true, c);
+            v[b] = zero ? 0.0
+                        : a.V[a.g.v_step[c] * a.cols + (long)blockIdx.x * a.g.K[u] +
+                              surf_index(a.g.d[limb_odd(u, 0)], a.g.d[limb_odd(u, 1)], a.g.d[limb_odd(u, 2)],
+                                         i[limb_perm(true, c, 0)], i[limb_perm(true, c, 1)], i[limb_perm(true, c, 2)])];
         }
-        __syncthreads();
-        solve();
-        for (int e = threadIdx.x; e < m3; e += blockDim.x) U[e] = X[e];
-        __syncthreads();
+        unfold8(v);
+#pragma unroll
+        for (int b = 0; b < 8; ++b) {
+            if (((b & 1) && i[0] == cen) || ((b & 2) && i[1] == cen) || ((b & 4) && i[2] == cen)) continue;
+            const int q0 = (b & 1) ? m - i[0] : 1 + i[0], q1 = (b & 2) ? m - i[1] : 1 + i[1], q2 = (b & 4) ? m - i[2] : 1 + i[2];
+            X[((q0 - 1) * m + (q1 - 1)) * m + (q2 - 1)] -= v[b];
+        }
     }
+    __syncthreads();
+    wide_solve<NN>(X, S, (const double *)PP.lam, a.sinm);
     const double c2h2 = PP.c2h2;
     for (int e = threadIdx.x; e < n * n * n; e += blockDim.x) {
         const int m2 = e % n, m1 = (e / n) % n, m0 = e / (n * n);
         const bool bnd = m0 == 0 || m1 == 0 || m2 == 0;
         const int z = o0 + m0, y = o1 + m1, x = o2 + m2;
         const long gi = ((long)z * N + y) * N + x;
-        const double u = bnd ? phiB_at<double>(PP, n, z, y, x) : U[((m0 - 1) * m + (m1 - 1)) * m + (m2 - 1)];
-        PP.phi[gi] = u + c2h2 * (double)f[gi];
+        const double u = bnd ? phiB_at<double>(PP, n, z, y, x) : X[((m0 - 1) * m + (m1 - 1)) * m + (m2 - 1)];
+        PP.phi[gi] = fma(c2h2, (double)f[gi], u);
     }
+}
+
+// ---- the layer operator S of a patch size (plan time) ------------------------
+// Column j of (1 + E L_odd^-1) of one table: the parity-symmetric field of rep j
+// with amplitude 1, solved, E of it read at the reps.
+template <int NN>
+__global__ void __launch_bounds__(256) k_wide_columns(int u, WideGeom g, const double *lam, const double *sinm,
+                                                      double *work, int j0, double *M) {
+    constexpr int n = NN, m = n - 1, m3 = m * m * m;
+    extern __shared__ double smw[];
+    double *X = work + (long)blockIdx.x * m3, *S = smw;
+    const int j = j0 + blockIdx.x, K = g.K[u];
+    const int d0 = g.d[limb_odd(u, 0)], d1 = g.d[limb_odd(u, 1)], d2 = g.d[limb_odd(u, 2)], cen = g.d[0] - 1;
+    wide_dense_dst<NN>(S, sinm);
+    for (int e = threadIdx.x; e < m3; e += blockDim.x) X[e] = 0.0;
+    __syncthreads();
+    if (threadIdx.x < 8) {
+        int i[3];
+        surf_rep(d0, d1, d2, j, i);
+        const int b = threadIdx.x;
+        if (!(((b & 1) && i[0] == cen) || ((b & 2) && i[1] == cen) || ((b & 4) && i[2] == cen))) {
+            const int q0 = (b & 1) ? m - i[0] : 1 + i[0], q1 = (b & 2) ? m - i[1] : 1 + i[1], q2 = (b & 4) ? m - i[2] : 1 + i[2];
+            const bool neg = ((b & 1) && limb_odd(u, 0)) ^ ((b & 2) && limb_odd(u, 1)) ^ ((b & 4) && limb_odd(u, 2));
+            X[((q0 - 1) * m + (q1 - 1)) * m + (q2 - 1)] = neg ? -1.0 : 1.0;
+        }
+    }
+    __syncthreads();
+    wide_solve<NN>(X, S, lam, sinm);
+    const double e200 = stencil_coef(10, 2, 0, 0), e210 = stencil_coef(10, 2, 1, 0);
+    for (int r = threadIdx.x; r < K; r += blockDim.x) {
+        int i[3];
+        surf_rep(d0, d1, d2, r, i);
+        M[(long)r * K + j] = (r == j ? 1.0 : 0.0) + wide_E<m>(X, 1 + i[0], 1 + i[1], 1 + i[2], e200, e210);
+    }
+}
+// One step of the in-place Gauss-Jordan inverse (1 + E L_odd^-1 is close to 1:
+// its spectrum lies within 0.03 of it, so no pivoting), from A to B.
+__global__ void __launch_bounds__(256) k_wide_invert(const double *A, double *B, int K, int k) {
+    const int j = blockIdx.x * blockDim.x + threadIdx.x, i = blockIdx.y;
+    if (j >= K) return;
+    const double ip = 1.0 / A[(long)k * K + k], ik = A[(long)i * K + k], kj = A[(long)k * K + j];
+    double v;
+    if (i == k) v = j == k ? ip : kj * ip;
+    else v = j == k ? -ik * ip : A[(long)i * K + j] - ik * (kj * ip);
+    B[(long)i * K + j] = v;
+}
+// Digits of a table: the columns take sums over the mirror images of a rep, so
+// they are divided by their number.
+__global__ void __launch_bounds__(256) k_wide_table(int u, WideGeom g, const double *M, unsigned char *A, double *rf) {
+    __shared__ int smax;
+    const int row = blockIdx.x, K = g.K[u];
+    const int d0 = g.d[limb_odd(u, 0)], d1 = g.d[limb_odd(u, 1)], d2 = g.d[limb_odd(u, 2)], cen = g.d[0] - 1;
+    if (threadIdx.x == 0) smax = 0;
+    __syncthreads();
+    auto entry = [&](int k) -> double {
+        if (row >= K || k >= K) return 0.0;
+        int i[3];
+        surf_rep(d0, d1, d2, k, i);
+        const double s = (i[0] == cen ? 1.0 : 0.5) * (i[1] == cen ? 1.0 : 0.5) * (i[2] == cen ? 1.0 : 0.5);
+        return s * M[(long)row * K + k];
+    };
+    int mx = 0;
+    for (int k = threadIdx.x; k < K; k += blockDim.x) mx = max(mx, biased_exp(entry(k)));
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    if ((threadIdx.x & 31) == 0) atomicMax(&smax, mx);
+    __syncthreads();
+    const int e = smax;
+    if (threadIdx.x == 0) rf[g.rf_off[u] + row] = limb_row_factor(e);
+    unsigned char *At = A + g.a_off[u] + (long)(row / kLimbM) * g.kst[u] * kLimbAStep;
+    for (int q = threadIdx.x; q < g.kst[u] * 2; q += blockDim.x) {
+        unsigned long long Y[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) Y[j] = digit_bytes(e ? to_limb_int(entry(8 * q + j), e) : 0);
+        unsigned char *o = At + limb_chunk_off(row % kLimbM, q, kLimbABlk);
+#pragma unroll
+        for (int i = 0; i < kLimbs; ++i) *(uint4 *)(o + i * kLimbABlk) = digit_chunk(Y, i);
+    }
+}
+
+size_t wide_smem(int n, bool first) {
+    const int m = n - 1;
+    const size_t S = n == 16 || n == 32 ? 0 : (size_t)m * m, X = n > 16 ? 0 : (size_t)m * m * m;
+    return 8 * (S + X + (first ? (size_t)wide_geometry(n).v_total : 0));
 }
 
 }  // namespace
@@ -443,50 +674,157 @@ cudaError_t launch_boundary_outer(const mlc_plan_s *pl, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-// Fixed-point steps of the two-layer Dirichlet solve after the first: the
-// error contracts by about 0.025 per step, so ten take it below 1e-16.
-constexpr int kWideDirichletIters = 10;
+// Scratch of the layer operator: per 64 patches digits and factors, per patch w.
+void wide_scratch(int n, size_t *tile_bytes, size_t *item_bytes) {
+    const WideGeom w = wide_geometry(n);
+    *tile_bytes = (size_t)w.b_total + 8 * kLimbN * sizeof(double);
+    *item_bytes = (size_t)w.v_total * sizeof(double);
+}
 
-cudaError_t launch_dirichlet_wide(const mlc_plan_s *pl, const Items &it, cudaStream_t st) {
+#define MLC_WIDE_N(X) X(4) X(8) X(12) X(16) X(24) X(32)
+
+// The layer operator's tables for a patch size, built once per device and kept
+// until the process exits (27 MB at n = 32), as the Green's function tables are.
+// They are built for h = 1, so that they do not depend on which plan came first.
+cudaError_t wide_tables(int device, int n, const double *sinm, const unsigned char **A, const double **rf) {
+    struct Tab { unsigned char *A; double *rf; };
+    static std::mutex mu;
+    static std::map<std::pair<int, int>, Tab> tabs;
+    std::lock_guard<std::mutex> lk(mu);
+    const auto key = std::make_pair(device, n);
+    auto it = tabs.find(key);
+    if (it == tabs.end()) {
+        const WideGeom g = wide_geometry(n);
+        Tab t{nullptr, nullptr};
+        double *work = nullptr, *lam = nullptr, *M[2] = {nullptr, nullptr};
+        constexpr int kCols = 304;  // columns per launch
+        const int m = n - 1;
+        std::vector<double> lh((size_t)m * m * m);  // (2/n)^3 / eigenvalue of L_odd
+        for (int a = 0; a < m; ++a)
+            for (int b = 0; b < m; ++b)
+                for (int c = 0; c < m; ++c) {
+                    double l = 0.0;
+                    for (int s0 = -2; s0 <= 2; ++s0)
+                        for (int s1 = -2; s1 <= 2; ++s1)
+                            for (int s2 = -2; s2 <= 2; ++s2)
+                                if (const double q = stencil_coef(10, s0, s1, s2))
+                                    l += q * std::cos(M_PI * s0 * (a + 1) / n) * std::cos(M_PI * s1 * (b + 1) / n) *
+                                         std::cos(M_PI * s2 * (c + 1) / n);
+                    lh[((size_t)a * m + b) * m + c] = std::pow(2.0 / n, 3) / l;
+                }
+        const size_t m3 = (size_t)(n - 1) * (n - 1) * (n - 1), kk = (size_t)g.K[0] * g.K[0] * sizeof(double);
+        cudaError_t e = cudaMalloc((void **)&t.A, g.a_bytes);
+        if (e == cudaSuccess) e = cudaMalloc((void **)&t.rf, g.rf_rows * sizeof(double));
+        if (e == cudaSuccess) e = cudaMalloc((void **)&work, kCols * m3 * sizeof(double));
+        if (e == cudaSuccess) e = cudaMalloc((void **)&lam, m3 * sizeof(double));
+        if (e == cudaSuccess) e = cudaMemcpy(lam, lh.data(), m3 * sizeof(double), cudaMemcpyHostToDevice);
+        for (auto &p : M)
+            if (e == cudaSuccess) e = cudaMalloc((void **)&p, kk);
+        for (int u = 0; u < 8 && e == cudaSuccess; ++u) {
+            const int K = g.K[u];
+            for (int j = 0; j < K; j += kCols) {
+                const int nj = std::min(kCols, K - j);
+                switch (n) {
+#define MLC_X(NN) case NN: k_wide_columns<NN><<<nj, 256, wide_smem(NN, false)>>>(u, g, lam, sinm, work, j, M[0]); break;
+                    MLC_WIDE_N(MLC_X)
+#undef MLC_X
+                }
+            }
+            int cur = 0;
+            for (int k = 0; k < K; ++k, cur ^= 1)
+                k_wide_invert<<<dim3((K + 255) / 256, K), 256>>>(M[cur], M[cur ^ 1], K, k);
+            if (K) k_wide_table<<<g.tiles[u] * kLimbM, 256>>>(u, g, M[cur], t.A, t.rf);
+            e = cudaGetLastError();
+            if (e == cudaSuccess) e = cudaDeviceSynchronize();
+        }
+        cudaFree(work);
+        cudaFree(lam);
+        for (auto &p : M) cudaFree(p);
+        if (e != cudaSuccess) {
+            cudaFree(t.A);
+            cudaFree(t.rf);
+            return e;
+        }
+        it = tabs.emplace(key, t).first;
+    }
+    *A = it->second.A;
+    *rf = it->second.rf;
+    return cudaSuccess;
+}
+
+cudaError_t launch_dirichlet_wide(const mlc_plan_s *pl, const Items &all, cudaStream_t st) {
     NvtxRange nvtx("mlc:dirichlet_wide");
     const Geom &g = pl->g;
-    DirWArgs a{};
-    a.it = it;
-    a.sinm = (const double *)pl->sinm;
-    a.iters = kWideDirichletIters;
-    const int m = g.n - 1;
-    // n > 16: the arrays live in the plan's workspace; shared memory holds the dense DST-I matrix
-    const size_t sm = 8 * ((g.n > 16 ? 0 : 3 * (size_t)m * m * m) + (size_t)m * m);
-#define MLC_DIRW(NN)                                                                                      \
-    case NN:                                                                                              \
-        if (g.f32in) k_dirichlet_wide<float, NN><<<it.nitems, 256, sm, st>>>(a);                          \
-        else k_dirichlet_wide<double, NN><<<it.nitems, 256, sm, st>>>(a);                                 \
+    const int n = g.n;
+    const long group = limb_group(all.cap, all.nitems, g.wide_tile_bytes, g.wide_item_bytes);
+    if (group <= 0) return cudaErrorInvalidValue;
+    for (long c0 = 0; c0 < all.nitems; c0 += group) {
+        Items it = all;
+        it.nitems = (int)std::min<long>(group, all.nitems - c0);
+        if (all.items) it.items = all.items + c0;
+        else it.first = all.first + (int)c0;
+        const int items = it.nitems, ct = (int)limb_ctiles(items);
+        DirWArgs a{};
+        a.it = it;
+        a.sinm = (const double *)pl->sinm;
+        a.g = wide_geometry(n);
+        a.Bd = (unsigned char *)it.a1;
+        a.cf = (double *)(a.Bd + ct * a.g.b_total);
+        double *V = a.cf + 8 * ct * kLimbN;
+        a.V = V;
+        a.cols = items;
+        a.ctiles = ct;
+        switch (n) {
+#define MLC_X(NN)                                                                                             \
+    case NN:                                                                                                  \
+        if (g.f32in) k_wide_first<float, NN><<<items, 256, wide_smem(NN, true), st>>>(a);                     \
+        else k_wide_first<double, NN><<<items, 256, wide_smem(NN, true), st>>>(a);                            \
         break;
-    switch (g.n) {
-        MLC_DIRW(4)
-        MLC_DIRW(8)
-        MLC_DIRW(12)
-        MLC_DIRW(16)
-        MLC_DIRW(24)
-        MLC_DIRW(32)
-        default: return cudaErrorInvalidValue;
+            MLC_WIDE_N(MLC_X)
+#undef MLC_X
+            default: return cudaErrorInvalidValue;
+        }
+        LimbJob job{};
+        int t0 = 0;
+        for (int c = 0; c < 8; ++c) {
+            const int u = limb_table(true, c);
+            if (!a.g.K[u]) continue;  // n = 4 has no layer rep that is odd along every axis away from the faces
+            job.part[job.nparts++] = LimbPart{pl->wide_A + a.g.a_off[u], (long)a.g.kst[u] * kLimbAStep, pl->wide_rf + a.g.rf_off[u],
+                                              nullptr, a.g.b_step[c] * ct, a.g.v_step[c] * items, (long)c * ct * kLimbN,
+                                              a.g.kst[u], a.g.K[u], items, ct, t0};
+            t0 += a.g.tiles[u] * ct;
+        }
+        job.B = a.Bd;
+        job.cf = a.cf;
+        job.cf_step = 1;
+        job.V = V;
+        job.ntiles = t0;
+        job.wait_tries = 1 << 22;
+        cudaError_t e = cudaGetLastError();
+        if (e == cudaSuccess) e = launch_limb_gemm(job, it, st);
+        if (e != cudaSuccess) return e;
+        switch (n) {
+#define MLC_X(NN)                                                                                             \
+    case NN:                                                                                                  \
+        if (g.f32in) k_wide_last<float, NN><<<items, 256, wide_smem(NN, false), st>>>(a);                     \
+        else k_wide_last<double, NN><<<items, 256, wide_smem(NN, false), st>>>(a);                            \
+        break;
+            MLC_WIDE_N(MLC_X)
+#undef MLC_X
+        }
     }
-#undef MLC_DIRW
     return cudaGetLastError();
 }
 
 void configure_wide() {
     const int big = 200 * 1024;
-#define MLC_DIRW_ATTR(NN)                                                                                   \
-    cudaFuncSetAttribute(k_dirichlet_wide<float, NN>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);   \
-    cudaFuncSetAttribute(k_dirichlet_wide<double, NN>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
-    MLC_DIRW_ATTR(4)
-    MLC_DIRW_ATTR(8)
-    MLC_DIRW_ATTR(12)
-    MLC_DIRW_ATTR(16)
-    MLC_DIRW_ATTR(24)
-    MLC_DIRW_ATTR(32)
-#undef MLC_DIRW_ATTR
+#define MLC_X(NN)                                                                                          \
+    cudaFuncSetAttribute(k_wide_first<float, NN>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);       \
+    cudaFuncSetAttribute(k_wide_first<double, NN>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);      \
+    cudaFuncSetAttribute(k_wide_last<float, NN>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);        \
+    cudaFuncSetAttribute(k_wide_last<double, NN>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
+    MLC_WIDE_N(MLC_X)
+#undef MLC_X
 #define MLC_RESO_ATTR(KK)                                                                                   \
     cudaFuncSetAttribute(k_resid_outer<float, KK>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);      \
     cudaFuncSetAttribute(k_resid_outer<double, KK>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);

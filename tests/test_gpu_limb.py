@@ -193,3 +193,53 @@ def test_ring_products_against_the_oracle(torch_cuda, N, n, s, Q, P, g_beta, tie
         on = g[:, ax] % n == 0
         u, v = (g[on, e] for e in range(3) if e != ax)
         assert np.abs(B[ax, g[on, ax] // n, u, v] - st["phiB"][on]).max() <= 1e-12 * np.abs(st["phiB"]).max()
+
+
+@pytest.mark.parametrize("N,n,s,tier", [
+    (4, 4, 16, 0),       # one patch; blocks of 7, 4, 2 and 1 layer reps
+    (20, 4, 16, 1),      # 125 patches: two column tiles, the second ragged
+    (24, 8, 16, 1),
+    (24, 12, 20, 0),
+    (32, 16, 16, 0),     # the largest patch whose work array is in shared memory
+    (48, 24, 20, 1),
+    (32, 32, 16, 0),     # 721 reps: six row tiles
+])
+def test_q10_dirichlet_solves_its_equation(torch_cuda, N, n, s, tier):
+    """The two-layer Dirichlet step by two DST solves around the layer operator: its result satisfies
+    the operator's equation with both boundary layers.  Bound: the result is within 100 roundings
+    (2^-53) of the solution, relative to the largest value, and a residual sums |a_j| / h^2 of that,
+    plus as many roundings of its own evaluation."""
+    torch = torch_cuda
+    from paper_1702_08111_gb300 import mlc
+    plan = _plan(torch, N, n, s, 10, tier)
+    f = np.random.default_rng(N + n).uniform(-1, 1, (N,) * 3).astype(np.float32 if tier else np.float64)
+    phi = plan.solve(torch.from_numpy(f).cuda()).cpu().numpy()
+    f = f.astype(np.float64)
+    B, B2 = plan.export(mlc.STAGE_PHIB), plan.export(mlc.STAGE_PHIB_OUTER)
+    a = {(0, 0, 0): -1079 / 210, (1, 0, 0): 24 / 35, (1, 1, 0): 17 / 210, (1, 1, 1): 11 / 420, (2, 0, 0): -1 / 60,
+         (2, 1, 0): -1 / 420}
+    np_, h = N // n, 1.0 / N
+    rng = np.random.default_rng(1)
+    for i in {(0, 0, 0), (np_ - 1,) * 3, tuple(int(v) for v in rng.integers(0, np_, 3))}:
+        o = [n * v for v in i]
+        U = np.zeros((n + 3,) * 3)      # relative nodes [-1, n + 1]^3
+        inside = tuple(slice(o[d] + 1, o[d] + n) for d in range(3))
+        U[2:n + 1, 2:n + 1, 2:n + 1] = phi[inside] - 2 / 35 * h * h * f[inside]
+        for ax in range(3):
+            e = [d for d in range(3) if d != ax]
+            cut = tuple(slice(o[d], o[d] + n + 1) for d in e)
+            for side in (0, 1):
+                at = [slice(1, n + 2)] * 3
+                at[ax] = 1 + n * side
+                U[tuple(at)] = B[ax, i[ax] + side][cut]
+                at[ax] = (n + 2) * side
+                U[tuple(at)] = B2[ax, i[ax] + side, side][cut]
+        r, total = -f[inside], 0.0
+        for s0 in range(-2, 3):
+            for s1 in range(-2, 3):
+                for s2 in range(-2, 3):
+                    c = a.get(tuple(sorted((abs(s0), abs(s1), abs(s2)), reverse=True)), 0.0) / (h * h)
+                    if c:
+                        r = r + c * U[2 + s0:n + 1 + s0, 2 + s1:n + 1 + s1, 2 + s2:n + 1 + s2]
+                        total += abs(c)
+        assert np.abs(r).max() <= 200 * 2.0 ** -53 * total * np.abs(U).max() + 8 * 2.0 ** -53
