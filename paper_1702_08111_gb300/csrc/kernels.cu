@@ -1305,6 +1305,262 @@ __global__ void __launch_bounds__(256) k_inv_x_pruned(InvXPArgs a) {
     }
 }
 
+// One 128-point inverse transform of a Hermitian line by an 8-lane group: the
+// radix-2 decimation in frequency of fft_dif<7>, butterfly for butterfly, with
+// the stages of half size 64 to 8 in registers (lane t holds the entries
+// t + 8 j), one exchange through the group's scratch (8 b + r at 9 b + r), and
+// the stages 4, 2, 1 on the lane's entries 8 b + r, b = t and t + 8.  QUARTER:
+// only the first 32 entries of the (bit-reversed) result, the positions that are
+// multiples of 4, so the first two stages are sums and b = t < 4.  src(i): entry i
+// of the line; out(b, r, real part): entry 8 b + r of the result.
+template <bool QUARTER, typename S, typename O>
+__device__ __forceinline__ void inv128_line(int t, const float2 (&w6)[8], const float2 (&w5)[4], const float2 (&w4)[2],
+                                            float2 w3, const float2 (&w2)[4], float2 *xs, unsigned gm, S &&src, O &&out) {
+    float2 v[16];
+#pragma unroll
+    for (int j = 0; j < 16; ++j) v[j] = src(t + 8 * j);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        const float2 a = v[j], b = v[j + 8];
+        v[j] = cadd(a, b);
+        if (!QUARTER) v[j + 8] = cmul(csub(a, b), w6[j]);
+    }
+    constexpr int NV = QUARTER ? 4 : 16;
+#pragma unroll
+    for (int g = 0; g < (QUARTER ? 8 : 16); g += 8)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const float2 a = v[g + j], b = v[g + j + 4];
+            v[g + j] = cadd(a, b);
+            if (!QUARTER) v[g + j + 4] = cmul(csub(a, b), w5[j]);
+        }
+#pragma unroll
+    for (int g = 0; g < NV; g += 4)
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const float2 a = v[g + j], b = v[g + j + 2];
+            v[g + j] = cadd(a, b);
+            v[g + j + 2] = cmul(csub(a, b), w4[j]);
+        }
+#pragma unroll
+    for (int g = 0; g < NV; g += 2) {
+        const float2 a = v[g], b = v[g + 1];
+        v[g] = cadd(a, b);
+        v[g + 1] = cmul(csub(a, b), w3);
+    }
+#pragma unroll
+    for (int j = 0; j < NV; ++j) xs[9 * j + t] = v[j];
+    __syncwarp(gm);
+#pragma unroll
+    for (int h = 0; h < (QUARTER ? 1 : 2); ++h) {
+        const int b = t + 8 * h;
+        if (!QUARTER || t < 4) {
+            float2 u[8];
+#pragma unroll
+            for (int r = 0; r < 8; ++r) u[r] = xs[9 * b + r];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const float2 a = u[r], c = u[r + 4];
+                u[r] = cadd(a, c);
+                u[r + 4] = r == 0 ? csub(a, c) : cmul(csub(a, c), w2[r]);
+            }
+#pragma unroll
+            for (int g = 0; g < 8; g += 4)
+#pragma unroll
+                for (int r = 0; r < 2; ++r) {
+                    const float2 a = u[g + r], c = u[g + r + 2];
+                    u[g + r] = cadd(a, c);
+                    u[g + r + 2] = r == 0 ? csub(a, c) : mul_mi(csub(a, c), true);
+                }
+#pragma unroll
+            for (int g = 0; g < 8; g += 2) {
+                out(b, g, u[g].x + u[g + 1].x);
+                out(b, g + 1, u[g].x - u[g + 1].x);
+            }
+        }
+    }
+    __syncwarp(gm);
+}
+
+// Pruned inverse real transform along x for M = 128 (same contract and bits as
+// k_inv_x_pruned): 8-lane groups take one needed row each, entirely in registers,
+// and store their results directly.  Rows that are read only at multiples of 4
+// (the coarse lattice and the face planes on it) get a quarter of the transform.
+// n = 32, s = 28, Q = 6: 256 whole and 465 quarter rows per patch, and 7488
+// direct sums of 65 terms for the rows that need x on the face planes only.
+// Bound: reads of the staged block (46 KB per z row, 13.5 GB for 4096 patches,
+// 2 ms of HBM time) and the shared-memory loads of the direct sums.  The kernel
+// it replaces kept all rows of a z row in shared memory through seven passes, one
+// CTA per SM: 512 patches of 32^3 took 2.17 ms, now 0.58.
+template <bool OUTER>
+__global__ void __launch_bounds__(128) k_inv_x128(InvXPArgs a) {
+    constexpr int M = 128, MH = 65, XP = 152;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ int rows[2][128];   // needed rows: whole, quarter
+    __shared__ int nrow[2];
+    __shared__ unsigned wmask[2][4];
+    __shared__ int xinfo[M];       // per x position: class bits (1 alpha, 2 plane, 4 coarse) | off slot + 1 << 3 | plane slot << 12 | coarse index << 20
+    __shared__ unsigned long long bar;
+    const int W = a.W, n = a.n, s = a.s, ga = a.ga, pl0 = a.pl0, wa = a.wa, nc = a.nc, npa = a.npa;
+    float2 *tw = (float2 *)smem_raw;  // M twiddles
+    float2 *raw = tw + M;             // MH x W (block of a.blk entries, 16-byte aligned)
+    float2 *xs_all = raw + a.blk;     // 16 groups x XP
+    const int jz = blockIdx.x % a.nz, zi = a.zrow[jz];
+    int p;
+    const PlanPtrs &PP = item_plan(a.it, blockIdx.x / a.nz, p);
+    const int z = zi - s;
+    const float2 *twg = (const float2 *)a.tw;
+    for (int j = threadIdx.x; j < M; j += blockDim.x) {
+        float2 w = twg[j & (M / 2 - 1)];
+        if (j >= M / 2) { w.x = -w.x; w.y = -w.y; }
+        tw[j] = w;
+    }
+    const float2 *in = (const float2 *)a.it.a4 + ((long)(blockIdx.x / a.nz) * a.nz + jz) * a.blk;  // scratch slot = item
+    const unsigned bytes = (unsigned)(a.blk * sizeof(float2));
+    if (threadIdx.x == 0) {  // stage the contiguous block with one bulk copy
+        mbar_init(&bar, 1);
+        mbar_expect_tx(&bar, bytes);
+        if (!a.skip_copy) bulk_g2s(raw, in, bytes, &bar);
+    }
+    const int kl = -s / 4;
+    const bool zP = on_plane(z, n, ga, pl0), zA = in_alpha(z, n, ga), zC = (z & 3) == 0;
+    const int zO = OUTER ? off_slot(z, n, ga, pl0, npa) : -1;
+    {   // per row y = threadIdx.x - s: whole, quarter or none; per x position: its classes
+        const int yi = threadIdx.x, y = yi - s;
+        const bool yA = in_alpha(y, n, ga), yP = on_plane(y, n, ga, pl0), yC = (y & 3) == 0;
+        const bool zQ = zP || zO >= 0, yQ = yP || (OUTER && off_slot(y, n, ga, pl0, npa) >= 0);
+        const bool in_box = yi < W;
+        const bool whole = in_box && ((zQ && yA) || (yQ && zA) || (OUTER && zC && yC && zA && yA));
+        const bool quarter = in_box && !whole && zC && yC;
+        const unsigned mw = __ballot_sync(0xffffffffu, whole), mq = __ballot_sync(0xffffffffu, quarter);
+        if ((threadIdx.x & 31) == 0) { wmask[0][threadIdx.x >> 5] = mw; wmask[1][threadIdx.x >> 5] = mq; }
+        const int x = yi <= n + s ? yi : yi - M;
+        const bool box = x >= -s && x <= n + s, xA = in_alpha(x, n, ga), xP = on_plane(x, n, ga, pl0);
+        const int xO = OUTER && xA ? off_slot(x, n, ga, pl0, npa) : -1;
+        xinfo[yi] = box ? ((xA ? 1 : 0) | (xP ? 2 : 0) | ((x & 3) == 0 ? 4 : 0) | ((xO + 1) << 3) |
+                           ((xP ? (x - pl0) / n : 0) << 12) | (((x >> 2) - kl) << 20))
+                        : 0;
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int wd = yi >> 5, lane = yi & 31;
+            const unsigned mine = wmask[q][wd];
+            int before = __popc(mine & ((1u << lane) - 1u));
+            for (int e = 0; e < wd; ++e) before += __popc(wmask[q][e]);
+            if ((mine >> lane) & 1u) rows[q][before] = yi;
+            if (yi == 127) nrow[q] = before + ((mine >> lane) & 1u);
+        }
+    }
+    __syncthreads();
+    const bool arrived = mbar_wait_bounded(&bar, 0, a.wait_tries);
+    if (__syncthreads_or(!arrived)) {  // uniform decision for the whole CTA
+        if (threadIdx.x == 0) {
+            atomicExch(PP.err, 1);
+            mbar_wait_bounded(&bar, 0, a.wait_tries);  // one more bounded wait for the copy in flight
+        }
+        return;
+    }
+    float *cl = (float *)PP.cl + (long)p * nc * nc * nc;
+    float *fp = (float *)PP.fp + (long)p * 3 * npa * wa * wa;
+    float *f2 = OUTER ? (float *)PP.fp2 + (long)p * 6 * npa * wa * wa : nullptr;
+    const long ncl = (long)nc * nc * nc, nfp = 3L * npa * wa * wa, nf2 = 2 * nfp;
+    const int grp = threadIdx.x >> 3, t = threadIdx.x & 7;
+    const unsigned gm = 0xffu << (threadIdx.x & 24);
+    float2 *xs = xs_all + grp * XP;
+    float2 w6[8], w5[4], w4[2], w3, w2[4];  // inverse twiddles of this lane's butterflies
+    auto itw = [&](int j) { float2 w = tw[j]; w.y = -w.y; return w; };
+#pragma unroll
+    for (int j = 0; j < 8; ++j) w6[j] = itw(t + 8 * j);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) w5[j] = itw((t + 8 * j) << 1);
+#pragma unroll
+    for (int j = 0; j < 2; ++j) w4[j] = itw((t + 8 * j) << 2);
+    w3 = itw(t << 3);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) w2[j] = itw(j << 4);
+    for (int q = 0; q < 2; ++q)
+        for (int l = grp; l < nrow[q]; l += 16) {
+            const int yi = rows[q][l], y = yi - s;
+            const bool yA = in_alpha(y, n, ga), yP = on_plane(y, n, ga, pl0), yC = (y & 3) == 0;
+            const int yO = OUTER && yA && zA ? off_slot(y, n, ga, pl0, npa) : -1;
+            const int zOO = yA && zA ? zO : -1;
+            const long c0 = zC && yC ? ((long)((z >> 2) - kl) * nc + ((y >> 2) - kl)) * nc : -1;
+            const long a0 = zP && yA ? ((long)((z - pl0) / n) * wa + (y + ga)) * wa + ga : -1;
+            const long a1 = yP && zA ? ((long)(npa + (y - pl0) / n) * wa + (z + ga)) * wa + ga : -1;
+            const long a2 = zA && yA ? ((long)(2 * npa) * wa + (z + ga)) * wa + (y + ga) : -1;
+            auto src = [&](int i) -> float2 {
+                float2 v;
+                if (i < MH) {
+                    v = raw[i * W + yi];
+                } else {
+                    v = raw[(M - i) * W + yi];
+                    v.y = -v.y;
+                }
+                return v;
+            };
+            auto out = [&](int b, int r, float v) {
+                const int pos = (int)(__brev((unsigned)(8 * b + r)) >> 25), xf = xinfo[pos];
+                if (!xf) return;
+                const int x = pos <= n + s ? pos : pos - M;
+                if ((xf & 4) && c0 >= 0) {
+                    const long i = c0 + (xf >> 20);
+                    if (in_range(i, ncl, PP.err)) cl[i] = v;
+                }
+                if ((xf & 1) && a0 >= 0 && in_range(a0 + x, nfp, PP.err)) fp[a0 + x] = v;
+                if ((xf & 1) && a1 >= 0 && in_range(a1 + x, nfp, PP.err)) fp[a1 + x] = v;
+                if ((xf & 2) && a2 >= 0) {
+                    const long i = a2 + (long)((xf >> 12) & 0xff) * wa * wa;
+                    if (in_range(i, nfp, PP.err)) fp[i] = v;
+                }
+                if (OUTER && (xf & 1) && yA && zA) {  // [patch][axis][j][side][u][v], in-plane (u, v) as for fp
+                    const int o2 = ((xf >> 3) & 0x1ff) - 1;
+                    if (zOO >= 0) {
+                        const long i = ((long)zOO * wa + (y + ga)) * wa + (x + ga);
+                        if (in_range(i, nf2, PP.err)) f2[i] = v;
+                    }
+                    if (yO >= 0) {
+                        const long i = ((long)(2 * npa + yO) * wa + (z + ga)) * wa + (x + ga);
+                        if (in_range(i, nf2, PP.err)) f2[i] = v;
+                    }
+                    if (o2 >= 0) {
+                        const long i = ((long)(4 * npa + o2) * wa + (z + ga)) * wa + (y + ga);
+                        if (in_range(i, nf2, PP.err)) f2[i] = v;
+                    }
+                }
+            };
+            if (q == 0) inv128_line<false>(t, w6, w5, w4, w3, w2, xs, gm, src, out);
+            else inv128_line<true>(t, w6, w5, w4, w3, w2, xs, gm, src, out);
+        }
+    // rows that only need x on the face planes (OUTER: and one node off them):
+    // direct sums over the half spectrum, neighbouring threads on neighbouring rows
+    if (zA && !zP && zO < 0) {
+        const int nsub = OUTER ? 3 : 1, na = n + 2 * ga + 1;  // x = plane, plane - 1, plane + 1
+        for (int e = threadIdx.x; e < na * npa * nsub; e += blockDim.x) {
+            const int y = e % na - ga, js = e / na, j = js / nsub, sub = js % nsub, yi = y + s;
+            const bool yP = on_plane(y, n, ga, pl0), yC = (y & 3) == 0;
+            if (yP || (OUTER && off_slot(y, n, ga, pl0, npa) >= 0) || (zC && yC)) continue;  // done by a transformed row
+            const int x = pl0 + j * n + (sub == 1 ? -1 : (sub == 2 ? 1 : 0));
+            if (sub && !in_alpha(x, n, ga)) continue;
+            const int pos = x & (M - 1);
+            float acc = 0.f;
+#pragma unroll 5
+            for (int k = 0; k < MH; ++k) {
+                const float2 X = raw[k * W + yi];
+                const float2 w = tw[(k * pos) & (M - 1)];  // exp(+2 pi i k pos / M) = conj(tw)
+                const float re = X.x * w.x + X.y * w.y;
+                acc += (k == 0 || 2 * k == M) ? re : 2.f * re;
+            }
+            if (sub == 0) {
+                const long i = (((long)(2 * npa + j)) * wa + (z + ga)) * wa + (y + ga);
+                if (in_range(i, nfp, PP.err)) fp[i] = acc;
+            } else {  // off-plane slot 2 j + side of axis 2
+                const long i = ((long)(2 * 2 * npa + 2 * j + (sub == 2 ? 1 : 0)) * wa + (z + ga)) * wa + (y + ga);
+                if (in_range(i, nf2, PP.err)) f2[i] = acc;
+            }
+        }
+    }
+}
+
 // Pruned inverse real transform along x for M = 64 (same contract as
 // k_inv_x_pruned; local fields leave in the working precision R).  The needed
 // rows go in pairs: with A, B the Hermitian half spectra of two rows,
@@ -2790,8 +3046,8 @@ template <int LOG2M>
 void set_patch_attrs() {
     const int big = 200 * 1024;
     cudaFuncSetAttribute(k_fwd_x<LOG2M, float, true, float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
-    cudaFuncSetAttribute(k_inv_x_pruned<LOG2M, float, float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         LOG2M == 7 ? (int)kPatchSmem : big);
+    if constexpr (LOG2M < 7)
+        cudaFuncSetAttribute(k_inv_x_pruned<LOG2M, float, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
 }
 
 // Local convolutions of a set of patches: forward x (real), fused slab (y,
@@ -2889,6 +3145,10 @@ cudaError_t run_patch_conv_t(const mlc_plan_s *pl, const Items &it, const void *
             const size_t sm64 = ((size_t)M + (size_t)g.a4blk + (thr / 8) * 72) * sizeof(typename Cx<R>::T) +
                                 (size_t)a.maxfft * 68 * sizeof(R);
             k_inv_x64<R><<<nb * a.nz, thr, sm64, st>>>(a);
+        } else if constexpr (LOG2M == 7) {
+            const size_t sm128 = ((size_t)M + (size_t)g.a4blk + 16 * 152) * sizeof(float2);
+            if (g.wide) k_inv_x128<true><<<nb * a.nz, 128, sm128, st>>>(a);
+            else k_inv_x128<false><<<nb * a.nz, 128, sm128, st>>>(a);
         } else {
             k_inv_x_pruned<LOG2M, R, R><<<nb * a.nz, 256, sm, st>>>(a);
         }
@@ -2920,6 +3180,8 @@ void configure_kernels() {
     set_patch_attrs<5>();
     set_patch_attrs<6>();
     set_patch_attrs<7>();
+    cudaFuncSetAttribute(k_inv_x128<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    cudaFuncSetAttribute(k_inv_x128<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     cudaFuncSetAttribute(k_inv_x64<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     cudaFuncSetAttribute(k_slab64r<17>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     cudaFuncSetAttribute(k_slab64r<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);

@@ -243,3 +243,32 @@ def test_q10_dirichlet_solves_its_equation(torch_cuda, N, n, s, tier):
                         r = r + c * U[2 + s0:n + 1 + s0, 2 + s1:n + 1 + s1, 2 + s2:n + 1 + s2]
                         total += abs(c)
         assert np.abs(r).max() <= 200 * 2.0 ** -53 * total * np.abs(U).max() + 8 * 2.0 ** -53
+
+
+@pytest.mark.parametrize("N,n,s,Q,kw", [
+    (8, 4, 60, 4, {"b": 1, "mode": 1}),   # the widest box of the smallest patch: many face planes
+    (16, 8, 56, 4, {"mode": 1}),
+    (36, 12, 52, 6, {"mode": 1}),
+    (32, 16, 20, 6, {}),                  # just above the 64-point period
+    (48, 24, 40, 4, {"mode": 1}),
+    (48, 24, 12, 6, {}),
+    (32, 32, 12, 6, {}),                  # inner box = patch
+    (64, 32, 32, 4, {}),
+    (64, 16, 28, 10, {}),                 # the planes next to the face planes
+])
+def test_128_point_inverse_against_fp64(torch_cuda, N, n, s, Q, kw):
+    """Split-tier local fields with a 128-point period (registers, whole and quarter rows, direct
+    sums) against the FP64 tier's products.  Tolerance: the split tier's bar, 1e-6 of the largest
+    value, at the lattice points and for the boundary values the face planes give."""
+    torch = torch_cuda
+    from paper_1702_08111_gb300 import mlc
+    f = np.random.default_rng(N + s).uniform(0, 1, (N,) * 3)
+    got = []
+    for tier in (1, 0):
+        plan = _plan(torch, N, n, s, Q, tier, **kw)
+        assert plan.info.M == 128
+        plan.solve(torch.from_numpy(f.astype(np.float32).astype(np.float64 if tier == 0 else np.float32)).cuda())
+        got.append([plan.export(st) for st in (mlc.STAGE_COARSE_SAMPLES, mlc.STAGE_PHIB)
+                    + ((mlc.STAGE_PHIB_OUTER,) if Q == 10 else ())])
+    for x, y in zip(*got):
+        assert np.abs(x - y).max() <= 1e-6 * np.abs(y).max()
