@@ -2460,9 +2460,42 @@ __device__ __forceinline__ void dst31_fast(T (&x)[31], const T (&sv)[17]) {
     for (int j = 1; j <= 15; ++j) x[2 * j - 1] = dm[j - 1];  // y_{2j}
 }
 
+// The third axis of a Dirichlet solve.  With sine modes k1, k2 on axes 1 and 2
+// the stencil is a tridiagonal system along axis 0, a (u_{i-1} + u_{i+1}) + d u_i =
+// r_i with |d| > 2 |a|, solved by Gaussian elimination: four operations per value
+// where transforming the axis and back takes two DST-I (19 per value at n = 32).
+// E_i = (2/n)^2 / (d - a^2 e_{i-1}) (e the reciprocals without the factor) and
+// a' = a (n/2)^2 carry the normalisation of the other axes' transforms.  Lines of
+// X at stride m^2; E in the same places; a' per line after the m^3 values of E.
+// The step is bound by the FP64 pipe: 256^3, n = 16 split 1.27 -> 1.04 ms, n = 32
+// FP64 2.42 -> 1.95 ms, 180^3, n = 12 0.75 -> 0.57 ms, 512^3, n = 32 16.6 -> 13.5 ms.
+template <typename T, int m>
+__device__ __forceinline__ void dirichlet_tri(T *X, const T *E, int line) {
+    const T a = E[m * m * m + line];
+    T *xl = X + line;
+    const T *el = E + line;
+    T x[m];
+#pragma unroll
+    for (int i = 0; i < m; ++i) x[i] = FT<T>::rn(xl[i * m * m]);
+    T g = x[0] * el[0];
+    x[0] = g;
+#pragma unroll
+    for (int i = 1; i < m; ++i) {
+        g = FT<T>::rn(FT<T>::fma(-a, g, x[i])) * el[i * m * m];
+        x[i] = g;
+    }
+    T u = FT<T>::rn(x[m - 1]);
+    xl[(m - 1) * m * m] = u;
+#pragma unroll
+    for (int i = m - 2; i >= 0; --i) {
+        u = FT<T>::rn(FT<T>::fma(-el[i * m * m], a * u, x[i]));
+        xl[i * m * m] = u;
+    }
+}
+
 // Local Dirichlet solve of one patch (Sec. 4, final step): the (Q-th order)
-// stencil problem on the closed patch with boundary data phi^B, by DST-I in
-// all three axes, then phi = u + (h^2/12) f.  T: the arithmetic between the
+// stencil problem on the closed patch with boundary data phi^B, by DST-I on
+// two axes and tridiagonal solves along the third, then phi = u + (h^2/12) f.  T: the arithmetic between the
 // loads and the final FP64 store, FP64 (the FP64 pipe) or double-float (the
 // FP32 pipe; GB300 issues FP64 on ~1/67 of the FP32 lanes).  TF: the charge.
 // Patches up to n = 24 keep their m^3 work array in shared memory; larger
@@ -2565,29 +2598,28 @@ __global__ void __launch_bounds__(256, NN > 16 ? 1 : (std::is_same<T, double>::v
         (void)sa;
         __syncthreads();  // the next pass may update the same edge nodes
     }
-    // DST-I along axes 2, 1, 0; scale by the inverse eigenvalues; DST-I along 2, 1, 0
+    // DST-I along axes 2 and 1, the tridiagonal solves along axis 0, DST-I along 2 and 1
     if constexpr (NN == 16) {
         // n = 16: one thread per line with the split-radix DST (dst15_fast)
         T sv[9];
         sv[0] = FT<T>::zero();
 #pragma unroll
         for (int i = 1; i <= 8; ++i) sv[i] = Sh[i - 1];  // sin(pi i / 16)
-        for (int pass = 0; pass < 6; ++pass) {
-            const int axis = 2 - (pass % 3);
+#pragma unroll 1
+        for (int pass = 0; pass < 5; ++pass) {
+            if (pass == 2) {
+                for (int l = threadIdx.x; l < m * m; l += blockDim.x) dirichlet_tri<T, m>(X, lam, l);
+                __syncthreads();
+                continue;
+            }
+            const bool ax2 = pass == 0 || pass == 3;
             for (int l = threadIdx.x; l < m * m; l += blockDim.x) {
                 const int q1 = l % m, q0 = l / m;
-                int base, str;
-                if (axis == 2) { base = (q0 * m + q1) * m; str = 1; }
-                else if (axis == 1) { base = q0 * m * m + q1; str = m; }
-                else { base = q0 * m + q1; str = m * m; }
+                const int base = ax2 ? l * m : q0 * m * m + q1, str = ax2 ? 1 : m;
                 T x[15];
 #pragma unroll
                 for (int t = 0; t < 15; ++t) x[t] = FT<T>::rn(X[base + t * str]);
                 dst15_fast(x, sv);
-                if (pass == 2) {
-#pragma unroll
-                    for (int t = 0; t < 15; ++t) x[t] = x[t] * lam[base + t * str];
-                }
 #pragma unroll
                 for (int t = 0; t < 15; ++t) X[base + t * str] = x[t];
             }
@@ -2599,22 +2631,21 @@ __global__ void __launch_bounds__(256, NN > 16 ? 1 : (std::is_same<T, double>::v
         sv[0] = FT<T>::zero();
 #pragma unroll
         for (int i = 1; i <= 16; ++i) sv[i] = Sh[i - 1];  // sin(pi i / 32)
-        for (int pass = 0; pass < 6; ++pass) {
-            const int axis = 2 - (pass % 3);
+#pragma unroll 1
+        for (int pass = 0; pass < 5; ++pass) {
+            if (pass == 2) {
+                for (int l = threadIdx.x; l < m * m; l += blockDim.x) dirichlet_tri<T, m>(X, lam, l);
+                __syncthreads();
+                continue;
+            }
+            const bool ax2 = pass == 0 || pass == 3;
             for (int l = threadIdx.x; l < m * m; l += blockDim.x) {
                 const int q1 = l % m, q0 = l / m;
-                int base, str;
-                if (axis == 2) { base = (q0 * m + q1) * m; str = 1; }
-                else if (axis == 1) { base = q0 * m * m + q1; str = m; }
-                else { base = q0 * m + q1; str = m * m; }
+                const int base = ax2 ? l * m : q0 * m * m + q1, str = ax2 ? 1 : m;
                 T x[31];
 #pragma unroll
                 for (int t = 0; t < 31; ++t) x[t] = FT<T>::rn(X[base + t * str]);
                 dst31_fast(x, sv);
-                if (pass == 2) {
-#pragma unroll
-                    for (int t = 0; t < 31; ++t) x[t] = x[t] * lam[base + t * str];
-                }
 #pragma unroll
                 for (int t = 0; t < 31; ++t) X[base + t * str] = x[t];
             }
@@ -2627,16 +2658,18 @@ __global__ void __launch_bounds__(256, NN > 16 ? 1 : (std::is_same<T, double>::v
     // the same instruction stream (the middle node enters with weight 0 for
     // even k).
     const int par = threadIdx.x & 1, ntl = blockDim.x >> 1;
-    for (int pass = 0; pass < 6; ++pass) {
-        const int axis = 2 - (pass % 3);
+    for (int pass = 0; pass < 5; ++pass) {
+        if (pass == 2) {
+            for (int l = threadIdx.x; l < m * m; l += blockDim.x) dirichlet_tri<T, m>(X, lam, l);
+            __syncthreads();
+            continue;
+        }
+        const bool ax2 = pass == 0 || pass == 3;
         for (int l0 = 0; l0 < m * m; l0 += ntl) {  // uniform trip count across the CTA
             const int l = l0 + (threadIdx.x >> 1);
             const bool valid = l < m * m;
             const int q1 = l % m, q0 = l / m;
-            int base = 0, str = 1;
-            if (axis == 2) { base = (q0 * m + q1) * m; str = 1; }
-            else if (axis == 1) { base = q0 * m * m + q1; str = m; }
-            else { base = q0 * m + q1; str = m * m; }
+            const int base = ax2 ? l * m : q0 * m * m + q1, str = ax2 ? 1 : m;
             T x[m];
 #pragma unroll
             for (int t = 0; t < m; ++t) x[t] = valid ? FT<T>::rn(X[base + t * str]) : FT<T>::zero();
@@ -2659,9 +2692,7 @@ __global__ void __launch_bounds__(256, NN > 16 ? 1 : (std::is_same<T, double>::v
                     T acc[4] = {FT<T>::zero(), FT<T>::zero(), FT<T>::zero(), FT<T>::zero()};
 #pragma unroll
                     for (int t = 1; t <= h; ++t) acc[(t - 1) & 3] = FT<T>::fma(row[t - 1], u[t], acc[(t - 1) & 3]);
-                    T v = (acc[0] + acc[1]) + (acc[2] + acc[3]);
-                    if (pass == 2) v = v * lam[base + (k - 1) * str];
-                    X[base + (k - 1) * str] = v;
+                    X[base + (k - 1) * str] = (acc[0] + acc[1]) + (acc[2] + acc[3]);
                 }
             }
         }

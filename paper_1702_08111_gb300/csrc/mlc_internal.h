@@ -134,7 +134,8 @@ struct PlanPtrs {
     void *resid;          // face-plane residuals (FP64 or double-float pairs, 8 bytes each)
     const void *phiB;     // boundary values on the face planes (FP64 or double-float pairs)
     double *phi;
-    const void *lam;      // Dirichlet inverse eigenvalues (2/n)^3 h^2 / lambda (FP64 or double-float)
+    const void *lam;      // Dirichlet tables: pivots and off-diagonals of the eliminations along axis 0
+                          // (FP64 or double-float); Q = 10: inverse eigenvalues (2/n)^3 h^2 / lambda
     int N, np;
     double c2h2, inv_h2;  // h^2 / 12, 1 / h^2
     double h2;            // h^2
@@ -206,7 +207,7 @@ struct mlc_plan_s {
     float2 *khat_c_df;       // coarse spectrum and twiddles as double-float (hi, lo) pairs
     float4 *tw_c_df;
     void *sinm;              // (n-1) x n/2 half DST-I matrix sin(pi k t / n), fine precision
-    void *lam;               // (n-1)^3 (2/n)^3 h^2 / stencil eigenvalue, fine precision
+    void *lam;               // Dirichlet tables, fine precision (PlanPtrs::lam)
     // workspace (device)
     void *scratch = nullptr;       // own local-convolution scratch, min(chunk, NP) patches (a1
                                    // then a4), allocated by the first solve that needs it

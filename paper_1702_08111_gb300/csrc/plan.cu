@@ -598,14 +598,38 @@ mlc_status build_tables(mlc_plan_s *pl) {
             sinm[(size_t)k * hn + t] = std::sin(M_PI * (double)r / (double)n);
         }
     }
-    for (int a = 0; a < m; ++a)
-        for (int c = 0; c < m; ++c)
-            for (int e = 0; e < m; ++e)
-                lam[((size_t)a * m + c) * m + e] = (g.h * g.h) / symbol(g.Q, cth[a], cth[c], cth[e]);
-    // in the fine precision (FP64 or double-float pairs); the DST-I
-    // normalisation (2/n)^3 is folded into lam
-    const double dnorm = std::pow(2.0 / n, 3);
-    for (double &v : lam) v *= dnorm;
+    if (g.wide) {  // inverse eigenvalues, with the DST-I normalisation (2/n)^3
+        const double dnorm = std::pow(2.0 / n, 3);
+        for (int a = 0; a < m; ++a)
+            for (int c = 0; c < m; ++c)
+                for (int e = 0; e < m; ++e)
+                    lam[((size_t)a * m + c) * m + e] = dnorm * ((g.h * g.h) / symbol(g.Q, cth[a], cth[c], cth[e]));
+    } else {
+        // the elimination along axis 0 for sine modes on axes 1 and 2 (dirichlet_tri):
+        // the symbol is d + 2 a cos(theta_0); pivots for every node, then a per mode pair.
+        // Extended precision: the lowest modes' systems are nearly singular (d + 2 a is
+        // n^-2 of d), so a cosine rounded to FP64 would show n^2-fold in the result
+        lam.resize((size_t)m * m * m + (size_t)m * m);
+        const double c2 = std::pow(2.0 / n, 2), ih2 = 1.0 / (g.h * g.h);
+        std::vector<long double> cl(m);
+        for (int k = 0; k < m; ++k) cl[k] = std::cos(std::acos(-1.0L) * (k + 1) / n);
+        // the operator's coefficients (App. A.1), b_k times h^2
+        long double sb[4] = {-4.0L, 1.0L / 3, 1.0L / 6, 0.0L};
+        if (g.Q == 6) sb[0] = -64.0L / 15, sb[1] = 7.0L / 15, sb[2] = 0.1L, sb[3] = 1.0L / 30;
+        for (int k1 = 0; k1 < m; ++k1)
+            for (int k2 = k1; k2 < m; ++k2) {  // the same for (k2, k1)
+                const long double x = cl[k1], y = cl[k2];
+                const long double off = (sb[1] + 2 * sb[2] * (x + y) + 4 * sb[3] * x * y) * ih2;
+                const long double diag = (sb[0] + 2 * sb[1] * (x + y) + 4 * sb[2] * x * y) * ih2;
+                long double e = 0.0;
+                for (int i = 0; i < m; ++i) {
+                    e = 1.0L / (diag - off * off * e);
+                    lam[((size_t)i * m + k1) * m + k2] = lam[((size_t)i * m + k2) * m + k1] = (double)(e * c2);
+                }
+                lam[((size_t)m * m + k1) * m + k2] = lam[((size_t)m * m + k2) * m + k1] = (double)(off / c2);
+            }
+    }
+    // in the fine precision (FP64 or double-float pairs)
     if (g.fine == FINE_DF) {
         float2 *a = nullptr, *c = nullptr;
         TRY(dev_upload(pl, &a, to_df(sinm)));
