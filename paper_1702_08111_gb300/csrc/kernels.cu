@@ -713,48 +713,66 @@ __host__ __device__ constexpr int brev6(int i) {
     return ((i & 1) << 5) | ((i & 2) << 3) | ((i & 4) << 1) | ((i & 8) >> 1) | ((i & 16) >> 3) | ((i & 32) >> 5);
 }
 
-// Same contract as k_slab, for M = 64 (64 threads: one line each).  Passes:
-// forward y on the nin nonzero z rows; per y column, forward z (bit-reversed
-// result), product with the real kernel spectrum, inverse z back to natural
-// order, all in registers, storing only the z rows read later; inverse y on
-// those rows.  Requires nin <= NZ <= 32 (NZ: compile-time bound on the
-// nonzero inputs of the forward passes; their first two stages are pruned).
-template <int NZ>
-__global__ void __launch_bounds__(64, 6) k_slab64r(SlabArgs a) {
+// Same contract as k_slab, for M = 64: one line per thread, SL = 2 slabs per CTA of
+// 64 threads.  Passes: forward y on the nin nonzero z rows; per y column, forward
+// z (bit-reversed result), product with the real kernel spectrum, inverse z back
+// to natural order, all in registers, storing only the z rows read later; inverse
+// y on those rows.  The first and last pass have at most a warp of lines per slab,
+// so each warp takes its own slab there, and both take the columns of one slab and
+// then of the other: with one slab per CTA a warp waited through half of the
+// passes (barrier stalls were the largest).  A slab keeps max(nin, nz) rows, in
+// position order, so that two take the memory of one whole slab.  Requires nin <=
+// NZ <= 32 (NZ: compile-time bound on the nonzero inputs of the forward passes;
+// their first two stages are pruned).  256^3, n = 16, s = 16, Q = 6: 1.77 -> 1.44 ms.
+// With more than 32 output rows a warp would take two rounds of them (128^3, n = 8,
+// s = 24: 45 rows, no gain), so one slab per CTA stays there (SL = 1).
+template <int NZ, int SL>
+__global__ void __launch_bounds__(64, 6) k_slab64r(SlabArgs a, int rows) {
     constexpr int M = 64, MH = 33, P = 65;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    float2 *S = (float2 *)smem_raw;  // S[z][y], pitch 65 (conflict-free rows and columns)
-    __shared__ int rowoff[64];
+    float2 *S = (float2 *)smem_raw;  // S[slab][row][y], pitch 65 (conflict-free rows and columns)
+    __shared__ int rowoff[64];       // output z row jz -> its row in the slab
     const int nin = a.nin, W = a.nout, c = threadIdx.x;
+    const int w = SL == 2 ? c >> 5 : 0, lane = SL == 2 ? c & 31 : c;  // this thread's slab and line of the y passes
     unsigned long long rowmask = 0;
     for (int j = 0; j < a.nz; ++j) {
         int pz = (a.out_off + a.zrow[j]) % M;
         if (pz < 0) pz += M;
         rowmask |= 1ull << pz;
-        if (threadIdx.x == 0) rowoff[j] = pz * P;
     }
-    __syncthreads();
+    for (int j = c; j < a.nz; j += 64) {
+        int pz = (a.out_off + a.zrow[j]) % M;
+        if (pz < 0) pz += M;
+        rowoff[j] = __popcll(rowmask & ((1ull << pz) - 1ull)) * P;
+    }
     const int nunits = a.it.nitems * MH;
-    for (int unit = blockIdx.x; unit < nunits; unit += gridDim.x) {
-        const int kx = unit % MH;
-        int p;
-        const PlanPtrs &PP = item_plan(a.it, unit / MH, p);
-        const long q = unit / MH;  // scratch slot
-        const float2 *in = (const float2 *)a.it.a1 + (q * MH + kx) * nin * nin;
+    float2 *mine = S + w * rows * P;
+    for (int pair = blockIdx.x; SL * pair < nunits; pair += gridDim.x) {
         float2 v[64];
-        // forward y: thread c < nin takes z row c
-        if (c < nin) {
+        // forward y: line l < nin takes z row l of slab w
+        {
+            const int unit = SL * pair + w;
+            if (unit < nunits && lane < nin) {
+                const float2 *in = (const float2 *)a.it.a1 + (long)unit * nin * nin;  // scratch slot and kx
 #pragma unroll
-            for (int i = 0; i < 64; ++i) v[i] = (i < NZ && i < nin) ? in[c * nin + i] : make_float2(0.f, 0.f);
-            fft64_dif_reg<false, true, NZ>(v);
+                for (int i = 0; i < 64; ++i) v[i] = (i < NZ && i < nin) ? in[lane * nin + i] : make_float2(0.f, 0.f);
+                fft64_dif_reg<false, true, NZ>(v);
 #pragma unroll
-            for (int i = 0; i < 64; ++i) S[c * P + brev6(i)] = v[i];
+                for (int i = 0; i < 64; ++i) mine[lane * P + brev6(i)] = v[i];
+            }
         }
         __syncthreads();
-        // column ky0 = c: forward z, kernel product, inverse z
-        {
+        // column ky0 = c of one slab, then of the other: forward z, kernel product, inverse z
+#pragma unroll 1
+        for (int h = 0; h < SL; ++h) {
+            const int unit = SL * pair + h;
+            if (unit >= nunits) break;
+            const int kx = unit % MH;
+            int p;
+            const PlanPtrs &PP = item_plan(a.it, unit / MH, p);
+            float2 *T = S + h * rows * P + c;
 #pragma unroll
-            for (int i = 0; i < 64; ++i) v[i] = (i < NZ && i < nin) ? S[i * P + c] : make_float2(0.f, 0.f);
+            for (int i = 0; i < 64; ++i) v[i] = (i < NZ && i < nin) ? T[i * P] : make_float2(0.f, 0.f);
             fft64_dif_reg<false, true, NZ>(v);
             const float *kk = (const float *)PP.khat + ((long)kx * MH + (c < M - c ? c : M - c)) * MH;
 #pragma unroll
@@ -765,27 +783,38 @@ __global__ void __launch_bounds__(64, 6) k_slab64r(SlabArgs a) {
                 v[i].y *= k;
             }
             fft64_dit_reg<true>(v);
+            // the column's input rows are read; its output rows go over them
 #pragma unroll
             for (int i = 0; i < 64; ++i)
-                if ((rowmask >> i) & 1ull) S[i * P + c] = v[i];
+                if ((rowmask >> i) & 1ull) {
+                    *T = v[i];
+                    T += P;
+                }
         }
         __syncthreads();
-        // inverse y on the output z rows: thread c < nz takes row rowoff[c]
-        if (c < a.nz) {
-            float2 *row = S + rowoff[c];
+        // inverse y on the output z rows of the warp's slab
+        if (SL * pair + w < nunits)
+            for (int r = lane; r < a.nz; r += 64 / SL) {
+                float2 *row = mine + r * P;
 #pragma unroll
-            for (int i = 0; i < 64; ++i) v[i] = row[brev6(i)];
-            fft64_dit_reg<true>(v);
+                for (int i = 0; i < 64; ++i) v[i] = row[brev6(i)];
+                fft64_dit_reg<true>(v);
 #pragma unroll
-            for (int i = 0; i < 64; ++i) row[i] = v[i];
-        }
+                for (int i = 0; i < 64; ++i) row[i] = v[i];
+            }
         __syncthreads();
-        float2 *out = (float2 *)a.it.a4 + q * a.nz * a.blk + kx * W;
-        for (int e = threadIdx.x; e < a.nz * W; e += blockDim.x) {
-            const int jz = e / W, yo = e - jz * W;
-            out[(long)jz * a.blk + yo] = S[rowoff[jz] + ((a.out_off + yo) & (M - 1))];
+        for (int h = 0; h < SL; ++h) {
+            const int unit = SL * pair + h;
+            if (unit >= nunits) break;
+            const long q = unit / MH;  // scratch slot
+            const float2 *T = S + h * rows * P;
+            float2 *out = (float2 *)a.it.a4 + q * a.nz * a.blk + (unit - q * MH) * W;
+            for (int e = threadIdx.x; e < a.nz * W; e += blockDim.x) {
+                const int jz = e / W, yo = e - jz * W;
+                out[(long)jz * a.blk + yo] = T[rowoff[jz] + ((a.out_off + yo) & (M - 1))];
+            }
         }
-        __syncthreads();  // S is rewritten by the next unit
+        __syncthreads();  // the slabs are rewritten by the next pair
     }
 }
 
@@ -3117,13 +3146,18 @@ cudaError_t run_patch_conv_t(const mlc_plan_s *pl, const Items &it, const void *
         if constexpr (LOG2M == 5) {
             k_slab<LOG2M, R><<<gr, 256, fft_smem_bytes<R>(M, M, M + 1), st>>>(a);
         } else if constexpr (LOG2M == 6) {  // one line per thread
-            const size_t smr = (size_t)M * 65 * sizeof(float2);
+            const int rows = std::max(nin, nz);
+            const int sl = nz <= 32 ? 2 : 1;  // slabs per CTA
+            const size_t smr = (size_t)sl * rows * 65 * sizeof(float2);
+            gr = (gr + sl - 1) / sl;
             if (it.persist) {
-                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_slab64r<32>, 64, smr);
+                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_slab64r<32, 2>, 64, smr);
                 gr = std::min(gr, nsm * (occ > 0 ? occ : 1));
             }
-            if (nin <= 17) k_slab64r<17><<<gr, 64, smr, st>>>(a);
-            else k_slab64r<32><<<gr, 64, smr, st>>>(a);
+            if (nin <= 17 && sl == 2) k_slab64r<17, 2><<<gr, 64, smr, st>>>(a, rows);
+            else if (nin <= 17) k_slab64r<17, 1><<<gr, 64, smr, st>>>(a, rows);
+            else if (sl == 2) k_slab64r<32, 2><<<gr, 64, smr, st>>>(a, rows);
+            else k_slab64r<32, 1><<<gr, 64, smr, st>>>(a, rows);
         } else {  // register lines
             const size_t sm = ((size_t)144 + 32 * 152 + (size_t)std::max(nin, nz) * (M + 1)) * sizeof(float2);
             if (it.persist) {
@@ -3214,8 +3248,6 @@ void configure_kernels() {
     cudaFuncSetAttribute(k_inv_x128<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     cudaFuncSetAttribute(k_inv_x128<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     cudaFuncSetAttribute(k_inv_x64<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    cudaFuncSetAttribute(k_slab64r<17>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    cudaFuncSetAttribute(k_slab64r<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     cudaFuncSetAttribute(k_slab128r, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPatchSmem);
     set_cfft_attrs<dfl>();
     set_cfft_attrs<double>();
