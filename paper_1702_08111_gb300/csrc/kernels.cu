@@ -1411,6 +1411,117 @@ __device__ __forceinline__ void inv128_line(int t, const float2 (&w6)[8], const 
     __syncwarp(gm);
 }
 
+// Forward real transform along x of the patch charges for M = 128 (same output
+// and bits as k_fwd_x): 8-lane groups take one line each through the radix-2
+// stages in registers (as inv128_line, forward), the stage sums with the zeros
+// beyond n = 32 left out and only the half spectrum finished; the CTA gathers its
+// plane's lines in shared memory, so that the rows of a (kx, zi) leave whole.
+// One CTA per (patch, zi).  Bound by the 2.3 GB it writes (512^3, n = 32); the
+// shared-memory passes it replaces took 3.55 ms there, now 1.58.
+__global__ void __launch_bounds__(128) k_fwd_x128(FwdXArgs a) {
+    constexpr int M = 128, MH = 65, XP = 152;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    float2 *xs_all = (float2 *)smem_raw;       // 16 groups x XP
+    float2 *buf = xs_all + 16 * XP;            // [kx][line]
+    const int nin = a.nin, n = a.n, zi = blockIdx.x % nin;
+    int p;
+    const PlanPtrs &PP = item_plan(a.it, blockIdx.x / nin, p);
+    const int N = PP.N, np = PP.np;
+    const int i2 = p % np, i1 = (p / np) % np, i0 = p / (np * np);
+    const float *f = (const float *)PP.f;
+    const int grp = threadIdx.x >> 3, t = threadIdx.x & 7;
+    const unsigned gm = 0xffu << (threadIdx.x & 24);
+    float2 *xs = xs_all + grp * XP;
+    const float2 *tw = (const float2 *)a.tw;   // M/2 twiddles
+    float2 w6[5], w5[4], w4[2], w3, w2[4];
+#pragma unroll
+    for (int j = 0; j < 5; ++j) w6[j] = tw[t + 8 * j];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) w5[j] = tw[(t + 8 * j) << 1];
+#pragma unroll
+    for (int j = 0; j < 2; ++j) w4[j] = tw[(t + 8 * j) << 2];
+    w3 = tw[t << 3];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) w2[j] = tw[j << 4];
+    const int z = i0 * n + zi;
+    for (int l = grp; l < nin; l += 16) {
+        const int y = i1 * n + l;
+        float2 v[16];
+#pragma unroll
+        for (int j = 0; j < 5; ++j) {
+            const int m = t + 8 * j, x = i2 * n + m;
+            float c = 0.f;
+            if (m < nin && z < N && y < N && x < N) {
+                float w = (zi == 0 || zi == n) ? 0.5f : 1.f;
+                w *= (l == 0 || l == n) ? 0.5f : 1.f;
+                w *= (m == 0 || m == n) ? 0.5f : 1.f;
+                c = w * f[((long)z * N + y) * N + x];
+            }
+            v[j] = make_float2(c, 0.f);
+            v[j + 8] = cmul(v[j], w6[j]);
+        }
+#pragma unroll
+        for (int g = 0; g < 16; g += 8) {  // entries 5..7 of each half are zero
+            const float2 e0 = v[g], e4 = v[g + 4];
+            v[g] = cadd(e0, e4);
+            v[g + 4] = cmul(csub(e0, e4), w5[0]);
+#pragma unroll
+            for (int j = 1; j < 4; ++j) v[g + j + 4] = cmul(v[g + j], w5[j]);
+        }
+#pragma unroll
+        for (int g = 0; g < 16; g += 4)
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const float2 b = v[g + j], c = v[g + j + 2];
+                v[g + j] = cadd(b, c);
+                v[g + j + 2] = cmul(csub(b, c), w4[j]);
+            }
+#pragma unroll
+        for (int g = 0; g < 16; g += 2) {
+            const float2 b = v[g], c = v[g + 1];
+            v[g] = cadd(b, c);
+            v[g + 1] = cmul(csub(b, c), w3);
+        }
+#pragma unroll
+        for (int j = 0; j < 16; ++j) xs[9 * j + t] = v[j];
+        __syncwarp(gm);
+        const int kt = 2 * (int)(__brev((unsigned)t) >> 29);  // kx of entry 8 b + r: 16 brev(r) + kt + (b >= 8)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            float2 u[8];
+#pragma unroll
+            for (int r = 0; r < 8; ++r) u[r] = xs[9 * (t + 8 * h) + r];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const float2 b = u[r], c = u[r + 4];
+                u[r] = cadd(b, c);
+                u[r + 4] = r == 0 ? csub(b, c) : cmul(csub(b, c), w2[r]);
+            }
+#pragma unroll
+            for (int g = 0; g < 8; g += 4)
+#pragma unroll
+                for (int r = 0; r < 2; ++r) {
+                    const float2 b = u[g + r], c = u[g + r + 2];
+                    u[g + r] = cadd(b, c);
+                    u[g + r + 2] = r == 0 ? csub(b, c) : mul_mi(csub(b, c), false);
+                }
+#pragma unroll
+            for (int g = 0; g < 8; g += 2) {  // r even: kx < 64
+                const int kx = 16 * ((g & 4 ? 1 : 0) + (g & 2 ? 2 : 0)) + kt + h;
+                buf[kx * nin + l] = cadd(u[g], u[g + 1]);
+            }
+            if (h == 0 && t == 0) buf[64 * nin + l] = csub(u[0], u[1]);
+        }
+        __syncwarp(gm);
+    }
+    __syncthreads();
+    float2 *out = (float2 *)a.it.a1 + ((long)(blockIdx.x / nin) * MH * nin + zi) * nin;  // scratch slot = item
+    for (int e = threadIdx.x; e < MH * nin; e += blockDim.x) {
+        const int kx = e / nin, l = e - kx * nin;
+        out[(long)kx * nin * nin + l] = buf[e];
+    }
+}
+
 // Pruned inverse real transform along x for M = 128 (same contract and bits as
 // k_inv_x_pruned): 8-lane groups take one needed row each, entirely in registers,
 // and store their results directly.  Rows that are read only at multiples of 4
@@ -1591,58 +1702,65 @@ __global__ void __launch_bounds__(128) k_inv_x128(InvXPArgs a) {
 }
 
 // Pruned inverse real transform along x for M = 64 (same contract as
-// k_inv_x_pruned; local fields leave in the working precision R).  The needed
-// rows go in pairs: with A, B the Hermitian half spectra of two rows,
-// Z = A + iB transforms to a + ib, so one complex 64-point register transform
-// (radix 8 x 8, 8-thread group) yields both real rows; the Hermitian expansion
-// happens in the loads.  The per-x output classification comes from a
-// 64-entry table built once per CTA.
-template <typename R>
-__global__ void __launch_bounds__(128, sizeof(R) == 4 ? 8 : 4) k_inv_x64(InvXPArgs a) {
-    using C = typename Cx<R>::T;
+// k_inv_x_pruned, Q = 4 and 6).  The needed rows go in pairs: with A, B the
+// Hermitian half spectra of two rows, Z = A + iB transforms to a + ib, so one
+// complex 64-point register transform (radix 8 x 8, 8-thread group) yields both
+// real rows; the Hermitian expansion happens in the loads.  Lane t of a group
+// ends with the positions t + 8 k of both rows and stores them from there, eight
+// neighbouring values per store, with the classes of each position from a table.
+// 256^3, n = 16, s = 16, Q = 6: 0.84 -> 0.76 ms against a version that passed
+// the rows through shared memory to threads in output order.
+__global__ void __launch_bounds__(128, 8) k_inv_x64(InvXPArgs a) {
     constexpr int M = 64, MH = 33;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ int rows[64], rinfo[64];  // needed rows; their class bits (1 alpha, 2 plane, 4 coarse) | slot << 3
+    __shared__ int rows[64];
     __shared__ int nfft_s;
     __shared__ unsigned wmask[2];
-    __shared__ int xflag[M], xplane[M], xcoarse[M];  // per x position: class bits, face-plane slot, coarse index
-    const int W = a.W, n = a.n, s = a.s, ga = a.ga, pl0 = a.pl0, wa = a.wa, nc = a.nc;
-    C *tw = (C *)smem_raw;        // M twiddles
-    C *raw = tw + M;              // MH x W (block of a.blk entries, 16-byte aligned)
-    C *xs = raw + a.blk;          // blockDim/8 groups x 72 exchange entries
-    constexpr int RP = 68;           // row pitch of rbuf: 4 (mod 16) keeps the group stores conflict-free
-    R *rbuf = (R *)(xs + (blockDim.x >> 3) * 72);  // transformed real rows (up to maxfft rows)
+    __shared__ int xinfo[M];  // per x position: class bits (1 alpha, 2 plane, 4 coarse) | plane slot << 3 | coarse index << 16
+    __shared__ unsigned long long bar;
+    const int W = a.W, n = a.n, s = a.s, ga = a.ga, pl0 = a.pl0, wa = a.wa, nc = a.nc, npa = a.npa;
+    float2 *tw = (float2 *)smem_raw;  // M twiddles
+    float2 *raw = tw + M;             // MH x W (block of a.blk entries, 16-byte aligned)
+    float2 *xs = raw + a.blk;         // blockDim/8 groups x 72 exchange entries
     const int jz = blockIdx.x % a.nz, zi = a.zrow[jz];
     int p;
     const PlanPtrs &PP = item_plan(a.it, blockIdx.x / a.nz, p);
     const int z = zi - s;
-    const C *twg = (const C *)a.tw;
+    const float2 *twg = (const float2 *)a.tw;
     for (int j = threadIdx.x; j < M; j += blockDim.x) {
-        C w = twg[j & (M / 2 - 1)];
+        float2 w = twg[j & (M / 2 - 1)];
         if (j >= M / 2) { w.x = -w.x; w.y = -w.y; }
         tw[j] = w;
     }
-    const C *in = (const C *)a.it.a4 + ((long)(blockIdx.x / a.nz) * a.nz + jz) * a.blk;  // scratch slot = item
-    // stage the contiguous block with one TMA bulk copy
-    __shared__ unsigned long long bar;
-    const unsigned bytes = (unsigned)(a.blk * sizeof(C));
-    if (threadIdx.x == 0) {
+    const float2 *in = (const float2 *)a.it.a4 + ((long)(blockIdx.x / a.nz) * a.nz + jz) * a.blk;  // scratch slot = item
+    const unsigned bytes = (unsigned)(a.blk * sizeof(float2));
+    if (threadIdx.x == 0) {  // stage the contiguous block with one bulk copy
         mbar_init(&bar, 1);
         mbar_expect_tx(&bar, bytes);
         if (!a.skip_copy) bulk_g2s(raw, in, bytes, &bar);
     }
     const int kl = -s / 4;
-    // x classification: bit 0 in the field box, 1 in alpha, 2 on a face plane, 3 coarse
+    const bool zP = on_plane(z, n, ga, pl0), zA = in_alpha(z, n, ga), zC = (z & 3) == 0;
     if (threadIdx.x < M) {
         const int pos = threadIdx.x;
         const int x = pos <= n + s ? pos : pos - M;
-        const bool box = x >= -s && x <= n + s;
-        const bool xA = in_alpha(x, n, ga), xP = on_plane(x, n, ga, pl0), xC = (x & 3) == 0;
-        xflag[pos] = box ? (1 | (xA ? 2 : 0) | (xP ? 4 : 0) | (xC ? 8 : 0)) : 0;
-        xplane[pos] = xP ? (x - pl0) / n : 0;
-        xcoarse[pos] = (x >> 2) - kl;
+        const bool box = x >= -s && x <= n + s, xA = in_alpha(x, n, ga), xP = on_plane(x, n, ga, pl0);
+        xinfo[pos] = box ? ((xA ? 1 : 0) | (xP ? 2 : 0) | ((x & 3) == 0 ? 4 : 0) | ((xP ? (x - pl0) / n : 0) << 3) |
+                            (((x >> 2) - kl) << 16))
+                         : 0;
+        // rows of this z that need a full transform, compacted with warp ballots (W <= 64)
+        const int y = pos - s;
+        const bool need = pos < W && ((zP && in_alpha(y, n, ga)) || (on_plane(y, n, ga, pl0) && zA) || (zC && (y & 3) == 0));
+        const unsigned m = __ballot_sync(0xffffffffu, need);
+        if ((pos & 31) == 0) wmask[pos >> 5] = m;
     }
     __syncthreads();
+    if (threadIdx.x < M) {
+        const int yi = threadIdx.x, lane = yi & 31;
+        const unsigned m0 = wmask[0], m1 = wmask[1], mine = yi < 32 ? m0 : m1;
+        if ((mine >> lane) & 1u) rows[(yi < 32 ? 0 : __popc(m0)) + __popc(mine & ((1u << lane) - 1u))] = yi;
+        if (yi == 0) nfft_s = __popc(m0) + __popc(m1);
+    }
     const bool arrived = mbar_wait_bounded(&bar, 0, a.wait_tries);
     if (__syncthreads_or(!arrived)) {  // uniform decision for the whole CTA
         if (threadIdx.x == 0) {
@@ -1651,56 +1769,27 @@ __global__ void __launch_bounds__(128, sizeof(R) == 4 ? 8 : 4) k_inv_x64(InvXPAr
         }
         return;
     }
-    const bool zP = on_plane(z, n, ga, pl0), zA = in_alpha(z, n, ga), zC = (z & 3) == 0;
-    // rows of this z that need a full transform, compacted with warp ballots (W <= 64)
-    if (threadIdx.x < 64) {
-        const int yi = threadIdx.x, y = yi - s;
-        const bool yA = in_alpha(y, n, ga), yP = on_plane(y, n, ga, pl0), yC = (y & 3) == 0;
-        // outer: the rows one node off a face plane too (their x values off the
-        // face planes come from direct sums below, like the face-plane ones)
-        const bool zQ = zP || (a.outer && off_slot(z, n, ga, pl0, a.npa) >= 0);
-        const bool yQ = yP || (a.outer && off_slot(y, n, ga, pl0, a.npa) >= 0);
-        const bool need = yi < W && ((zQ && yA) || (yQ && zA) || (zC && yC));
-        const unsigned m = __ballot_sync(0xffffffffu, need);
-        if ((threadIdx.x & 31) == 0) wmask[threadIdx.x >> 5] = m;
-    }
-    __syncthreads();
-    if (threadIdx.x < 64) {
-        const int yi = threadIdx.x;
-        const unsigned m0 = wmask[0], m1 = wmask[1];
-        const unsigned mine = yi < 32 ? m0 : m1;
-        const int lane = yi & 31;
-        if ((mine >> lane) & 1u) {
-            const int before = (yi < 32 ? 0 : __popc(m0)) + __popc(mine & ((1u << lane) - 1u));
-            const int y = yi - s;
-            const bool yA = in_alpha(y, n, ga), yP = on_plane(y, n, ga, pl0), yC = (y & 3) == 0;
-            rows[before] = yi;
-            rinfo[before] = (yA ? 1 : 0) | (yP ? 2 : 0) | (yC ? 4 : 0) | ((yP ? (y - pl0) / n : 0) << 3);
-        }
-        if (yi == 0) nfft_s = __popc(m0) + __popc(m1);
-    }
-    __syncthreads();
     const int nfft = nfft_s, npair = (nfft + 1) / 2;
-    R *cl = (R *)PP.cl + (long)p * nc * nc * nc;
-    R *fp = (R *)PP.fp + (long)p * 3 * a.npa * wa * wa;
-    const int zc = (z >> 2) - kl, jz0 = zP ? (z - pl0) / n : 0;
+    float *cl = (float *)PP.cl + (long)p * nc * nc * nc;
+    float *fp = (float *)PP.fp + (long)p * 3 * npa * wa * wa;
+    const long ncl = (long)nc * nc * nc, nfp = 3L * npa * wa * wa;
     const int grp = threadIdx.x >> 3, t = threadIdx.x & 7, ngrp = blockDim.x >> 3;
-    C *gx = xs + grp * 72;
-    C wt[8];
+    float2 *gx = xs + grp * 72;
+    float2 wt[8];
 #pragma unroll
     for (int k1 = 0; k1 < 8; ++k1) wt[k1] = tw[(t * k1) & 63];
-    const C zero = Cx<R>::mk(0, 0);
+    const float2 zero = make_float2(0.f, 0.f);
     for (int q0 = 0; q0 < npair; q0 += ngrp) {  // uniform trip count across the CTA
         const int q = q0 + grp;
         const bool valid = q < npair;
         const int ya = valid ? rows[2 * q] : 0;
         const bool hasb = valid && 2 * q + 1 < nfft;
         const int yb = hasb ? rows[2 * q + 1] : 0;
-        C v[8];
+        float2 v[8];
 #pragma unroll
         for (int n2 = 0; n2 < 8; ++n2) {
             const int k = 8 * n2 + t;
-            C A = zero, B = zero;
+            float2 A = zero, B = zero;
             if (valid) {
                 if (k < MH) {
                     A = raw[k * W + ya];
@@ -1714,69 +1803,48 @@ __global__ void __launch_bounds__(128, sizeof(R) == 4 ? 8 : 4) k_inv_x64(InvXPAr
             v[n2].x = A.x - B.y;  // Z = A + i B
             v[n2].y = A.y + B.x;
         }
-        line64_regs<C, R, false>(v, t, wt, true, gx);
-        if (valid) {
+        line64_regs<float2, float, false>(v, t, wt, true, gx);
+        for (int h = 0; h < 2; ++h) {
+            if (!(h ? hasb : valid)) continue;
+            const int y = (h ? yb : ya) - s;
+            const bool yA = in_alpha(y, n, ga), yP = on_plane(y, n, ga, pl0), yC = (y & 3) == 0;
+            const long c0 = zC && yC ? ((long)((z >> 2) - kl) * nc + ((y >> 2) - kl)) * nc : -1;
+            const long a0 = zP && yA ? ((long)((z - pl0) / n) * wa + (y + ga)) * wa + ga : -1;
+            const long a1 = yP && zA ? ((long)(npa + (y - pl0) / n) * wa + (z + ga)) * wa + ga : -1;
+            const long a2 = zA && yA ? ((long)(2 * npa) * wa + (z + ga)) * wa + (y + ga) : -1;
 #pragma unroll
             for (int k2 = 0; k2 < 8; ++k2) {
-                rbuf[(2 * q) * RP + t + 8 * k2] = v[k2].x;
-                if (hasb) rbuf[(2 * q + 1) * RP + t + 8 * k2] = v[k2].y;
+                const int pos = t + 8 * k2, xf = xinfo[pos], x = pos <= n + s ? pos : pos - M;
+                const float val = h ? v[k2].y : v[k2].x;
+                if ((xf & 4) && c0 >= 0 && in_range(c0 + (xf >> 16), ncl, PP.err)) cl[c0 + (xf >> 16)] = val;
+                if (xf & 1) {
+                    if (a0 >= 0 && in_range(a0 + x, nfp, PP.err)) fp[a0 + x] = val;
+                    if (a1 >= 0 && in_range(a1 + x, nfp, PP.err)) fp[a1 + x] = val;
+                }
+                if ((xf & 2) && a2 >= 0) {
+                    const long i = a2 + (long)((xf >> 3) & 0xff) * wa * wa;
+                    if (in_range(i, nfp, PP.err)) fp[i] = val;
+                }
             }
         }
     }
-    __syncthreads();
-    // outputs of the transformed rows (consecutive x per thread: coalesced stores)
-    const int dl = blockDim.x / W, dxi = blockDim.x - dl * W;
-    for (int e = threadIdx.x, l = e / W, xi = e - l * W; l < nfft; xi += dxi, l += dl) {
-        if (xi >= W) { xi -= W; ++l; if (l >= nfft) break; }
-        const int yi = rows[l], yf = rinfo[l];
-        const int x = xi - s, y = yi - s;
-        const int pos = x & (M - 1), xf = xflag[pos];
-        const bool yA = yf & 1, yP = yf & 2, yC = yf & 4;
-        const bool xA = xf & 2, xP = xf & 4, xC = xf & 8;
-        const bool wC = zC && yC && xC, w0 = zP && yA && xA, w1 = yP && zA && xA, w2 = zA && yA && xP;
-        int o0 = -1, o1 = -1, o2 = -1;
-        if (a.outer && xA && yA && zA) {
-            o0 = off_slot(z, n, ga, pl0, a.npa);
-            o1 = off_slot(y, n, ga, pl0, a.npa);
-            o2 = off_slot(x, n, ga, pl0, a.npa);
-        }
-        if (!(wC || w0 || w1 || w2 || o0 >= 0 || o1 >= 0 || o2 >= 0)) continue;
-        const R val = rbuf[l * RP + pos];
-        const long ncl = (long)nc * nc * nc, nfp = 3L * a.npa * wa * wa;
-        if (wC) {
-            const long i = ((long)zc * nc + ((y >> 2) - kl)) * nc + xcoarse[pos];
-            if (in_range(i, ncl, PP.err)) cl[i] = val;
-        }
-        if (w0) {
-            const long i = (((long)jz0) * wa + (y + ga)) * wa + (x + ga);
-            if (in_range(i, nfp, PP.err)) fp[i] = val;
-        }
-        if (w1) {
-            const long i = (((long)(a.npa + (yf >> 3))) * wa + (z + ga)) * wa + (x + ga);
-            if (in_range(i, nfp, PP.err)) fp[i] = val;
-        }
-        if (w2) {
-            const long i = (((long)(2 * a.npa + xplane[pos])) * wa + (z + ga)) * wa + (y + ga);
-            if (in_range(i, nfp, PP.err)) fp[i] = val;
-        }
-    }
-    // rows that only need x on the face planes: direct sums over the half spectrum
-    if (zA) {
-        for (int e = threadIdx.x; e < W * a.npa; e += blockDim.x) {
-            const int yi = e / a.npa, j = e % a.npa;
-            const int y = yi - s;
-            const bool yA = in_alpha(y, n, ga), yP = on_plane(y, n, ga, pl0), yC = (y & 3) == 0;
-            if (!yA || zP || yP || (zC && yC)) continue;  // not needed, or done by an FFT row
-            const int x = pl0 + j * n;
-            const int pos = x & (M - 1);
-            R acc = R(0.0);
+    // rows that only need x on the face planes: direct sums over the half
+    // spectrum, neighbouring threads on neighbouring rows
+    if (zA && !zP) {
+        const int na = n + 2 * ga + 1;
+        for (int e = threadIdx.x; e < na * npa; e += blockDim.x) {
+            const int y = e % na - ga, j = e / na, yi = y + s;
+            if (on_plane(y, n, ga, pl0) || (zC && (y & 3) == 0)) continue;  // done by a transformed row
+            const int pos = (pl0 + j * n) & (M - 1);
+            float acc = 0.f;
             for (int k = 0; k < MH; ++k) {
-                const C X = raw[k * W + yi];
-                C w = tw[(k * pos) & (M - 1)];  // exp(+2 pi i k pos / M) = conj(tw)
-                const R re = X.x * w.x + X.y * w.y;
-                acc += (k == 0 || 2 * k == M) ? re : R(2.0) * re;
+                const float2 X = raw[k * W + yi];
+                const float2 w = tw[(k * pos) & (M - 1)];  // exp(+2 pi i k pos / M) = conj(tw)
+                const float re = X.x * w.x + X.y * w.y;
+                acc += (k == 0 || 2 * k == M) ? re : 2.f * re;
             }
-            fp[(((long)(2 * a.npa + j)) * wa + (z + ga)) * wa + (y + ga)] = acc;
+            const long i = (((long)(2 * npa + j)) * wa + (z + ga)) * wa + (y + ga);
+            if (in_range(i, nfp, PP.err)) fp[i] = acc;
         }
     }
 }
@@ -3106,8 +3174,7 @@ template <int LOG2M>
 void set_patch_attrs() {
     const int big = 200 * 1024;
     cudaFuncSetAttribute(k_fwd_x<LOG2M, float, true, float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
-    if constexpr (LOG2M < 7)
-        cudaFuncSetAttribute(k_inv_x_pruned<LOG2M, float, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
+    cudaFuncSetAttribute(k_inv_x_pruned<LOG2M, float, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
 }
 
 // Local convolutions of a set of patches: forward x (real), fused slab (y,
@@ -3121,7 +3188,9 @@ cudaError_t run_patch_conv_t(const mlc_plan_s *pl, const Items &it, const void *
     mark(pl, 1, st);
     {
         FwdXArgs a{nullptr, nullptr, 0, g.n, 0, nin, nin, tw, it};
-        if (LOG2M == 6 && nin <= 24) {  // register transform of line pairs
+        if constexpr (LOG2M == 7) {  // nin <= 33
+            k_fwd_x128<<<nb * nin, 128, ((size_t)16 * 152 + (size_t)MH * nin) * sizeof(float2), st>>>(a);
+        } else if (LOG2M == 6 && nin <= 24) {  // register transform of line pairs
             k_fwd_x64<float, R><<<nb, 256, 0, st>>>(a);
         } else {
             dim3 grid(nb * nin, 1);
@@ -3207,9 +3276,8 @@ cudaError_t run_patch_conv_t(const mlc_plan_s *pl, const Items &it, const void *
         const size_t sm = fixed + (size_t)a.rb * line;
         if (LOG2M == 6 && !g.wide) {
             const int thr = 128;  // 16 line groups: one pass over the row pairs of a z row
-            const size_t sm64 = ((size_t)M + (size_t)g.a4blk + (thr / 8) * 72) * sizeof(typename Cx<R>::T) +
-                                (size_t)a.maxfft * 68 * sizeof(R);
-            k_inv_x64<R><<<nb * a.nz, thr, sm64, st>>>(a);
+            const size_t sm64 = ((size_t)M + (size_t)g.a4blk + (thr / 8) * 72) * sizeof(float2);
+            k_inv_x64<<<nb * a.nz, thr, sm64, st>>>(a);
         } else if constexpr (LOG2M == 7) {
             const size_t sm128 = ((size_t)M + (size_t)g.a4blk + 16 * 152) * sizeof(float2);
             if (g.wide) k_inv_x128<true><<<nb * a.nz, 128, sm128, st>>>(a);
@@ -3244,10 +3312,9 @@ cudaError_t launch_set_ptrs(PlanPtrs *d, const void *f, double *phi, cudaStream_
 void configure_kernels() {
     set_patch_attrs<5>();
     set_patch_attrs<6>();
-    set_patch_attrs<7>();
     cudaFuncSetAttribute(k_inv_x128<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     cudaFuncSetAttribute(k_inv_x128<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    cudaFuncSetAttribute(k_inv_x64<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    cudaFuncSetAttribute(k_inv_x64, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     cudaFuncSetAttribute(k_slab128r, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPatchSmem);
     set_cfft_attrs<dfl>();
     set_cfft_attrs<double>();
