@@ -3335,10 +3335,8 @@ void configure_kernels() {
     MLC_DIR_ATTR(32)
 #undef MLC_DIR_ATTR
 #define MLC_RES_ATTR(KK)                                                                            \
-    cudaFuncSetAttribute(k_resid<dfl, dfl, KK>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);    \
     cudaFuncSetAttribute(k_resid<float, dfl, KK>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);  \
-    cudaFuncSetAttribute(k_resid<float, double, KK>, cudaFuncAttributeMaxDynamicSharedMemorySize, big); \
-    cudaFuncSetAttribute(k_resid<double, double, KK>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
+    cudaFuncSetAttribute(k_resid<float, double, KK>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
     MLC_RES_ATTR(4)
     MLC_RES_ATTR(6)
     MLC_RES_ATTR(8)
@@ -3433,6 +3431,8 @@ const void *ring_moments(const mlc_plan_s *pl) {
 cudaError_t launch_resid(const mlc_plan_s *pl, const Items &it, cudaStream_t st) {
     NvtxRange nvtx("mlc:residuals");
     const Geom &g = pl->g;
+    // FP64 and double-float: the products of limb_conv.cu give the residuals themselves
+    if (g.conv != CONV_F32) return launch_resid_outer(pl, it, st);
     ResArgs a{};
     a.it = it; a.n = g.n; a.s = g.s; a.ga = g.ga; a.b = g.b;
     a.npa = g.npa; a.pl0 = g.pl0; a.wa = g.wa; a.nc = g.nc;
@@ -3442,13 +3442,8 @@ cudaError_t launch_resid(const mlc_plan_s *pl, const Items &it, cudaStream_t st)
     const size_t sm = 8 * (size_t)nk * (g.wa + nk);
     dim3 grid(it.nitems, 3 * g.npa);
 #define MLC_RES(KK)                                                                         \
-    if (g.fine == FINE_F64) {                                                               \
-        if (g.conv == CONV_F32) k_resid<float, double, KK><<<grid, 256, sm, st>>>(a);       \
-        else k_resid<double, double, KK><<<grid, 256, sm, st>>>(a);                         \
-    } else {                                                                                \
-        if (g.conv == CONV_F32) k_resid<float, dfl, KK><<<grid, 256, sm, st>>>(a);          \
-        else k_resid<dfl, dfl, KK><<<grid, 256, sm, st>>>(a);                               \
-    }
+    if (g.fine == FINE_F64) k_resid<float, double, KK><<<grid, 256, sm, st>>>(a);           \
+    else k_resid<float, dfl, KK><<<grid, 256, sm, st>>>(a);
     switch (2 * g.b + 2) {
         case 4: MLC_RES(4) break;
         case 6: MLC_RES(6) break;

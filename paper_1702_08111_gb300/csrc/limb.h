@@ -163,10 +163,12 @@ struct LimbPlanes {
 };
 
 // Geometry of the folded local convolution of one patch.  Rows of a table, in
-// order: the coarse lattice, then per axis the face planes, then per axis the
-// off-face planes; in-plane axes in increasing order.
+// order: the coarse lattice, then per axis the face planes (the residual phi^i -
+// I^H(phi^i), which is as linear in the charge as the field, so that no later pass
+// forms it), then per axis the off-face planes (the field); in-plane axes in
+// increasing order.
 struct LimbConvGeom {
-    int n, s, ga, nc, wa;
+    int n, s, ga, b, nc, wa;
     int hin[2];      // input reps along an axis: even n/2 + 1, odd n/2
     int hl[2];       // lattice reps, even (the centre included) and odd
     int hp[2];       // in-plane reps
@@ -201,15 +203,16 @@ __host__ __device__ inline int limb_plane_base(const LimbConvGeom &g, int u, int
         }
     return r;
 }
-// Fine coordinates (relative to the patch, table axes) of a row.
-__host__ __device__ inline void limb_row_point(const LimbConvGeom &g, int u, int row, int x[3]) {
+// Fine coordinates (relative to the patch, table axes) of a row; returns 0 for a
+// lattice point, 1 + axis for a face plane, 4 + axis for an off-face plane.
+__host__ __device__ inline int limb_row_point(const LimbConvGeom &g, int u, int row, int x[3]) {
     const int nl = limb_lat_rows(g, u);
     if (row < nl) {
         const int d2 = g.hl[limb_odd(u, 2)], d1 = g.hl[limb_odd(u, 1)];
         x[2] = -g.s + 4 * (row % d2);
         x[1] = -g.s + 4 * ((row / d2) % d1);
         x[0] = -g.s + 4 * (row / (d2 * d1));
-        return;
+        return 0;
     }
     row -= nl;
     for (int k = 0; k < 2; ++k)
@@ -222,11 +225,12 @@ __host__ __device__ inline void limb_row_point(const LimbConvGeom &g, int u, int
                 x[i2] = -g.ga + row % d2;
                 x[i1] = -g.ga + (row / d2) % d1;
                 x[a] = pl.c[row / (d2 * d1)];
-                return;
+                return 1 + 3 * k + a;
             }
             row -= m;
         }
     x[0] = x[1] = x[2] = 0;
+    return 0;
 }
 // Input rep (table axes) of column k of a table.
 __host__ __device__ inline void limb_col_point(const LimbConvGeom &g, int u, int k, int m[3]) {

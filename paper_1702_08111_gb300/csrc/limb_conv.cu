@@ -5,7 +5,8 @@
 //   k_limb_fold     charge -> even / odd parts along the three axes -> digits
 //   k_limb_gemm     per parity class, outputs x inputs by inputs x patches
 //   k_limb_unfold   even / odd outputs -> the coarse lattice of the field box
-//                   and the face planes (Q = 10: and the planes next to them)
+//                   and the residuals phi^i - I^H(phi^i) on the face planes (Q =
+//                   10: and the fields on the planes next to them)
 //
 // Only the values the later steps read are formed: a quarter of the field box
 // per axis for the lattice and a few planes of the inner box, 5947 of 117649
@@ -33,47 +34,92 @@ namespace mlc {
 namespace {
 
 // ---------------------------------------------------------------------------
-// Tables: one CTA per row of one table.  Entry (row, k) is the Green's function
-// (h = 1) between the row's point and the column's, folded along each axis:
-// 1/8 sum over the mirror images of the input point, negative along odd axes.
+// Tables.  Entry (row, k) is the Green's function (h = 1) between the row's point
+// and the column's, folded along each axis: 1/8 sum over the mirror images of the
+// input point, negative along odd axes.  Rows of face planes have the interpolant
+// of the lattice entries of their plane subtracted (R4: tensor-product Lagrange in
+// the plane).
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_limb_table(LimbConvGeom g, int u, const double *G1, int L, unsigned char *A,
-                                                    double *rf) {
+__device__ __forceinline__ double folded_green(const LimbConvGeom &g, int u, const double *G1, int L, const int (&x)[3],
+                                               int k) {
+    int m[3];
+    limb_col_point(g, u, k, m);
+    double v = 0.0;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+        long idx = 0;
+        bool neg = false;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            const bool mir = (c >> d) & 1;
+            const int lag = abs(x[d] - (mir ? g.n - m[d] : m[d]));
+            idx = idx * (L + 1) + lag;
+            neg ^= mir && limb_odd(u, d);
+        }
+        const double q = G1[idx];
+        v += neg ? -q : q;
+    }
+    return 0.125 * v;
+}
+
+// Entries of the lattice rows, [row][kst x 16]: one CTA per row.
+__global__ void __launch_bounds__(256) k_limb_lattice(LimbConvGeom g, int u, const double *G1, int L, double *Lv) {
+    int x[3];
+    limb_row_point(g, u, blockIdx.x, x);
+    for (int k = threadIdx.x; k < g.K[u]; k += blockDim.x)
+        Lv[(long)blockIdx.x * g.K[u] + k] = folded_green(g, u, G1, L, x, k);
+}
+
+struct LagrangeRows {
+    double w[4][12];  // weights of I^H for a coordinate mod 4 (lagrange_rows)
+};
+
+// Digits of one table: one CTA per row.
+__global__ void __launch_bounds__(256) k_limb_table(LimbConvGeom g, int u, const double *G1, int L, const double *Lv,
+                                                    const __grid_constant__ LagrangeRows lag, unsigned char *A, double *rf) {
     extern __shared__ double val[];  // kst x 16
     __shared__ int smax;
+    __shared__ int st_row[144];      // lattice rows of the interpolation stencil and their weights
+    __shared__ double st_w[144];
     const int row = blockIdx.x, K = g.K[u], kpad = g.kst[u] * 16, n = g.n;
     if (threadIdx.x == 0) smax = 0;
+    int x[3] = {0, 0, 0}, kind = 0, terms = 0;
+    if (row < g.rows[u]) kind = limb_row_point(g, u, row, x);
+    if (kind >= 1 && kind <= 3) {
+        const int S = 2 * g.b + 2, ax = kind - 1, iu = ax == 0 ? 1 : 0, iv = ax == 2 ? 1 : 2;
+        terms = S * S;
+        for (int e = threadIdx.x; e < terms; e += blockDim.x) {
+            const int j[2] = {e / S, e % S}, axes[2] = {iu, iv};
+            int i[3];
+            double w = 1.0;
+            i[ax] = (x[ax] + g.s) / 4;
+            for (int q = 0; q < 2; ++q) {
+                const int c = x[axes[q]], r = c & 3;
+                // a coordinate on the lattice is its own stencil (weight 1 at j = 0)
+                const int X = r == 0 ? c : 4 * ((c >> 2) - g.b + j[q]);
+                w *= r == 0 ? (j[q] == 0 ? 1.0 : 0.0) : lag.w[r][j[q]];
+                const bool mir = 2 * X > n, odd = limb_odd(u, axes[q]);
+                if (odd && 2 * X == n) w = 0.0;  // odd parts vanish at the centre
+                if (odd && mir) w = -w;
+                i[axes[q]] = w == 0.0 ? 0 : ((mir ? n - X : X) + g.s) / 4;
+            }
+            st_row[e] = w == 0.0 ? 0 : limb_lat_row(g, u, i[0], i[1], i[2]);
+            st_w[e] = w;
+        }
+    }
     __syncthreads();
     int mx = 0;
-    if (row < g.rows[u]) {
-        int x[3];
-        limb_row_point(g, u, row, x);
-        for (int k = threadIdx.x; k < kpad; k += blockDim.x) {
-            double v = 0.0;
-            if (k < K) {
-                int m[3];
-                limb_col_point(g, u, k, m);
-#pragma unroll
-                for (int c = 0; c < 8; ++c) {
-                    long idx = 0;
-                    bool neg = false;
-#pragma unroll
-                    for (int d = 0; d < 3; ++d) {
-                        const bool mir = (c >> d) & 1;
-                        const int lag = abs(x[d] - (mir ? n - m[d] : m[d]));
-                        idx = idx * (L + 1) + lag;
-                        neg ^= mir && limb_odd(u, d);
-                    }
-                    const double q = G1[idx];
-                    v += neg ? -q : q;
-                }
-                v *= 0.125;
-            }
-            val[k] = v;
-            mx = max(mx, biased_exp(v));
+    for (int k = threadIdx.x; k < kpad; k += blockDim.x) {
+        double v = 0.0;
+        if (k < K && row < g.rows[u]) {
+            v = kind == 0 ? Lv[(long)row * K + k] : folded_green(g, u, G1, L, x, k);
+            double iv = 0.0;
+            for (int e = 0; e < terms; ++e)
+                if (st_w[e] != 0.0) iv = fma(st_w[e], Lv[(long)st_row[e] * K + k], iv);
+            v -= iv;
         }
-    } else {
-        for (int k = threadIdx.x; k < kpad; k += blockDim.x) val[k] = 0.0;
+        val[k] = v;
+        mx = max(mx, biased_exp(v));
     }
     mx = __reduce_max_sync(0xffffffffu, mx);
     if ((threadIdx.x & 31) == 0) atomicMax(&smax, mx);
@@ -272,7 +318,7 @@ __global__ void __launch_bounds__(256) k_limb_unfold(const __grid_constant__ Unf
     for (int kind = 0; kind < 2; ++kind) {  // face planes, then the planes next to them
         const LimbPlanes &pl = kind ? g.off : g.face;
         if (!pl.nrep) continue;
-        TO *fp = (TO *)(kind ? PP.fp2 : PP.fp) + (long)p * 3 * pl.per_axis * wa * wa;
+        TO *fp = (TO *)(kind ? PP.fp2 : PP.resid) + (long)p * 3 * pl.per_axis * wa * wa;
         const int hp = g.hp[0], centre = n / 2 + g.ga;
         for (int ax = 0; ax < 3; ++ax) {
             const int cen[3] = {ax == 0 ? -1 : centre, ax == 1 ? -1 : centre, ax == 2 ? -1 : centre};
@@ -303,10 +349,10 @@ __global__ void __launch_bounds__(256) k_limb_unfold(const __grid_constant__ Unf
 }
 
 struct TabKey {
-    int device, n, s, ga, wide;
+    int device, n, s, ga, b, wide;
     const double *dgf;
     bool operator<(const TabKey &o) const {
-        return std::tie(device, n, s, ga, wide, dgf) < std::tie(o.device, o.n, o.s, o.ga, o.wide, o.dgf);
+        return std::tie(device, n, s, ga, b, wide, dgf) < std::tie(o.device, o.n, o.s, o.ga, o.b, o.wide, o.dgf);
     }
 };
 std::mutex g_tab_mu;
@@ -323,7 +369,7 @@ bool limb_conv_geometry(const Geom &G, bool share, LimbConvGeom &c) {
     c = LimbConvGeom{};
     c.share = share;
     const int n = G.n, s = G.s, ga = G.ga;
-    c.n = n; c.s = s; c.ga = ga; c.nc = G.nc; c.wa = G.wa;
+    c.n = n; c.s = s; c.ga = ga; c.b = G.b; c.nc = G.nc; c.wa = G.wa;
     c.hin[0] = n / 2 + 1; c.hin[1] = n / 2;
     c.hl[0] = (n / 2 + s) / 4 + 1;
     c.hl[1] = c.hl[0] - ((n / 2 + s) % 4 == 0 ? 1 : 0);
@@ -371,7 +417,7 @@ bool limb_conv_geometry(const Geom &G, bool share, LimbConvGeom &c) {
 cudaError_t limb_conv_tables(int device, const Geom &G, bool share, const double *dgf, int dgf_L,
                              std::shared_ptr<LimbConvTables> *out) {
     std::lock_guard<std::mutex> lk(g_tab_mu);
-    const TabKey key{device, G.n, G.s, G.ga, G.wide ? 1 : 0, dgf};
+    const TabKey key{device, G.n, G.s, G.ga, G.b, G.wide ? 1 : 0, dgf};
     if (auto have = g_tabs[key].lock()) {
         *out = have;
         return cudaSuccess;
@@ -384,12 +430,26 @@ cudaError_t limb_conv_tables(int device, const Geom &G, bool share, const double
         cudaGetLastError();
         return e;
     }
+    LagrangeRows lag;
+    lagrange_rows(G.b, lag.w);
+    double *Lv = nullptr;
+    size_t most = 0;
     for (int u = 0; u < 8; ++u)
-        if (t->g.tiles[u])
-            k_limb_table<<<t->g.tiles[u] * kLimbM, 256, (size_t)t->g.kst[u] * 16 * sizeof(double)>>>(t->g, u, dgf, dgf_L,
-                                                                                                 t->A, t->rf);
+        if (t->g.tiles[u]) most = std::max(most, (size_t)limb_lat_rows(t->g, u) * t->g.K[u]);
+    e = cudaMalloc((void **)&Lv, most * sizeof(double));
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return e;
+    }
+    for (int u = 0; u < 8; ++u) {
+        if (!t->g.tiles[u]) continue;
+        k_limb_lattice<<<limb_lat_rows(t->g, u), 256>>>(t->g, u, dgf, dgf_L, Lv);
+        k_limb_table<<<t->g.tiles[u] * kLimbM, 256, (size_t)t->g.kst[u] * 16 * sizeof(double)>>>(t->g, u, dgf, dgf_L, Lv, lag,
+                                                                                             t->A, t->rf);
+    }
     e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
+    cudaFree(Lv);
     if (e != cudaSuccess) return e;
     g_tabs[key] = t;
     *out = t;

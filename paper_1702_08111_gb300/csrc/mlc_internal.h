@@ -124,7 +124,7 @@ inline size_t conv_scratch_bytes(const Geom &g, long items) {
 // of every problem in the batch.
 struct PlanPtrs {
     const void *f;        // charge, N^3 (FP64 or FP32 by tier)
-    void *cl, *fp;        // local fields on the coarse lattice / alpha face planes
+    void *cl, *fp;        // local fields on the coarse lattice / (split tiers) alpha face planes
     const void *khat;     // split tiers: patch kernel spectrum octant (FP32)
     const void *momw;     // 1D moment weights a_k(m) = w_m q_k(2m/n - 1), P x (n+1), FP64
     double mom_scale;     // R^{-3/2}
@@ -214,7 +214,7 @@ struct mlc_plan_s {
     void *user_scratch = nullptr;  // caller-owned scratch (mlc_plan_set_scratch), if any
     int fault = 0;                 // test hook (mlc_debug_set_fault)
     void *cl;                // NP x nc^3 local fields on the coarse lattice of the field box (FP32 / double-float)
-    void *fpl;               // NP x 3 npa x wa^2 local fields on the face planes inside alpha (FP32 / double-float)
+    void *fpl;               // split tiers: NP x 3 npa x wa^2 local fields on the face planes inside alpha (FP32)
     double *mom;             // NP x npad
     float *mom_f;            // split tiers: FP32 copy of the moments
     float2 *mom_df;          // double-float tier: double-float copy of the moments

@@ -820,7 +820,7 @@ mlc_status create_plan(const mlc_params *params, const double *dgf_host, int dgf
         // that needs it, unless the caller provides one (mlc_plan_set_scratch)
         char *bc = nullptr, *bf = nullptr;
         TRY(dev_alloc(pl, &bc, NP * (size_t)G.nc * G.nc * G.nc * rb));
-        TRY(dev_alloc(pl, &bf, NP * 3 * (size_t)G.npa * G.wa * G.wa * rb));
+        if (G.conv == CONV_F32) TRY(dev_alloc(pl, &bf, NP * 3 * (size_t)G.npa * G.wa * G.wa * rb));
         pl->cl = bc;
         pl->fpl = bf;
         if (G.conv == CONV_F32) {
