@@ -139,51 +139,62 @@ __global__ void __launch_bounds__(256) k_limb_table(LimbConvGeom g, int u, const
 
 // ---------------------------------------------------------------------------
 // Folded charges.  One CTA per patch: the chi-weighted closed-patch charge is
-// folded along axis 0 while it is read (one parity at a time, so that the array
-// of (n/2 + 1) (n + 1)^2 values fits shared memory for every patch size) and
-// along axes 1 and 2 in place; each class is then scaled by its own largest
-// magnitude and written as digits, columns in the operand layout.  The bytes
-// written (14 per charge) bound it at large n; at n = 16 the FP64 pipe does:
-// three sums per value.
+// folded along axis 0 while it is read and along axes 1 and 2 in place, the odd
+// part of a pair at the place of its mirror image; each class is then scaled by
+// its own largest magnitude and written as digits, columns in the operand layout.
+// Both parities of axis 0 at once up to n = 16 (39 KB of shared memory), one after
+// the other above.  Three FP64 sums per value and 14 bytes written per charge; the
+// patch size is a constant, so that the index divisions are multiplications: 4096
+// patches of 16^3 0.50 -> 0.35 ms against one kernel for all sizes that read
+// the charges once per parity.
 // ---------------------------------------------------------------------------
 struct FoldArgs {
     Items it;
     unsigned char *B;
     double *cf;       // [class][cols_pad]
-    int n, ctiles;
+    int ctiles;
     LimbConvGeom g;
 };
+constexpr bool fold_both(int n) { return n <= 16; }
+constexpr size_t fold_smem(int n) {
+    return (size_t)(fold_both(n) ? n + 1 : n / 2 + 1) * (n + 1) * (n + 1) * sizeof(double);
+}
 
+template <int NN>
 __global__ void __launch_bounds__(256) k_limb_fold(const __grid_constant__ FoldArgs a) {
-    extern __shared__ double S[];  // [m0][m1][m2], m0 <= n/2; odd parts at the mirrored index
-    __shared__ int smax[4];
+    constexpr int n = NN, nb = n + 1, h = n / 2;
+    constexpr bool BOTH = fold_both(NN);
+    extern __shared__ double S[];  // [m0][m1][m2]; odd parts at the mirrored index
+    __shared__ int smax[8];
     int p;
     const PlanPtrs &PP = item_plan(a.it, blockIdx.x, p);
-    const int n = a.n, nb = n + 1, h = n / 2, N = PP.N, np = PP.np;
+    const int N = PP.N, np = PP.np;
     const int i2 = p % np, i1 = (p / np) % np, i0 = p / (np * np);
     const double *f = (const double *)PP.f;
     const int col = blockIdx.x, ct = col / kLimbN, cl = col % kLimbN;
     auto charge = [&](int m0, int m1, int m2) -> double {
         const int z = i0 * n + m0, y = i1 * n + m1, x = i2 * n + m2;
         if (z >= N || y >= N || x >= N) return 0.0;
+        const double v = f[((long)z * N + y) * N + x];
         const int faces = (m0 == 0 || m0 == n) + (m1 == 0 || m1 == n) + (m2 == 0 || m2 == n);
-        const double w = faces == 0 ? 1.0 : (faces == 1 ? 0.5 : (faces == 2 ? 0.25 : 0.125));
-        return w * f[((long)z * N + y) * N + x];
+        return faces == 0 ? v : v * (faces == 1 ? 0.5 : (faces == 2 ? 0.25 : 0.125));
     };
-    for (int p0 = 0; p0 < 2; ++p0) {
-        const int d0 = a.g.hin[p0];
-        for (int e = threadIdx.x; e < d0 * nb * nb; e += blockDim.x) {
+    for (int half = 0; half < (BOTH ? 1 : 2); ++half) {
+        const int planes = BOTH ? nb : (half ? h : h + 1);  // of this round
+        for (int e = threadIdx.x; e < (BOTH || !half ? h + 1 : h) * nb * nb; e += blockDim.x) {
             const int m2 = e % nb, m1 = (e / nb) % nb, m0 = e / (nb * nb);
-            double v = charge(m0, m1, m2);
-            if (m0 != h) {
+            const double v = charge(m0, m1, m2);
+            if (m0 == h) {
+                S[e] = v;
+            } else {
                 const double w = charge(n - m0, m1, m2);
-                v = p0 ? v - w : v + w;
+                S[e] = !BOTH && half ? v - w : v + w;
+                if (BOTH) S[((n - m0) * nb + m1) * nb + m2] = v - w;
             }
-            S[e] = v;
         }
-        if (threadIdx.x < 4) smax[threadIdx.x] = 0;
+        if (threadIdx.x < 8) smax[threadIdx.x] = 0;
         __syncthreads();
-        for (int e = threadIdx.x; e < d0 * h * nb; e += blockDim.x) {  // axis 1
+        for (int e = threadIdx.x; e < planes * h * nb; e += blockDim.x) {  // axis 1
             const int m2 = e % nb, m1 = (e / nb) % h, m0 = e / (nb * h);
             double *u = S + (m0 * nb + m1) * nb + m2, *w = S + (m0 * nb + n - m1) * nb + m2;
             const double x = *u, y = *w;
@@ -191,34 +202,36 @@ __global__ void __launch_bounds__(256) k_limb_fold(const __grid_constant__ FoldA
             *w = x - y;
         }
         __syncthreads();
-        // axis 2, and the largest exponent of each class (p1, p2)
-        int mx[4] = {0, 0, 0, 0};
-        for (int e = threadIdx.x; e < d0 * nb * (h + 1); e += blockDim.x) {
-            const int m2 = e % (h + 1), r = e / (h + 1), m1 = r % nb;
+        // axis 2, and the largest exponent of each class
+        int mx[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+        for (int e = threadIdx.x; e < planes * nb * (h + 1); e += blockDim.x) {
+            const int m2 = e % (h + 1), r = e / (h + 1), m1 = r % nb, m0 = r / nb;
+            const int c = (BOTH && m0 > h ? 4 : 0) + (m1 > h ? 2 : 0);
             double *u = S + r * nb + m2;
-            const int c = m1 > h ? 2 : 0;
+            double s = *u, t = 0.0;
             if (m2 < h) {
                 double *w = S + r * nb + n - m2;
-                const double x = *u, y = *w;
-                const double s = x + y, d = x - y;
+                const double y = *w;
+                t = s - y;
+                s = s + y;
                 *u = s;
-                *w = d;
-                if (c) { mx[2] = max(mx[2], biased_exp(s)); mx[3] = max(mx[3], biased_exp(d)); }
-                else { mx[0] = max(mx[0], biased_exp(s)); mx[1] = max(mx[1], biased_exp(d)); }
-            } else {
-                const int ex = biased_exp(*u);
-                if (c) mx[2] = max(mx[2], ex);
-                else mx[0] = max(mx[0], ex);
+                *w = t;
             }
+#pragma unroll
+            for (int q = 0; q < 8; q += 2)
+                if (c == q) {
+                    mx[q] = max(mx[q], biased_exp(s));
+                    mx[q + 1] = max(mx[q + 1], biased_exp(t));
+                }
         }
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
+        for (int q = 0; q < 8; ++q) {
             const int v = __reduce_max_sync(0xffffffffu, mx[q]);
             if ((threadIdx.x & 31) == 0 && v) atomicMax(&smax[q], v);
         }
         __syncthreads();
-        for (int q = 0; q < 4; ++q) {
-            const int c = 4 * p0 + q, u = limb_table(a.g.share, c), e = smax[q];
+        for (int q = 0; q < (BOTH ? 8 : 4); ++q) {
+            const int c = 4 * half + q, u = limb_table(a.g.share, c), e = smax[q];
             const bool live = e != 0 && e != 0x7ff;
             // infinities and NaN make the patch's whole local field NaN, as the transforms of one do
             if (threadIdx.x == 0)
@@ -226,12 +239,14 @@ __global__ void __launch_bounds__(256) k_limb_fold(const __grid_constant__ FoldA
                     e == 0x7ff ? __longlong_as_double(0x7ff8000000000000ll) : (live ? ldexp(PP.h2, e - 1022) : 0.0);
             unsigned char *Bt = a.B + a.g.b_step[c] * a.ctiles + (long)ct * a.g.kst[u] * kLimbBStep;
             const int K = a.g.K[u];
-            const int q0 = limb_perm(a.g.share, c, 0), q1 = limb_perm(a.g.share, c, 1), q2 = limb_perm(a.g.share, c, 2);
-            // step of S along each table axis and its start: odd reps run down from the mirrored end
-            const int st[3] = {nb * nb, nb, 1};
-            const int o1 = (q & 2) ? n * nb : 0, o2 = (q & 1) ? n : 0, base = o1 + o2;
-            auto step = [&](int ax) { return ax == 0 ? st[0] : (ax == 1 ? ((q & 2) ? -nb : nb) : ((q & 1) ? -1 : 1)); };
-            const int s0 = step(q0), s1 = step(q1), s2 = step(q2);
+            // step of S along each axis of the class and its start: odd reps run down from the mirrored end
+            const bool o0 = BOTH && limb_odd(c, 0), o1 = limb_odd(c, 1), o2 = limb_odd(c, 2);
+            const int base = (o0 ? n * nb * nb : 0) + (o1 ? n * nb : 0) + (o2 ? n : 0);
+            auto step = [&](int i) {  // along axis i of the class's table
+                const int ax = limb_perm(a.g.share, c, i);
+                return ax == 0 ? (o0 ? -nb * nb : nb * nb) : (ax == 1 ? (o1 ? -nb : nb) : (o2 ? -1 : 1));
+            };
+            const int s0 = step(0), s1 = step(1), s2 = step(2);
             const int d1 = a.g.hin[limb_odd(u, 1)], d2 = a.g.hin[limb_odd(u, 2)];
             for (int w = threadIdx.x; w < a.g.kst[u] * 2; w += blockDim.x) {
                 unsigned long long Y[8];
@@ -249,9 +264,10 @@ __global__ void __launch_bounds__(256) k_limb_fold(const __grid_constant__ FoldA
                 for (int i = 0; i < kLimbs; ++i) *(uint4 *)(o + i * kLimbBBlk) = digit_chunk(Y, i);
             }
         }
-        __syncthreads();
+        if (!BOTH) __syncthreads();
     }
 }
+#define MLC_FOLD_N(X) X(4) X(8) X(12) X(16) X(24) X(32)
 
 // ---------------------------------------------------------------------------
 // Unfold: one CTA per patch.  Each representative output point reads its value
@@ -457,8 +473,9 @@ cudaError_t limb_conv_tables(int device, const Geom &G, bool share, const double
 }
 
 void configure_limb_conv() {
-    const int big = 160 * 1024;
-    cudaFuncSetAttribute(k_limb_fold, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
+#define MLC_X(NN) cudaFuncSetAttribute(k_limb_fold<NN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fold_smem(NN));
+    MLC_FOLD_N(MLC_X)
+#undef MLC_X
 }
 
 // Local convolutions of one launch group: three launches.
@@ -471,8 +488,13 @@ static cudaError_t limb_conv_group(const mlc_plan_s *pl, const Items &it, cudaSt
     double *cf = (double *)(B + ct * g.b_total);
     double *V = cf + 8 * ct * kLimbN;
     mark(pl, 1, st);
-    FoldArgs fa{it, B, cf, g.n, (int)ct, g};
-    k_limb_fold<<<(unsigned)items, 256, (size_t)(g.n / 2 + 1) * (g.n + 1) * (g.n + 1) * sizeof(double), st>>>(fa);
+    FoldArgs fa{it, B, cf, (int)ct, g};
+    switch (g.n) {
+#define MLC_X(NN) case NN: k_limb_fold<NN><<<(unsigned)items, 256, fold_smem(NN), st>>>(fa); break;
+        MLC_FOLD_N(MLC_X)
+#undef MLC_X
+        default: return cudaErrorInvalidValue;
+    }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     mark(pl, 2, st);
