@@ -285,7 +285,7 @@ def dirichlet_counts(n, Q):
 
 
 Q10_ORBITS = ((0, 0, 0), (1, 0, 0), (1, 1, 0), (1, 1, 1), (2, 0, 0), (2, 1, 0))
-WIDE_DIRICHLET_ITERS = 10  # fixed-point steps after the first solve (the library's count)
+WIDE_DIRICHLET_ITERS = 10  # fixed-point steps after the first solve
 
 
 def dirichlet_wide_counts(n, iters=WIDE_DIRICHLET_ITERS):
@@ -326,9 +326,45 @@ def dirichlet_wide_counts(n, iters=WIDE_DIRICHLET_ITERS):
     return flops, inst
 
 
+def dirichlet_tri_counts(n, Q):
+    """Counts of the Dirichlet step as the library runs it: dirichlet_counts with
+    the two transforms along one axis and the eigenvalue scaling replaced by the
+    tridiagonal eliminations (two products and two FMAs per value)."""
+    flops, inst = dirichlet_counts(n, Q)
+    m = n - 1
+    line_inst = 97 if n == 16 else 30 + 97 + 8 * (15 + 4)
+    line_flops = 97 if n == 16 else 30 + 97 + 8 * (2 * 15 + 4)
+    return (flops - 2 * m * m * line_flops - m ** 3 + 6 * m ** 3, inst - 2 * m * m * line_inst - m ** 3 + 4 * m ** 3)
+
+
+LIMB_PAIRS = 28  # digit products of an exact-split product (digits i + j < 7)
+
+
+def limb_conv_macs(n, s, ga):
+    """Multiply-adds per patch of the folded local products of the FP64 and
+    double-float tiers: per parity class, outputs (coarse lattice of the field
+    box, face planes of the inner box) x inputs."""
+    def axis(lo_reps, odd):  # reps of a symmetric coordinate list with or without its centre
+        return lo_reps - (1 if odd else 0)
+    lat = (n // 2 + s) // 4 + 1
+    lat_centre = (n // 2 + s) % 4 == 0
+    planes = sum(1 for j in range(-(ga // n), ga // n + 2) if 2 * j * n < n)
+    total = 0
+    for c in range(8):
+        odd = [(c >> (2 - d)) & 1 for d in range(3)]
+        K = np.prod([axis(n // 2 + 1, o) for o in odd])
+        rows = np.prod([lat - (1 if o and lat_centre else 0) for o in odd])
+        hp = [axis(n // 2 + ga + 1, o) for o in odd]
+        rows += planes * (hp[1] * hp[2] + hp[0] * hp[2] + hp[0] * hp[1])
+        total += int(rows) * int(K)
+    return total
+
+
 def roofline_for(w, plan, per_launch, tier, traffic=None):
-    """Roofline of the dominant launch.  Slab kernel (local convolutions):
-    algorithmic work = nominal radix-2 FFT FLOPs (5 M log2 M per complex line)
+    """Roofline of the dominant launch.  FP64 and double-float local products:
+    algorithmic work = 2 FLOPs per multiply-add of the folded operator and digit
+    pair, peak = the measured FP16 / BF16 GEMM rate.  Slab kernel (local
+    convolutions of the split tiers): algorithmic work = nominal radix-2 FFT FLOPs (5 M log2 M per complex line)
     over the lines the pruned transform must produce (forward y on the n+1
     nonzero z rows, forward and inverse z on all M columns, inverse y on the z
     rows read later) plus 2 FLOPs per entry of the real-kernel product, per
@@ -341,63 +377,60 @@ def roofline_for(w, plan, per_launch, tier, traffic=None):
     M, Mh, NP = info.M, info.M // 2 + 1, (N // w.n) ** 3
     dom = max(per_launch, key=per_launch.get)
     fine64 = tier in ("fp64", "split")
+    if dom == "conv_slab" and tier in ("fp64", "df"):
+        flops = 2.0 * LIMB_PAIRS * limb_conv_macs(w.n, w.s, info.g_alpha)
+        peak = float(peaks().get("bf16_tflops") or 1893.8)
+        launch_ms = per_launch[dom]
+        achieved = NP * flops / (launch_ms * 1e-3) / 1e12
+        return {"bound": "tensor", "kernel": dom, "achieved": round(achieved, 4), "peak": round(peak, 4),
+                "unit": "TFLOP/s", "frac": round(achieved / peak, 4), "traffic": traffic,
+                "launch_ms": round(launch_ms, 4), "launches_per_step": 1, "flops_per_launch": NP * flops,
+                "units_per_launch": NP, "unit_of_work": "patch", "flops_per_unit": flops,
+                "peak_basis": "FP16 digit products (28 per FP64 product) against the measured dense GEMM rate"}
     if dom == "conv_slab" and M == 64:
         nin = w.n + 1
         nz = slab_rows(w, info.g_alpha)
         line_flops = 5.0 * M * np.log2(M)
         nominal = (nin + 2 * M + nz) * line_flops + 2.0 * M * M
-        prod = {"df": 2 * DF_MUL_INST, "fp64": 2, "split": 2, "split_df": 2}[tier]
-        inst = ((nin + M) * fft64_schedule_inst(tier if tier in ("fp64", "df") else "split", True, nin)
-                + (M + nz) * fft64_schedule_inst(tier if tier in ("fp64", "df") else "split", False)
-                + M * M * prod)
+        inst = ((nin + M) * fft64_schedule_inst("split", True, nin) + (M + nz) * fft64_schedule_inst("split", False)
+                + M * M * 2)
         # one launch per group of CONV_CHUNK patches (the library's default group size)
         nlaunch = -(-NP // CONV_CHUNK)
-        units, pipe_rate = min(NP, CONV_CHUNK) * Mh, (FP64_INST_PER_S if tier == "fp64" else FP32_LANE_INST_PER_S)
-        pipe = "FP64 pipe" if tier == "fp64" else "FP32 pipe"
-        sched = {"fp64": "FP64 radix-8x8", "df": "double-float radix-8x8"}.get(tier, "FP32 radix-2 register")
+        units, pipe_rate = min(NP, CONV_CHUNK) * Mh, FP32_LANE_INST_PER_S
+        pipe = "FP32 pipe"
+        sched = "FP32 radix-2 register"
         unit_name = "(patch, kx) slab"
     elif dom == "conv_slab" and M == 128:
-        # the 128-point slabs (n = 24, 32).  Split tiers (k_slab128r): radix
-        # 16 x 8 over 8-lane groups, per lane and line a 16-point DFT (196
-        # FP32 instructions; 164 when the inputs 8..15 are zero, the forward
-        # passes), 15 twiddle products (60) and two 8-point DFTs (112); the
-        # kernel product is 2 instructions per entry.  FP64 / double-float
-        # (k_slab_rows): shared-memory radix-2 stages, 8 operations per
-        # butterfly (4 adds, 2 multiplies + 2 FMAs for the twiddle), no
-        # pruning, inverse y on the nz columns read later.
+        # the 128-point slabs (k_slab128r): radix 16 x 8 over 8-lane groups, per
+        # lane and line a 16-point DFT (196 FP32 instructions; 164 when the
+        # inputs 8..15 are zero, the forward passes), 15 twiddle products (60)
+        # and two 8-point DFTs (112); the kernel product is 2 instructions per entry
         nin = w.n + 1
         nz = slab_rows(w, info.g_alpha)
         line_flops = 5.0 * M * np.log2(M)
         nominal = (nin + 2 * M + nz) * line_flops + 2.0 * M * M
-        if tier in ("split", "split_df"):
-            sparse_line, full_line = 8 * (164 + 60 + 112), 8 * (196 + 60 + 112)
-            inst = (nin + M) * sparse_line + (M + nz) * full_line + 2.0 * M * M
-            sched = "FP32 radix-16x8 register"
-        else:
-            bfly = (M // 2) * np.log2(M)
-            per_op = 1 if tier == "fp64" else (4 * DF_ADD_INST + 4 * DF_MUL_INST) / 8.0
-            inst = (nin + 2 * M + nz) * bfly * 8 * per_op + 2.0 * M * M * (DF_MUL_INST if tier == "df" else 1)
-            sched = {"fp64": "FP64 shared-memory radix-2 (row-streamed)",
-                     "df": "double-float shared-memory radix-2 (row-streamed)"}[tier]
+        sparse_line, full_line = 8 * (164 + 60 + 112), 8 * (196 + 60 + 112)
+        inst = (nin + M) * sparse_line + (M + nz) * full_line + 2.0 * M * M
+        sched = "FP32 radix-16x8 register"
         nlaunch = -(-NP // CONV_CHUNK)
-        units, pipe_rate = min(NP, CONV_CHUNK) * Mh, (FP64_INST_PER_S if tier == "fp64" else FP32_LANE_INST_PER_S)
-        pipe = "FP64 pipe" if tier == "fp64" else "FP32 pipe"
+        units, pipe_rate = min(NP, CONV_CHUNK) * Mh, FP32_LANE_INST_PER_S
+        pipe = "FP32 pipe"
         unit_name = "(patch, kx) slab"
     elif dom == "dirichlet" and getattr(w, "Q", 0) == 10:
-        nominal, inst = dirichlet_wide_counts(w.n)
+        nominal, inst = dirichlet_wide_counts(w.n, iters=1)  # two solves around the layer operator
         nlaunch = 1
         units, pipe_rate = NP, FP64_INST_PER_S
         pipe = "FP64 pipe"
-        sched = "FP64 two-layer fixed point on DST-I"
+        sched = "FP64 DST-I (two solves)"
         unit_name = "patch"
     elif dom == "dirichlet" and w.n in (16, 32):
-        nominal, inst = dirichlet_counts(w.n, w.Q)
+        nominal, inst = dirichlet_tri_counts(w.n, w.Q)
         if not fine64:
             inst = inst * DF_ADD_INST  # double-float: about 8 FP32 instructions per operation
         nlaunch = 1
         units, pipe_rate = NP, (FP64_INST_PER_S if fine64 else FP32_LANE_INST_PER_S)
         pipe = "FP64 pipe" if fine64 else "FP32 pipe"
-        sched = "FP64 split DST-I" if fine64 else "double-float split DST-I"
+        sched = ("FP64" if fine64 else "double-float") + " split DST-I and elimination"
         unit_name = "patch"
     else:
         return None
@@ -464,7 +497,8 @@ def run_ours(args, rank, world):
     # kernel launches of one solve: moments, 3 per local-convolution launch
     # group of 1024 patches, residuals, F^H, 5 coarse, boundary, Dirichlet
     NP = (N // w.n) ** 3
-    launches = 10 + 3 * ((NP + 1023) // 1024) + (3 if w.Q == 10 else 0)  # Q = 10: the second layer's 3
+    # (Q = 10: the second layer's 3, and 2 more of its Dirichlet step)
+    launches = 10 + 3 * ((NP + 1023) // 1024) + (5 if w.Q == 10 else 0)
     res = {"value": value, "ms": ms, "e2e_ms": e2e_ms, "per_launch": per_launch, "launches_per_step": launches,
            "roofline": roofline_for(w, plan, per_launch, tier, traffic_for(args.workload, tier, per_launch)),
            "clocks": clk.summary(), "phi": phi, "N": N, "tier": tier, "f_bytes": f_host.element_size() * N ** 3}
