@@ -340,15 +340,19 @@ def dirichlet_tri_counts(n, Q):
 LIMB_PAIRS = 28  # digit products of an exact-split product (digits i + j < 7)
 
 
-def limb_conv_macs(n, s, ga):
+def limb_conv_macs(n, s, ga, wide=False):
     """Multiply-adds per patch of the folded local products of the FP64 and
     double-float tiers: per parity class, outputs (coarse lattice of the field
-    box, face planes of the inner box) x inputs."""
+    box, face planes of the inner box; Q = 10, `wide`: and the planes one node off
+    them) x inputs."""
     def axis(lo_reps, odd):  # reps of a symmetric coordinate list with or without its centre
         return lo_reps - (1 if odd else 0)
     lat = (n // 2 + s) // 4 + 1
     lat_centre = (n // 2 + s) % 4 == 0
     planes = sum(1 for j in range(-(ga // n), ga // n + 2) if 2 * j * n < n)
+    if wide:
+        planes += sum(1 for j in range(-(ga // n), ga // n + 2) for y in (j * n - 1, j * n + 1)
+                      if -ga <= y <= n + ga and 2 * y < n)
     total = 0
     for c in range(8):
         odd = [(c >> (2 - d)) & 1 for d in range(3)]
@@ -378,7 +382,7 @@ def roofline_for(w, plan, per_launch, tier, traffic=None):
     dom = max(per_launch, key=per_launch.get)
     fine64 = tier in ("fp64", "split")
     if dom == "conv_slab" and tier in ("fp64", "df"):
-        flops = 2.0 * LIMB_PAIRS * limb_conv_macs(w.n, w.s, info.g_alpha)
+        flops = 2.0 * LIMB_PAIRS * limb_conv_macs(w.n, w.s, info.g_alpha, getattr(w, "Q", 0) == 10)
         peak = float(peaks().get("bf16_tflops") or 1893.8)
         launch_ms = per_launch[dom]
         achieved = NP * flops / (launch_ms * 1e-3) / 1e12

@@ -125,7 +125,9 @@ mlc_status mlc_params_init(mlc_params *p, int N, int n, int s, int P, int Q);
  * Create a plan on the current CUDA device (Sec. 4 with the regions
  * Omega_alpha = G(Omega_i, s - C b), Omega_beta = G(Omega_i, g_beta)).  Builds
  * the DGF table (App. A.1) if this device has none for (Q, nD, zeta), the
- * kernel spectra for the Hockney convolutions (App. A.2), the Legendre
+ * tables of the local convolutions (kernel spectra, App. A.2, or folded Green's
+ * functions, shared by the plans of one patch geometry: 30 MB at n = s = 16,
+ * 1.2 GB at n = 32) and the coarse one's spectrum, the Legendre
  * basis-field tables Delta^H(G^h * Q^p) (Sec. 4, Step 1) and the index tables,
  * and allocates the workspace.  Synchronises the device.
  * INVALID_ARG if: out is NULL; N, n, s, C, P, Q, levels break the rules
@@ -288,13 +290,14 @@ mlc_status mlc_debug_stage_bytes(mlc_plan_t plan, int stage, size_t *bytes);
  * a CUDA event before each launch and after the last.  mlc_debug_timing waits for the last solve's final event and
  * writes the 13 durations (ms) in launch order: moments; local convolutions:
  * forward x, fused slab (forward y and z, kernel spectrum, inverse z and y),
- * inverse x; residuals; assembly of F^H; coarse convolution x, y, z (forward,
+ * inverse x (FP64 and double-float tiers: folding, products, unfolding);
+ * residuals (nothing there); assembly of F^H; coarse convolution x, y, z (forward,
  * kernel, inverse), inverse y, inverse x; boundary values; Dirichlet solves.
  * count must be >= 13. */
 mlc_status mlc_debug_set_timing(mlc_plan_t plan, int enable);
 /* Test hook for the failure path of the bounded waits (no counterpart in the
- * paper): kind 1 makes later solves with this plan skip the bulk copy that the
- * local-convolution inverse-x kernel waits for, with the wait limited to 64
+ * paper): kind 1 makes later solves with this plan skip the bulk copies that the
+ * local convolutions' inverse-x kernel (split tiers) or products wait for, with the wait limited to 64
  * tests, so every such wait runs out, the kernel records the failure and
  * returns, and mlc_plan_status reports TIMEOUT (the potential is then not
  * valid).  kind 0 restores normal solves.  INVALID_ARG for other kinds. */

@@ -438,6 +438,7 @@ cudaError_t limb_conv_tables(int device, const Geom &G, bool share, const double
         *out = have;
         return cudaSuccess;
     }
+    for (auto i = g_tabs.begin(); i != g_tabs.end();) i = i->second.expired() ? g_tabs.erase(i) : std::next(i);
     auto t = std::make_shared<LimbConvTables>();
     if (!limb_conv_geometry(G, share, t->g)) return cudaErrorInvalidValue;
     cudaError_t e = cudaMalloc((void **)&t->A, (size_t)t->g.a_bytes);

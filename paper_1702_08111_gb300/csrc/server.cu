@@ -75,8 +75,8 @@ struct Pending {
 };
 
 // Upper bound of the device bytes a plan with these parameters holds (its
-// per-patch arrays and tables; the shared DGF table and the lanes' scratch
-// are not counted).
+// per-patch arrays and tables; what plans share, the DGF table and the
+// exact-split tables of a patch geometry, and the lanes' scratch are not counted).
 size_t estimate_bytes(const mlc_params &p) {
     const long N = p.N, n = p.n, s = p.s;
     if (n <= 0 || N <= 0 || N % n) return 0;
