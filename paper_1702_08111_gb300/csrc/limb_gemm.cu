@@ -10,13 +10,14 @@
 // digit pairs i + j < 7; after every 16 steps eight warps read the levels,
 // combine them into two 64-bit integers per output (exact) and hand the
 // accumulators back.  The FP64 conversion of a finished tile therefore runs
-// beside the next tile's MMAs.  It is kept to four operations per output, since
-// GB300 issues FP64 on two lanes per SM and cycle.
+// beside the next tile's MMAs, with one FP64 operation per output.
 //
-// Bound: the MMAs' operand reads.  M = 128, N = 64 reads 6 KB of shared memory per
-// 128 x 64 x 16 products, and a k-step takes 2690 cycles, 96 per MMA (64 B per
-// cycle) against 32 at the dense FP16 rate; a wider N does not fit seven
-// accumulators.  256^3, n = s = 16, Q = 6: 1.20 ms for 0.84 PFLOP of digit products.
+// Bound: the MMAs and the reads of the accumulators between them.  A k-step takes
+// 2690 cycles on average, 96 per MMA, of which the MMA itself takes 61 (measured by
+// leaving 15 of the 28 out) against 32 at the dense FP16 rate: M = 128, N = 64 reads
+// 6 KB of shared memory per 128 x 64 x 16 products, and a wider N does not fit seven
+// accumulators.  The copies are hidden (a third of their bytes takes the same time).
+// 256^3, n = s = 16, Q = 6: 1.20 ms for 0.84 PFLOP of digit products.
 #include "limb.h"
 #include "mlc_internal.h"
 
@@ -86,6 +87,31 @@ __device__ __forceinline__ void tmem_ld16(uint32_t t, uint32_t (&r)[16]) {
           "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
         : "r"(t));
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+
+// (hi 2^32 + lo) 2^k as FP64, rounded to nearest even, by integer operations, the
+// same value as fma(hi, 2^32, lo) 2^k without its five FP64 operations (two lanes
+// per SM): they show where a CTA has one tile (32^3, n = 8: the whole solve 199 ->
+// 192 us) and hide behind the next tile's MMAs elsewhere.  |hi| < 2^62; the result
+// is a normal number or 0.
+__device__ __forceinline__ double limb_sum_to_double(long long hi, long long lo, int k) {
+    long long H = hi + (lo >> 32);
+    unsigned L = (unsigned)lo;
+    const bool neg = H < 0;
+    if (neg) {
+        L = 0u - L;
+        H = ~H + (L == 0u ? 1 : 0);
+    }
+    if (H == 0 && L == 0u) return 0.0;
+    const unsigned long long low = (unsigned long long)L << 32;
+    const int s = H ? __clzll(H) : 64 + __clz((int)L);  // leading zeros of H : low, s >= 1
+    const unsigned long long M = s < 64 ? ((unsigned long long)H << s) | (low >> (64 - s)) : low << (s - 64);
+    const unsigned long long rest = s < 64 ? low << s : 0ull;
+    const unsigned rem = (unsigned)M & 0x7ffu;
+    unsigned long long m = M >> 11;  // 53 bits, leading one at bit 52
+    if (rem > 0x400u || (rem == 0x400u && (rest != 0ull || (m & 1ull)))) ++m;
+    const unsigned long long b = ((unsigned long long)(1023 + 95 - s + k - 1) << 52) + m;
+    return __longlong_as_double((long long)(b | (neg ? 1ull << 63 : 0ull)));
 }
 
 __device__ __forceinline__ const LimbPart &part_of(const LimbJob &job, int t) {
@@ -243,14 +269,14 @@ __global__ void __launch_bounds__(kThreads, 1) k_limb_gemm(const __grid_constant
             }
             if (!ok) break;
             const int row = rt * kLimbM + sub * 32 + lane, c0 = ct * kLimbN + half * 32;
-            const double rf = P.rf[row];
+            const int k = (int)((__double_as_longlong(P.rf[row]) >> 52) & 0x7ff) - 1023;  // rf = 2^k (or 0 with zero digits)
             const double *cf = job.cf + P.cf_off + (long)c0 * job.cf_step;
             double *v = job.V + P.v_off + (long)c0 * P.rows + row;
             if (row < P.rows) {
 #pragma unroll
                 for (int j = 0; j < 32; ++j)
                     if (c0 + j < P.cols)
-                        v[(long)j * P.rows] = fma((double)hi[j], 4294967296.0, (double)lo[j]) * rf * cf[j * job.cf_step];
+                        v[(long)j * P.rows] = limb_sum_to_double(hi[j], lo[j], k) * cf[j * job.cf_step];
             }
         }
         if (!ok) {
